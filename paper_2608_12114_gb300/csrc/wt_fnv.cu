@@ -1,7 +1,7 @@
 // sm_103a kernels of the per-buffer FNV-1a-64 digests that prove ingested bytes equal the
 // file's: the literal serial digest, and the tree digest (FNV-1a-64 of each 4 KiB leaf,
 // then FNV-1a-64 over the buffer's length and its leaf digests).  The second level of the
-// tree runs in parallel chunks for large buffers, with the exact result of the serial chain.
+// tree runs in parallel chunks, with the exact result of the serial chain.
 #include <cstring>
 
 #include "wt_device.cuh"
@@ -61,11 +61,12 @@ struct Fnv {
   __device__ __forceinline__ uint64_t value() const { return ((uint64_t)hi << 32) | lo; }
 };
 
-__device__ __forceinline__ uint32_t find_buf(const FnvBatch &b, uint64_t leaf) {
-  uint32_t lo = 0, hi = b.n - 1;
+// The buffer that holds entry i of a prefix array (uniform over a warp unless it straddles two).
+__device__ __forceinline__ uint32_t find_in(const uint32_t *prefix, uint32_t n, uint32_t i) {
+  uint32_t lo = 0, hi = n - 1;
   while (lo < hi) {
-    uint32_t mid = (lo + hi + 1) >> 1;
-    if (b.leaf_prefix[mid] <= leaf) lo = mid; else hi = mid - 1;
+    const uint32_t mid = (lo + hi + 1) >> 1;
+    if (prefix[mid] <= i) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
@@ -94,13 +95,13 @@ constexpr int kSliceStride = kSlice + 16;
 constexpr int kLanesPerLeaf = kSlice / 16;
 constexpr int kLeavesPerRound = 32 / kLanesPerLeaf;
 
-__device__ __forceinline__ void fnv_stage_fast(uint8_t (*dst)[kSliceStride], const uint8_t *wbase, uint32_t s0,
-                                               int lane) {
+__device__ __forceinline__ void fnv_stage_fast(uint8_t (*dst)[kSliceStride], const uint8_t *wbase, uint32_t pitch,
+                                               uint32_t s0, int lane) {
   const int sub = lane / kLanesPerLeaf, q = lane % kLanesPerLeaf;
-  const uint8_t *src = wbase + (size_t)sub * kLeafBytes + s0 + q * 16;
+  const uint8_t *src = wbase + (size_t)sub * pitch + s0 + q * 16;
 #pragma unroll
   for (int r = 0; r < 32; r += kLeavesPerRound)
-    cp_async16(smem_u32(&dst[r + sub][q * 16]), src + (size_t)r * kLeafBytes);
+    cp_async16(smem_u32(&dst[r + sub][q * 16]), src + (size_t)r * pitch);
   cp_async_commit();
 }
 
@@ -125,273 +126,307 @@ __device__ __forceinline__ void fnv_stage(uint8_t (*dst)[kSliceStride], const ui
   cp_async_commit();
 }
 
-__global__ void __launch_bounds__(kFnvWarps * 32) fnv_leaf_kernel(const __grid_constant__ FnvBatch b,
-                                                                   uint64_t *leaves) {
+// Runs h over this lane's llen bytes at lp, the warp staging slices of its 32 rows together
+// (buf is the warp's own).  fast (warp-uniform): row r starts at wbase + r * pitch, 16-byte
+// aligned, and its bytes up to the longest row's length may be read.
+template <class H>
+__device__ __forceinline__ void run_rows(H &h, uint8_t (*buf)[32][kSliceStride], const uint8_t *lp, uint32_t llen,
+                                         bool fast, const uint8_t *wbase, uint32_t pitch, int lane) {
+  // slices the longest row of the warp needs (warp-uniform)
+  const uint32_t nsl = (__reduce_max_sync(0xffffffffu, llen) + kSlice - 1) / kSlice;
+  if (nsl) {
+    if (fast) fnv_stage_fast(buf[0], wbase, pitch, 0, lane);
+    else fnv_stage(buf[0], lp, llen, 0, lane);
+  }
+  for (uint32_t si = 0; si < nsl; ++si) {
+    if (si + 1 < nsl) {
+      if (fast) fnv_stage_fast(buf[(si + 1) & 1], wbase, pitch, (si + 1) * kSlice, lane);
+      else fnv_stage(buf[(si + 1) & 1], lp, llen, (si + 1) * kSlice, lane);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncwarp();
+    const uint32_t s0 = si * kSlice;
+    if (s0 < llen) {
+      const uint32_t m = min((uint32_t)kSlice, llen - s0);
+      const uint8_t *row = buf[si & 1][lane];
+      uint32_t k = 0;
+      for (; k + 16 <= m; k += 16) h.vec(*reinterpret_cast<const uint4 *>(row + k));
+      for (; k < m; ++k) h.byte(row[k]);
+    }
+    __syncwarp();  // every lane is done with this buffer before it is refilled
+  }
+}
+
+// Device scratch of one batch.
+struct FnvScratch {
+  uint64_t *leaves;  // tree: leaf digests, buffer t's from word chunk_prefix[t] * kChunkLeaves on
+  uint32_t *tab;     // [chunks] transition table of the chunk
+  uint32_t *lstart;  // [chunks] low byte of the state at the chunk's start
+  uint64_t *sum;     // [chunks] the chunk's part of the state (D below)
+};
+
+template <class Tab>
+__global__ void __launch_bounds__(kFnvWarps * 32) fnv_leaf_kernel(const __grid_constant__ Tab b, uint64_t *leaves) {
   __shared__ __align__(16) uint8_t buf[kFnvWarps][2][32][kSliceStride];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint64_t total = b.leaf_prefix[b.n];
+  const uint32_t total = b.leaf_prefix[b.n];
   const uint64_t nwarps = (uint64_t)gridDim.x * kFnvWarps;
   for (uint64_t base = ((uint64_t)blockIdx.x * kFnvWarps + warp) * 32; base < total; base += nwarps * 32) {
     const uint64_t leaf = base + lane;
     const bool mine = leaf < total;
     const uint8_t *lp = nullptr;
     uint32_t llen = 0, t = 0xffffffffu;
+    uint64_t slot = 0;
     if (mine) {
-      t = find_buf(b, leaf);
-      const uint64_t off = (leaf - b.leaf_prefix[t]) * kLeafBytes;
-      lp = b.ptr[t] + off;
-      llen = (uint32_t)min(kLeafBytes, b.nbytes[t] - off);
+      t = find_in(b.leaf_prefix, b.n, (uint32_t)leaf);
+      const uint64_t i = leaf - b.leaf_prefix[t];
+      lp = b.ptr[t] + i * kLeafBytes;
+      llen = (uint32_t)min(kLeafBytes, b.nbytes[t] - i * kLeafBytes);
+      slot = (uint64_t)b.chunk_prefix[t] * kChunkLeaves + i;
     }
     const uint32_t t0 = __shfl_sync(0xffffffffu, t, 0);
     const bool fast = __all_sync(0xffffffffu, mine && t == t0 && llen == kLeafBytes &&
                                                    (reinterpret_cast<uintptr_t>(lp) & 15) == 0);
     const uint8_t *wbase = reinterpret_cast<const uint8_t *>(__shfl_sync(0xffffffffu, (unsigned long long)lp, 0));
-    // slices the longest leaf of the warp needs (warp-uniform)
-    const uint32_t nsl = (__reduce_max_sync(0xffffffffu, llen) + kSlice - 1) / kSlice;
     Fnv h;
-    if (nsl) {
-      if (fast) fnv_stage_fast(buf[warp][0], wbase, 0, lane);
-      else fnv_stage(buf[warp][0], lp, llen, 0, lane);
-    }
-    for (uint32_t si = 0; si < nsl; ++si) {
-      if (si + 1 < nsl) {
-        if (fast) fnv_stage_fast(buf[warp][(si + 1) & 1], wbase, (si + 1) * kSlice, lane);
-        else fnv_stage(buf[warp][(si + 1) & 1], lp, llen, (si + 1) * kSlice, lane);
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
-      }
-      __syncwarp();
-      const uint32_t s0 = si * kSlice;
-      if (mine && s0 < llen) {
-        const uint32_t m = min((uint32_t)kSlice, llen - s0);
-        const uint8_t *row = buf[warp][si & 1][lane];
-        uint32_t k = 0;
-        for (; k + 16 <= m; k += 16) h.vec(*reinterpret_cast<const uint4 *>(row + k));
-        for (; k < m; ++k) h.byte(row[k]);
-      }
-      __syncwarp();  // every lane is done with this buffer before it is refilled
-    }
-    if (mine) leaves[leaf] = h.value();
+    run_rows(h, buf[warp], lp, llen, fast, wbase, (uint32_t)kLeafBytes, lane);
+    if (mine) leaves[slot] = h.value();
   }
 }
 
-// ---- second level: FNV-1a over LE64(nbytes), then the LE64 of each leaf digest
+// ---- a long serial chain in parallel chunks
 //
-// The chain costs one dependent xor and 32 x 32 multiply per byte.  For a buffer of L
-// leaves that is 8 L bytes in one thread (a 1 GB tensor: 2 MB of chain).  Larger buffers
-// split the leaf stream into chunks of kChunkWords digests and combine them exactly in
-// parallel, from three facts about one FNV step (all arithmetic mod 2^32):
-//  1. the low byte of lo evolves on its own: l' = ((l ^ b) p) & 0xff;
-//  2. lo ^ b = lo + d with d = (l ^ b) - l, so lo' = (lo + d) p, and over a chunk of m bytes
-//     lo_end = p^m lo_start + B, where B depends only on the chunk's bytes and the low
-//     byte of lo_start (so the chain run from lo = that low byte alone gives B);
-//  3. hi' = hi p + t with t a function of lo and b alone, so hi_end = p^m hi_start + H,
-//     where H is the chunk's hi run from 0 along the true lo sequence.
-// Passes: (1) l_end for all 256 starting low bytes of every chunk; (2) per buffer, walk the
-// chunks' low bytes through those tables; (3) per chunk, B from its starting low byte;
-// (4) per buffer, lo at every chunk start (lo' = p^m lo + B); (5) per chunk, H from the true
-// lo start; (6) per buffer, fold the H values into hi.  The result equals the serial chain
-// bit for bit.
+// The chain costs one dependent xor and 32 x 32 multiply per byte (10 to 12 cycles), so the
+// second level of a 1 GB tensor, 2 MB of leaf digests, takes 11 ms in one thread.  It is cut
+// into chunks, one thread each, and combined exactly, from two facts about one FNV step
+// h' = (h ^ b) p mod 2^64:
+//  1. the low k bits of h evolve on their own, by a permutation of 2^k states whose top bit is
+//     free: starting from s ^ 2^(k-1) instead of s flips bit k-1 at the end and nothing else
+//     (p is odd).  So 8 starts describe what a chunk does to the low nibble, and, once the low
+//     nibble at its start is known, 8 starts what it does to the high nibble of the low byte;
+//  2. h ^ b = h + d with d = (l ^ b) - l, l the low byte of h, so over a chunk of m bytes
+//     h_end = p^m h_start + D, where D depends only on the chunk's bytes and the low byte l at
+//     its start: running the chain from h = l alone gives D = h_end - p^m l.
+// Passes: (1) every chunk's low-nibble table; (2) per buffer, the chunks' low nibbles through
+// those tables; (3) every chunk's high-nibble table; (4) as (2); (5) every chunk's D; (6) per
+// buffer, h from its start and the D.  The result equals the serial chain bit for bit.
+// Per byte (1) and (3) take 14 operations and (5) one run, where tables of the whole low byte
+// take 320 and separate runs for the low and the high word of h two.  Every buffer of more than
+// one chunk goes this way: 256-byte chunks keep the passes at a few microseconds each.
+// Measured on GB300 (whole calls, leaves included): 2.97 GB with two 1 GB tensors 1332 -> 814
+// us, 1253 tensors of 8 KiB to 8 MiB (1.56 GB) 1261 -> 457 us, against whole-byte tables over
+// 4096-byte chunks for buffers above 16 MiB and one thread per buffer below.
 
-// p^e mod 2^32 by square and multiply
-__device__ __forceinline__ uint32_t fnv_pow(uint32_t e) {
-  uint32_t r = 1, q = kFnvP;
+// p^e mod 2^64 by square and multiply
+__host__ __device__ __forceinline__ uint64_t fnv_pow(uint64_t q, uint32_t e) {
+  uint64_t r = 1;
   for (; e; e >>= 1, q *= q)
     if (e & 1) r *= q;
   return r;
 }
+constexpr uint64_t kFnvPrime = 0x100000001b3ull;
 
-struct FnvScratch {
-  uint64_t *leaves;   // [total leaves]
-  uint8_t *ltab;      // [chunks][256]: low byte at the chunk's end per starting low byte
-  uint32_t *lstart;   // [chunks]: low byte of lo at the chunk's start
-  uint32_t *bpart;    // [chunks]: B
-  uint32_t *lo_start; // [chunks]
-  uint32_t *hpart;    // [chunks]: H
-  uint64_t *head;     // [n]: hi << 32 | lo after LE64(nbytes); lo replaced by the final lo
-};
+// Byte k of v in every byte, or in bytes 0 and 2.
+template <int k>
+__device__ __forceinline__ uint32_t bytes4(uint32_t v) { return __byte_perm(v, 0, 0x1111u * k); }
+template <int k>
+__device__ __forceinline__ uint32_t bytes2(uint32_t v) { return __byte_perm(v, 0, 0x4040u | k | k << 8); }
 
-__device__ __forceinline__ uint32_t find_chunk_buf(const FnvBatch &b, uint32_t c) {
-  uint32_t lo = 0, hi = b.n - 1;
-  while (lo < hi) {
-    uint32_t mid = (lo + hi + 1) >> 1;
-    if (b.chunk_prefix[mid] <= c) lo = mid; else hi = mid - 1;
+// The low nibble from starts 0..7, eight-bit lanes in two registers: (u 3) < 2^8 for u < 16
+// and 3 = p mod 16, so one multiply advances four starts and no lane carries into the next.
+// The mask of one step merges with the xor of the next.
+struct LowNibble {
+  uint32_t r0 = 0x03020100u, r1 = 0x07060504u;
+  __device__ __forceinline__ void step(uint32_t bb) {
+    r0 = ((r0 ^ bb) & 0x0f0f0f0fu) * 3u;
+    r1 = ((r1 ^ bb) & 0x0f0f0f0fu) * 3u;
   }
-  return lo;
-}
-
-// Leaf digests [first, last) of chunk c.
-__device__ __forceinline__ void chunk_range(const FnvBatch &b, uint32_t c, uint64_t &first, uint64_t &last) {
-  const uint32_t t = find_chunk_buf(b, c);
-  first = b.leaf_prefix[t] + (uint64_t)(c - b.chunk_prefix[t]) * kChunkWords;
-  last = min(first + kChunkWords, b.leaf_prefix[t + 1]);
-}
-
-// Pass 1: one block of 64 threads per chunk, four starting low bytes per thread, two per
-// register in 16-bit lanes: (u 0xb3) < 2^16 for u < 256 and 0xb3 = p mod 256, so one
-// multiply advances two starts and the lanes never carry into each other.  The mask of one
-// byte step merges with the xor of the next (one three-input logic op).  The chunk's
-// digests are staged in shared memory and read as broadcasts.
-__global__ void __launch_bounds__(64) fnv_table_kernel(const __grid_constant__ FnvBatch b, FnvScratch sc) {
-  __shared__ uint64_t words[kChunkWords];
-  const uint32_t c = blockIdx.x, tid = threadIdx.x;
-  uint64_t first, last;
-  chunk_range(b, c, first, last);
-  const uint32_t w = (uint32_t)(last - first);
-  for (uint32_t i = tid; i < w; i += blockDim.x) words[i] = sc.leaves[first + i];
-  __syncthreads();
-  constexpr uint32_t kMask = 0x00ff00ffu;
-  uint32_t r0 = tid | (tid + 64) << 16, r1 = (tid + 128) | (tid + 192) << 16;
-  for (uint32_t i = 0; i < w; ++i) {
-    const uint64_t v = words[i];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const uint32_t half = k < 4 ? (uint32_t)v : (uint32_t)(v >> 32);
-      const uint32_t bb = __byte_perm(half, 0, 0x4040u | (k & 3) | (k & 3) << 8);  // b in both lanes
-      r0 = ((r0 & kMask) ^ bb) * 0xb3u;
-      r1 = ((r1 & kMask) ^ bb) * 0xb3u;
-    }
+  __device__ __forceinline__ void byte(uint32_t b) { step(bytes4<0>(b)); }
+  __device__ __forceinline__ void word(uint32_t v) {
+    step(bytes4<0>(v));
+    step(bytes4<1>(v));
+    step(bytes4<2>(v));
+    step(bytes4<3>(v));
   }
-  uint8_t *lt = sc.ltab + (size_t)c * 256;
-  lt[tid] = (uint8_t)r0;
-  lt[tid + 64] = (uint8_t)(r0 >> 16);
-  lt[tid + 128] = (uint8_t)r1;
-  lt[tid + 192] = (uint8_t)(r1 >> 16);
-}
-
-// Serial chain over leaves [l0, l1) from state h; kCombineAhead digests are loaded ahead.
-constexpr int kCombineAhead = 16;
-template <class H>
-__device__ __forceinline__ void fnv_leaf_run(H &h, const uint64_t *leaves, uint64_t l0, uint64_t l1) {
-  uint64_t r[kCombineAhead];
+  __device__ __forceinline__ void vec(const uint4 &v) { word(v.x), word(v.y), word(v.z), word(v.w); }
+  // the low nibble at the end for start j in bits 4j .. 4j + 3
+  __device__ __forceinline__ uint32_t table() const {
+    uint32_t t = 0;
 #pragma unroll
-  for (int j = 0; j < kCombineAhead; ++j) r[j] = l0 + j < l1 ? leaves[l0 + j] : 0;
-  for (uint64_t l = l0; l < l1; l += kCombineAhead) {
-#pragma unroll
-    for (int j = 0; j < kCombineAhead; ++j) {
-      if (l + j < l1) {
-        const uint64_t v = r[j];
-        const uint64_t ln = l + j + kCombineAhead;
-        if (ln < l1) r[j] = leaves[ln];
-        h.le64(v);
-      }
-    }
-  }
-}
-
-// The low word alone (fact 2): what pass 3 needs.
-struct FnvLo {
-  uint32_t lo;
-  __device__ __forceinline__ void le64(uint64_t v) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) lo = (lo ^ (uint32_t)((v >> (8 * k)) & 0xffu)) * kFnvP;
+    for (int j = 0; j < 4; ++j) t |= (r0 >> (8 * j) & 15u) << (4 * j) | (r1 >> (8 * j) & 15u) << (16 + 4 * j);
+    return t;
   }
 };
 
-// One warp per buffer.  Small buffers: lane 0 runs the whole chain.  Chunked buffers: pass 2,
-// the low-byte walk, in lane 0, over table rows the warp copies into a shared-memory ring
-// kWalkAhead chunks ahead (one lookup per chunk instead of one L2 round trip).
-constexpr int kWalkAhead = 8;
+// The low byte from starts nib + 16 j (j = 0..7), sixteen-bit lanes in four registers:
+// (u 0xb3) < 2^16 for u < 256 and 0xb3 = p mod 256.
+struct HighNibble {
+  uint32_t r[4];
+  __device__ __forceinline__ explicit HighNibble(uint32_t nib) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = (nib | 0x100000u) + (nib << 16) + 0x200020u * i;
+  }
+  __device__ __forceinline__ void step(uint32_t bb) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = ((r[i] & 0x00ff00ffu) ^ bb) * 0xb3u;
+  }
+  __device__ __forceinline__ void byte(uint32_t b) { step(bytes2<0>(b)); }
+  __device__ __forceinline__ void word(uint32_t v) {
+    step(bytes2<0>(v));
+    step(bytes2<1>(v));
+    step(bytes2<2>(v));
+    step(bytes2<3>(v));
+  }
+  __device__ __forceinline__ void vec(const uint4 &v) { word(v.x), word(v.y), word(v.z), word(v.w); }
+  __device__ __forceinline__ uint32_t table() const {
+    uint32_t t = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t |= (r[i] >> 4 & 15u) << (8 * i) | (r[i] >> 20 & 15u) << (8 * i + 4);
+    return t;
+  }
+};
 
-__global__ void __launch_bounds__(32) fnv_combine_kernel(const __grid_constant__ FnvBatch b, FnvScratch sc) {
-  __shared__ __align__(16) uint8_t rows[kWalkAhead][256];
-  const uint32_t t = blockIdx.x;
-  const int lane = threadIdx.x;
-  const uint64_t l0 = b.leaf_prefix[t], l1 = b.leaf_prefix[t + 1];
-  const uint32_t c0 = b.chunk_prefix[t], c1 = b.chunk_prefix[t + 1];
+// One entry of a table of 8 starts: start s < 16, the upper 8 from the lower by fact 1.
+__device__ __forceinline__ uint32_t through(uint32_t table, uint32_t s) {
+  return (table >> ((s & 7u) << 2) & 15u) ^ (s & 8u);
+}
+// The table of `a` followed by `b`.
+__device__ __forceinline__ uint32_t then(uint32_t a, uint32_t b) {
+  uint32_t t = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) t |= through(b, a >> (4 * j) & 15u) << (4 * j);
+  return t;
+}
+
+// State at the start of buffer t's serial stream, and the stream's bytes: the tree digest's
+// second level starts after LE64(nbytes) and runs over the leaf digests.
+template <class Tab>
+__device__ __forceinline__ uint64_t stream_head(const Tab &b, uint32_t t) {
   Fnv h;
   h.le64(b.nbytes[t]);
-  if (c0 == c1) {
-    if (lane == 0) {
-      fnv_leaf_run(h, sc.leaves, l0, l1);
-      *b.out[t] = h.value();
+  return h.value();
+}
+template <class Tab>
+__device__ __forceinline__ uint64_t stream_bytes(const Tab &b, uint32_t t) {
+  return 8ull * (b.leaf_prefix[t + 1] - b.leaf_prefix[t]);
+}
+
+// Passes 1, 3 and 5 (PASS 0, 1, 2): one thread per chunk.  Blocks of two warps spread a few
+// thousand chunks over the SMs.  The leaf digests of a batch lie in whole chunks one after
+// another (and up to a whole warp's), so every row may be read to its end.
+constexpr int kChunkWarps = 2;
+template <class Tab, int PASS>
+__global__ void __launch_bounds__(kChunkWarps * 32) fnv_chunk_kernel(const __grid_constant__ Tab b, FnvScratch sc) {
+  __shared__ __align__(16) uint8_t buf[kChunkWarps][2][32][kSliceStride];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t first = (blockIdx.x * kChunkWarps + warp) * 32, c = first + lane;
+  const uint32_t total = b.chunk_prefix[b.n];
+  if (first >= total) return;
+  uint32_t len = 0, nchunk = 0, t = 0;
+  if (c < total) {
+    t = find_in(b.chunk_prefix, b.n, c);
+    nchunk = b.chunk_prefix[t + 1] - b.chunk_prefix[t];
+    len = (uint32_t)min((uint64_t)b.chunk, stream_bytes(b, t) - (uint64_t)(c - b.chunk_prefix[t]) * b.chunk);
+  }
+  // a buffer of one chunk starts from a known state: it needs no table
+  const bool mine = PASS == 2 ? nchunk > 0 : nchunk > 1;
+  if (!mine) len = 0;
+  const uint8_t *wbase = reinterpret_cast<const uint8_t *>(sc.leaves) + (uint64_t)first * b.chunk;
+  const uint8_t *lp = wbase + (uint64_t)lane * b.chunk;
+  if constexpr (PASS == 0) {
+    LowNibble h;
+    run_rows(h, buf[warp], lp, len, true, wbase, b.chunk, lane);
+    if (mine) sc.tab[c] = h.table();
+  } else if constexpr (PASS == 1) {
+    HighNibble h(mine ? sc.lstart[c] : 0);
+    run_rows(h, buf[warp], lp, len, true, wbase, b.chunk, lane);
+    if (mine) sc.tab[c] = h.table();
+  } else {
+    uint32_t l = 0;
+    if (mine) l = nchunk > 1 ? sc.lstart[c] : (uint32_t)stream_head(b, t) & 0xffu;
+    Fnv h;
+    h.lo = l;
+    h.hi = 0;
+    run_rows(h, buf[warp], lp, len, true, wbase, b.chunk, lane);
+    if (mine) sc.sum[c] = h.value() - (len == b.chunk ? b.chunk_pow : fnv_pow(kFnvPrime, len)) * l;
+  }
+}
+
+// Passes 2 and 4 (HIGH): one block per buffer.  Each thread composes the tables of a run of
+// chunks, warp 0 composes and walks the threads' tables, and each thread walks its run.
+constexpr int kWalkThreads = 256;
+template <class Tab, bool HIGH>
+__global__ void __launch_bounds__(kWalkThreads) fnv_walk_kernel(const __grid_constant__ Tab b, FnvScratch sc) {
+  __shared__ uint32_t f[kWalkThreads];
+  __shared__ uint32_t start[kWalkThreads];
+  constexpr uint32_t kIdentity = 0x76543210u;
+  const uint32_t t = blockIdx.x, i = threadIdx.x;
+  const uint32_t c0 = b.chunk_prefix[t], nc = b.chunk_prefix[t + 1] - c0;
+  if (nc <= 1) return;
+  const uint32_t run = (nc + kWalkThreads - 1) / kWalkThreads;
+  const uint32_t a = min(nc, i * run), e = min(nc, a + run);
+  uint32_t g = kIdentity;
+  for (uint32_t k = a; k < e; ++k) g = then(g, sc.tab[c0 + k]);
+  f[i] = g;
+  __syncthreads();
+  if (i < 32) {
+    constexpr uint32_t kPer = kWalkThreads / 32;
+    g = kIdentity;
+#pragma unroll
+    for (uint32_t k = 0; k < kPer; ++k) g = then(g, f[i * kPer + k]);
+    uint32_t s = (uint32_t)stream_head(b, t) >> (HIGH ? 4 : 0) & 15u, mine = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < 32; ++k) {
+      if (k == i) mine = s;
+      s = through(__shfl_sync(0xffffffffu, g, k), s);
     }
-    return;
-  }
-  const uint32_t nc = c1 - c0;
-  // row of chunk c0 + j into slot j % kWalkAhead; one commit group per call, empty past the end
-  auto fetch = [&](uint32_t j) {
-    if (j < nc && lane < 16)
-      cp_async16(smem_u32(rows[j % kWalkAhead] + lane * 16), sc.ltab + (size_t)(c0 + j) * 256 + lane * 16);
-    cp_async_commit();
-  };
-  for (uint32_t j = 0; j < (uint32_t)kWalkAhead; ++j) fetch(j);
-  uint32_t l = h.lo & 0xffu;
-  for (uint32_t j = 0; j < nc; ++j) {
-    cp_async_wait<kWalkAhead - 1>();  // this lane's copy of row j has landed
-    __syncwarp();                     // and every lane's
-    if (lane == 0) {
-      sc.lstart[c0 + j] = l;
-      l = rows[j % kWalkAhead][l];
+#pragma unroll
+    for (uint32_t k = 0; k < kPer; ++k) {
+      start[i * kPer + k] = mine;
+      mine = through(f[i * kPer + k], mine);
     }
-    __syncwarp();  // lane 0 is done with slot j % kWalkAhead before it is refilled
-    fetch(j + kWalkAhead);
   }
-  cp_async_wait<0>();
-  if (lane == 0) sc.head[t] = h.value();
-}
-
-// Pass 3: one thread per chunk, the low word from its starting low byte: B = lo_end - p^m l.
-__global__ void fnv_bpart_kernel(const __grid_constant__ FnvBatch b, FnvScratch sc) {
-  const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= b.chunk_prefix[b.n]) return;
-  uint64_t first, last;
-  chunk_range(b, c, first, last);
-  const uint32_t l = sc.lstart[c];
-  FnvLo h{l};
-  fnv_leaf_run(h, sc.leaves, first, last);
-  sc.bpart[c] = h.lo - fnv_pow(8 * (uint32_t)(last - first)) * l;
-}
-
-// Pass 4: one thread per chunked buffer, lo at every chunk start.
-__global__ void fnv_scan_kernel(const __grid_constant__ FnvBatch b, FnvScratch sc) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= b.n) return;
-  const uint32_t c0 = b.chunk_prefix[t], c1 = b.chunk_prefix[t + 1];
-  if (c0 == c1) return;
-  const uint64_t l0 = b.leaf_prefix[t], l1 = b.leaf_prefix[t + 1];
-  const uint32_t pfull = fnv_pow(8 * kChunkWords);
-  const uint64_t head = sc.head[t];
-  uint32_t lo = (uint32_t)head;
-  for (uint32_t c = c0; c < c1; ++c) {
-    sc.lo_start[c] = lo;
-    const uint64_t first = l0 + (uint64_t)(c - c0) * kChunkWords;
-    const uint32_t w = (uint32_t)min((uint64_t)kChunkWords, l1 - first);
-    lo = (w == kChunkWords ? pfull : fnv_pow(8 * w)) * lo + sc.bpart[c];
+  __syncthreads();
+  uint32_t s = start[i];
+  for (uint32_t k = a; k < e; ++k) {
+    sc.lstart[c0 + k] = HIGH ? sc.lstart[c0 + k] | s << 4 : s;
+    s = through(sc.tab[c0 + k], s);
   }
-  sc.head[t] = (head & 0xffffffff00000000ull) | lo;
 }
 
-// Pass 5: one thread per chunk, the exact chain from (lo_start, 0).
-__global__ void fnv_exact_kernel(const __grid_constant__ FnvBatch b, FnvScratch sc) {
-  const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= b.chunk_prefix[b.n]) return;
-  uint64_t first, last;
-  chunk_range(b, c, first, last);
-  Fnv h;
-  h.lo = sc.lo_start[c];
-  h.hi = 0;
-  fnv_leaf_run(h, sc.leaves, first, last);
-  sc.hpart[c] = h.hi;
-}
-
-// Pass 6: one thread per chunked buffer, hi folded over its chunks.
-__global__ void fnv_finish_kernel(const __grid_constant__ FnvBatch b, FnvScratch sc) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= b.n) return;
-  const uint32_t c0 = b.chunk_prefix[t], c1 = b.chunk_prefix[t + 1];
-  if (c0 == c1) return;
-  const uint64_t l0 = b.leaf_prefix[t], l1 = b.leaf_prefix[t + 1];
-  const uint32_t pfull = fnv_pow(8 * kChunkWords);
-  const uint64_t head = sc.head[t];
-  uint32_t hi = (uint32_t)(head >> 32);
-  for (uint32_t c = c0; c < c1; ++c) {
-    const uint64_t first = l0 + (uint64_t)(c - c0) * kChunkWords;
-    const uint32_t w = (uint32_t)min((uint64_t)kChunkWords, l1 - first);
-    hi = (w == kChunkWords ? pfull : fnv_pow(8 * w)) * hi + sc.hpart[c];
+// Pass 6: one block per buffer folds h = p^m h + D over its chunks: each thread its run of whole
+// chunks by Horner's rule, moved to the end of the whole chunks by a power of p^m; the sum of
+// those; then the last chunk.
+template <class Tab>
+__global__ void __launch_bounds__(kWalkThreads) fnv_fold_kernel(const __grid_constant__ Tab b, FnvScratch sc) {
+  __shared__ uint64_t part[kWalkThreads / 32];
+  const uint32_t t = blockIdx.x, i = threadIdx.x;
+  const uint32_t c0 = b.chunk_prefix[t], nc = b.chunk_prefix[t + 1] - c0;
+  const uint32_t whole = nc ? nc - 1 : 0;
+  uint64_t h = 0;
+  if (whole) {
+    const uint32_t run = (whole + kWalkThreads - 1) / kWalkThreads;
+    const uint32_t a = min(whole, i * run), e = min(whole, a + run);
+    for (uint32_t k = a; k < e; ++k) h = h * b.chunk_pow + sc.sum[c0 + k];
+    if (a < e) h *= fnv_pow(b.chunk_pow, whole - e);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+    if ((i & 31) == 0) part[i >> 5] = h;
+    __syncthreads();
   }
-  *b.out[t] = ((uint64_t)hi << 32) | (uint32_t)head;
+  if (i != 0) return;
+  h = stream_head(b, t);
+  if (whole) {
+    h *= fnv_pow(b.chunk_pow, whole);
+    for (int w = 0; w < kWalkThreads / 32; ++w) h += part[w];
+  }
+  if (nc) {
+    const uint32_t len = (uint32_t)(stream_bytes(b, t) - (uint64_t)whole * b.chunk);
+    h = h * fnv_pow(kFnvPrime, len) + sc.sum[c0 + whole];
+  }
+  b.out[t] = h;
 }
 
 // One thread per buffer: the literal serial FNV-1a-64.
@@ -408,20 +443,19 @@ __global__ void fnv_plain_kernel(const __grid_constant__ FnvBatch b) {
   const uint64_t nv = (n - i) >> 4;
   for (uint64_t k = 0; k < nv; ++k) h.vec(v[k]);
   for (i += nv << 4; i < n; ++i) h.byte(p[i]);
-  *b.out[t] = h.value();
+  b.out[t] = h.value();
 }
 
 }  // namespace
 
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Scratch layout of one batch: leaves, ltab, lstart, bpart, lo_start, hpart, head
-// (256-byte aligned).
+// Scratch layout of one batch: the leaf digests (whole chunks, up to a whole warp's), then the
+// per-chunk arrays, each 256-byte aligned.
 static FnvScratch fnv_layout(const FnvBatch &b, void *base, size_t *bytes) {
-  const uint64_t L = b.leaf_prefix[b.n];
-  const uint64_t C = b.chunk_prefix[b.n];
-  constexpr int kParts = 7;
-  const size_t len[kParts] = {L * 8, C * 256, C * 4, C * 4, C * 4, C * 4, (size_t)b.n * 8};
+  const size_t C = b.chunk_prefix[b.n];
+  constexpr int kParts = 4;
+  const size_t len[kParts] = {((C + 31) & ~(size_t)31) * kTreeChunk, C * 4, C * 4, C * 8};
   size_t off[kParts];
   size_t o = 0;
   for (int i = 0; i < kParts; ++i) {
@@ -432,72 +466,94 @@ static FnvScratch fnv_layout(const FnvBatch &b, void *base, size_t *bytes) {
   FnvScratch sc;
   const uintptr_t p = reinterpret_cast<uintptr_t>(base);
   sc.leaves = reinterpret_cast<uint64_t *>(p + off[0]);
-  sc.ltab = reinterpret_cast<uint8_t *>(p + off[1]);
+  sc.tab = reinterpret_cast<uint32_t *>(p + off[1]);
   sc.lstart = reinterpret_cast<uint32_t *>(p + off[2]);
-  sc.bpart = reinterpret_cast<uint32_t *>(p + off[3]);
-  sc.lo_start = reinterpret_cast<uint32_t *>(p + off[4]);
-  sc.hpart = reinterpret_cast<uint32_t *>(p + off[5]);
-  sc.head = reinterpret_cast<uint64_t *>(p + off[6]);
+  sc.sum = reinterpret_cast<uint64_t *>(p + off[3]);
   return sc;
 }
 
-size_t fnv_fill_batch(FnvBatch &b, const void *const *ptr, const uint64_t *nbytes, uint64_t *const *out, size_t n) {
-  memset(&b, 0, sizeof b);
-  b.n = (uint32_t)n;
-  uint64_t leaves = 0;
-  uint32_t chunks = 0;
-  for (size_t k = 0; k < n; ++k) {
-    b.leaf_prefix[k] = leaves;
-    b.chunk_prefix[k] = chunks;
+size_t fnv_fill_batch(FnvBatch &b, const void *const *ptr, const uint64_t *nbytes, uint64_t *out, size_t n, bool plain,
+                      size_t *taken) {
+  uint64_t leaves = 0, chunks = 0;
+  b.out = out;
+  b.chunk = kTreeChunk;
+  size_t k = 0;
+  for (; k < n && k < (size_t)kMaxFnv; ++k) {
+    const uint64_t l = (nbytes[k] + kLeafBytes - 1) / kLeafBytes;
+    if (k && leaves + l > 1ull << 31) break;
+    b.leaf_prefix[k] = (uint32_t)leaves;
+    b.chunk_prefix[k] = (uint32_t)chunks;
     b.ptr[k] = static_cast<const uint8_t *>(ptr[k]);
     b.nbytes[k] = nbytes[k];
-    b.out[k] = out[k];
-    const uint64_t l = (nbytes[k] + kLeafBytes - 1) / kLeafBytes;
     leaves += l;
-    if (l > kParallelLeaves) chunks += (uint32_t)((l + kChunkWords - 1) / kChunkWords);
+    chunks += (l + kChunkLeaves - 1) / kChunkLeaves;
   }
-  b.leaf_prefix[n] = leaves;
-  b.chunk_prefix[n] = chunks;
+  b.n = (uint32_t)k;
+  b.leaf_prefix[k] = (uint32_t)leaves;
+  b.chunk_prefix[k] = (uint32_t)chunks;
+  b.chunk_pow = fnv_pow(kFnvPrime, b.chunk);
+  *taken = k;
   size_t bytes = 0;
-  fnv_layout(b, nullptr, &bytes);
+  if (!plain) fnv_layout(b, nullptr, &bytes);
   return bytes;
+}
+
+// A buffer of more than one chunk makes the table and walk passes necessary.
+static bool fnv_chained(const FnvBatch &b) {
+  for (uint32_t t = 0; t < b.n; ++t)
+    if (b.chunk_prefix[t + 1] - b.chunk_prefix[t] > 1) return true;
+  return false;
 }
 
 int fnv_tree_launches(const FnvBatch &b) {
   if (b.n == 0) return 0;
-  return (b.leaf_prefix[b.n] ? 1 : 0) + 1 + (b.chunk_prefix[b.n] ? 5 : 0);
+  return (b.chunk_prefix[b.n] ? 2 : 0) + (fnv_chained(b) ? 4 : 0) + 1;
 }
+
+template <class Tab>
+static cudaError_t run_fnv_tree(const Tab &b, const FnvScratch &sc, bool chained, cudaStream_t s) {
+  const uint64_t total = b.leaf_prefix[b.n];
+  const uint32_t blocks = (b.chunk_prefix[b.n] + kChunkWarps * 32 - 1) / (kChunkWarps * 32);
+  if (total > 0) {
+    const uint64_t warps = (total + 31) / 32;
+    const uint64_t want = (warps + kFnvWarps - 1) / kFnvWarps;
+    const uint64_t cap = (uint64_t)num_sms() * 24;
+    fnv_leaf_kernel<Tab><<<(int)(want < cap ? want : cap), kFnvWarps * 32, 0, s>>>(b, sc.leaves);
+    if (chained) {
+      fnv_chunk_kernel<Tab, 0><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
+      fnv_walk_kernel<Tab, false><<<b.n, kWalkThreads, 0, s>>>(b, sc);
+      fnv_chunk_kernel<Tab, 1><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
+      fnv_walk_kernel<Tab, true><<<b.n, kWalkThreads, 0, s>>>(b, sc);
+    }
+    fnv_chunk_kernel<Tab, 2><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
+  }
+  fnv_fold_kernel<Tab><<<b.n, kWalkThreads, 0, s>>>(b, sc);
+  return cudaGetLastError();
+}
+
+// The same batch with a table of `Tab`'s size: a call of few buffers passes a small parameter.
+template <class Tab>
+static Tab shrink(const FnvBatch &b) {
+  Tab t;
+  t.n = b.n;
+  t.chunk = b.chunk;
+  t.chunk_pow = b.chunk_pow;
+  t.out = b.out;
+  memcpy(t.ptr, b.ptr, b.n * sizeof b.ptr[0]);
+  memcpy(t.nbytes, b.nbytes, b.n * sizeof b.nbytes[0]);
+  memcpy(t.leaf_prefix, b.leaf_prefix, (b.n + 1) * sizeof b.leaf_prefix[0]);
+  memcpy(t.chunk_prefix, b.chunk_prefix, (b.n + 1) * sizeof b.chunk_prefix[0]);
+  return t;
+}
+
+using FnvSmall = FnvTab<32>;
 
 cudaError_t launch_fnv_tree(const FnvBatch &b, void *scratch, cudaStream_t s) {
   if (b.n == 0) return cudaSuccess;
   const FnvScratch sc = fnv_layout(b, scratch, nullptr);
-  const uint64_t total = b.leaf_prefix[b.n];
-  const uint32_t chunks = b.chunk_prefix[b.n];
-  cudaError_t e;
-  if (total > 0) {
-    const uint64_t warps = (total + 31) / 32;
-    const uint64_t blocks = (warps + kFnvWarps - 1) / kFnvWarps;
-    const uint64_t cap = (uint64_t)num_sms() * 24;
-    fnv_leaf_kernel<<<(int)(blocks < cap ? blocks : cap), kFnvWarps * 32, 0, s>>>(b, sc.leaves);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (chunks) {
-    fnv_table_kernel<<<chunks, 64, 0, s>>>(b, sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  fnv_combine_kernel<<<b.n, 32, 0, s>>>(b, sc);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (chunks) {
-    fnv_bpart_kernel<<<(chunks + 127) / 128, 128, 0, s>>>(b, sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    fnv_scan_kernel<<<(b.n + 127) / 128, 128, 0, s>>>(b, sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    fnv_exact_kernel<<<(chunks + 127) / 128, 128, 0, s>>>(b, sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    fnv_finish_kernel<<<(b.n + 127) / 128, 128, 0, s>>>(b, sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  const bool chained = fnv_chained(b);
+  if (b.n <= (uint32_t)FnvSmall::kMax) return run_fnv_tree(shrink<FnvSmall>(b), sc, chained, s);
+  return run_fnv_tree(b, sc, chained, s);
 }
 
 cudaError_t launch_fnv_plain(const FnvBatch &b, cudaStream_t s) {

@@ -10,37 +10,44 @@
 namespace wt {
 
 // ---------------------------------------------------------------- FNV-1a-64
-constexpr int kMaxFnv = 512;  // buffers per launch: the batch is an 18 KB kernel parameter
 constexpr uint64_t kLeafBytes = 4096;
 // Largest buffer a digest call accepts (1 TiB, above any device's memory): bounds the leaf and
 // chunk counts so that no size the caller passes can wrap them.
 constexpr uint64_t kMaxFnvBufferBytes = 1ull << 40;
 
-// The tree digest's second level is a serial FNV chain over 8 bytes per leaf.  Buffers of
-// more than kParallelLeaves leaves split that chain into chunks of kChunkWords leaf digests
-// and combine the chunks in parallel (exact; see the kernels), others run it in one thread.
-constexpr uint64_t kParallelLeaves = 4096;
-constexpr uint32_t kChunkWords = 512;
+// The tree digest's second level is a serial FNV chain over 8 bytes per leaf.  It runs in
+// chunks of kTreeChunk bytes, one thread each, combined exactly (see the kernels).
+constexpr uint32_t kTreeChunk = 256;
+constexpr uint32_t kChunkLeaves = kTreeChunk / 8;
 
-struct FnvBatch {
+// The buffers of one batch, as a kernel parameter.  24 bytes each, so that the largest
+// batch just fits the 32,764-byte parameter space.
+template <int N>
+struct FnvTab {
+  static constexpr int kMax = N;
   uint32_t n;
-  uint32_t pad;
-  uint64_t leaf_prefix[kMaxFnv + 1];   // first global leaf of buffer i; [n] = total leaves
-  uint32_t chunk_prefix[kMaxFnv + 1];  // first global chunk of buffer i; [n] = total chunks
-  const uint8_t *ptr[kMaxFnv];
-  uint64_t nbytes[kMaxFnv];
-  uint64_t *out[kMaxFnv];  // device address of the digest of buffer i
+  uint32_t chunk;       // bytes of a chunk of the serial stream
+  uint64_t chunk_pow;   // p^chunk mod 2^64
+  uint64_t *out;        // device address of the first buffer's digest (contiguous)
+  const uint8_t *ptr[N];
+  uint64_t nbytes[N];
+  uint32_t leaf_prefix[N + 1];   // first leaf of buffer i in the batch; [n] = total
+  uint32_t chunk_prefix[N + 1];  // first chunk of buffer i in the batch; [n] = total
 };
+constexpr int kMaxFnv = 1344;  // buffers per batch
+using FnvBatch = FnvTab<kMaxFnv>;
 
-// Fills n, ptr, nbytes, out and both prefixes from the buffers; returns the device scratch
-// bytes launch_fnv_tree needs for the batch (leaf digests, then the chunk tables).
-size_t fnv_fill_batch(FnvBatch &b, const void *const *ptr, const uint64_t *nbytes, uint64_t *const *out, size_t n);
+// Device scratch per chunk beyond the leaf digests: a transition table, the starting low byte
+// and the chunk's sum.
+constexpr size_t kChunkScratchBytes = 4 + 4 + 8;
 
-// Device scratch per chunk of the parallel second level: a 256-entry low-byte table and four
-// 32-bit words (starting low byte, B, starting lo, H).
-constexpr size_t kChunkScratchBytes = 256 + 4 * 4;
+// Fills b with the leading buffers of the list (*taken of them, at least one) and returns the
+// device scratch bytes that launch_fnv_tree, or with `plain` launch_fnv_plain, needs for them.
+// Digest i goes to out[i].
+size_t fnv_fill_batch(FnvBatch &b, const void *const *ptr, const uint64_t *nbytes, uint64_t *out, size_t n, bool plain,
+                      size_t *taken);
 
-// Kernel launches of launch_fnv_tree for the batch: leaves, combine, and five chunk passes.
+// Kernel launches of launch_fnv_tree for the batch.
 int fnv_tree_launches(const FnvBatch &b);
 
 cudaError_t launch_fnv_tree(const FnvBatch &b, void *scratch, cudaStream_t s);

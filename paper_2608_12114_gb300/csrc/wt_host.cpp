@@ -2391,12 +2391,10 @@ static int checksum_impl(wt_handle *h, const void *const *ptr, const uint64_t *n
   }
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   std::lock_guard<std::mutex> g(h->mu);
-  std::vector<uint64_t *> outs(n);
-  for (size_t i = 0; i < n; ++i) outs[i] = out_dev + i;
-  for (size_t i0 = 0; i0 < n; i0 += wt::kMaxFnv) {
-    const size_t m = std::min<size_t>(wt::kMaxFnv, n - i0);
-    std::unique_ptr<wt::FnvBatch> b(new wt::FnvBatch);
-    const size_t scratch = wt::fnv_fill_batch(*b, ptr + i0, nbytes + i0, outs.data() + i0, m);
+  std::unique_ptr<wt::FnvBatch> b(new (std::nothrow) wt::FnvBatch);
+  if (!b) return set_err(WT_ENOMEM, "wt_checksum: out of host memory");
+  for (size_t i0 = 0, m = 0; i0 < n; i0 += m) {
+    const size_t scratch = wt::fnv_fill_batch(*b, ptr + i0, nbytes + i0, out_dev + i0, n - i0, plain, &m);
     if (plain) {
       CU(wt::launch_fnv_plain(*b, s));
       h->kernel_launches++;

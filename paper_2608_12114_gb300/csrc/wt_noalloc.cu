@@ -33,11 +33,10 @@
 namespace {
 
 constexpr uint64_t kNoAllocMaxLeaves = 1ull << 20;  // 4096-byte leaves: 4 GiB of input per call
-// leaf digests plus the chunk tables of the parallel second level (at most one chunk per
-// kChunkWords leaves and one partial chunk per buffer of a batch)
-constexpr uint64_t kNoAllocWords =
-    kNoAllocMaxLeaves +
-    ((kNoAllocMaxLeaves / wt::kChunkWords + wt::kMaxFnv) * wt::kChunkScratchBytes + wt::kMaxFnv * 8 + 2048) / 8;
+// whole chunks of leaf digests (at most one chunk per kChunkLeaves leaves, one partial chunk
+// per buffer of a batch, and the rest of a warp's 32) and the second level's per-chunk arrays
+constexpr uint64_t kNoAllocChunks = kNoAllocMaxLeaves / wt::kChunkLeaves + wt::kMaxFnv + 32;
+constexpr uint64_t kNoAllocWords = (kNoAllocChunks * (wt::kTreeChunk + wt::kChunkScratchBytes) + 1024) / 8;
 __device__ __align__(256) uint64_t g_noalloc_leaves[kNoAllocWords];
 
 std::mutex g_mu;
@@ -111,12 +110,9 @@ extern "C" __attribute__((visibility("default"))) int wt_checksum_noalloc(
   }
   // Batches run in order on one stream, so each reuses the array from slot 0.
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
-  static thread_local wt::FnvBatch b;  // 18 KB: kept off the stack
-  uint64_t *outs[wt::kMaxFnv];
-  for (size_t i0 = 0; i0 < n; i0 += wt::kMaxFnv) {
-    const size_t m = n - i0 < (size_t)wt::kMaxFnv ? n - i0 : (size_t)wt::kMaxFnv;
-    for (size_t k = 0; k < m; ++k) outs[k] = out_dev + i0 + k;
-    const size_t need = wt::fnv_fill_batch(b, ptr + i0, nbytes + i0, outs, m);
+  static thread_local wt::FnvBatch b;  // 32 KB: kept off the stack
+  for (size_t i0 = 0, m = 0; i0 < n; i0 += m) {
+    const size_t need = wt::fnv_fill_batch(b, ptr + i0, nbytes + i0, out_dev + i0, n - i0, false, &m);
     if (need > sizeof(g_noalloc_leaves)) return fail(WT_EINVAL, "wt_checksum_noalloc: batch scratch exceeds the fixed array");
     e = wt::launch_fnv_tree(b, scratch, s);
     if (e != cudaSuccess) {

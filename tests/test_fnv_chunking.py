@@ -95,3 +95,70 @@ def test_chunked_chain_over_real_leaf_digests():
     leaves = [oracle.fnv1a64(data[i:i + 4096]) for i in range(0, data.size, 4096)]
     stream = struct.pack("<%dQ" % len(leaves), *leaves)
     assert chunked(struct.pack("<Q", data.size), stream, 8 * 5) == oracle.fnv_tree(data)
+
+
+# ----------------------------------------------------------------------------- nibble by nibble
+
+M64 = (1 << 64) - 1
+PRIME = 0x100000001B3
+
+
+def chain(h, data):
+    for b in data:
+        h = ((h ^ b) * PRIME) & M64
+    return h
+
+
+def nibble_tables(chunk, nib=None):
+    """The packed lanes of the chunk passes: the low nibble from starts 0..7 (eight-bit lanes,
+    multiplier 3), or with `nib` the high nibble from starts nib + 16 j (sixteen-bit lanes)."""
+    if nib is None:
+        regs, mask, mul, rep, width = [0x03020100, 0x07060504], 0x0F0F0F0F, 3, 0x01010101, 8
+    else:
+        regs = [(nib + 32 * i) | (nib + 32 * i + 16) << 16 for i in range(4)]
+        mask, mul, rep, width = 0x00FF00FF, 0xB3, 0x00010001, 16
+    for b in chunk:
+        for i, r in enumerate(regs):
+            u = (r ^ (b * rep)) & mask
+            assert all((u >> s & ((1 << width) - 1)) * mul < 1 << width for s in range(0, 32, width))
+            regs[i] = (u * mul) & 0xFFFFFFFF
+    lanes = [r >> s for r in regs for s in range(0, 32, width)]
+    return [v & 15 if nib is None else v >> 4 & 15 for v in lanes]
+
+
+def through(table, s):
+    return table[s & 7] ^ (s & 8)
+
+
+def chained(head, stream, m):
+    """h after `stream` from state `head`, in chunks of m bytes: low nibbles, high nibbles, the
+    64-bit sums D, the fold."""
+    chunks = [stream[i:i + m] for i in range(0, len(stream), m)]
+    low, s = [], head & 15
+    for c in chunks:
+        low.append(s)
+        s = through(nibble_tables(c), s)
+    start, s = [], head >> 4 & 15
+    for c, nib in zip(chunks, low):
+        start.append(nib | s << 4)
+        s = through(nibble_tables(c, nib), s)
+    h = head
+    for c, l in zip(chunks, start):
+        assert h & 0xFF == l
+        pm = pow(PRIME, len(c), 1 << 64)
+        h = (pm * h + chain(l, c) - pm * l) & M64
+    return h
+
+
+@pytest.mark.parametrize("n,m", [(1, 8), (7, 8), (8, 8), (1000, 24), (700, 256)])
+def test_nibble_chunks_equal_the_serial_chain(n, m):
+    rng = np.random.default_rng(n + m)
+    for fill in (None, 0, 255):
+        data = rng.integers(0, 256, n, dtype=np.uint8) if fill is None else np.full(n, fill, np.uint8)
+        assert chained(0xCBF29CE484222325, data.tobytes(), m) == oracle.fnv1a64(data)
+    tables = [nibble_tables(data.tobytes())] + [nibble_tables(data.tobytes(), k) for k in range(16)]
+    for t, table in enumerate(tables):  # the 8 starts that are not run follow from the 8 that are
+        for s in range(16):
+            l = s if t == 0 else (t - 1) | s << 4
+            end = chain(l, data.tobytes())
+            assert through(table, s) == (end & 15 if t == 0 else end >> 4 & 15)

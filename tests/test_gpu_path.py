@@ -316,6 +316,23 @@ def test_checksum_chunked_second_level(torch):
         assert got == want, noalloc
 
 
+@pytest.mark.parametrize("leaves", [(1, 31, 32, 33, 64, 65), (0, 1, 1025, 0, 2, 255 * 32 + 1), (257 * 32 + 5, 3),
+                                    (2,) * 1344, (1, 40) * 700])
+def test_checksum_second_level_chunks(torch, leaves):
+    """Second-level streams around one chunk (32 leaves), one chunk per walking thread (256
+    chunks) and one batch (1344 buffers), with empty buffers between; ragged last leaves."""
+    rng = np.random.default_rng(len(leaves))
+    sizes = [max(0, 4096 * n - int(rng.integers(0, 4096))) for n in leaves]
+    data = rng.integers(0, 256, max(sizes) + 16 * 64, dtype=np.uint8)
+    buf = torch.from_numpy(data).cuda()
+    offs = [16 * (i % 64) for i in range(len(sizes))]
+    with wt.Handle([]) as h:
+        out = torch.zeros(len(sizes), dtype=torch.int64, device="cuda")
+        h.checksum([buf.data_ptr() + o for o in offs], sizes, out.data_ptr(), 0)
+        got = [int(v) & (2 ** 64 - 1) for v in out.cpu().tolist()]
+    assert got == [oracle.fnv_tree(data[o:o + n]) for o, n in zip(offs, sizes)]
+
+
 def test_unaligned_operands_take_the_generic_kernel(torch):
     """W and x 2 bytes past a 16-byte boundary (element-aligned only): the scalar fallback,
     checked against the oracle; one and several columns."""
