@@ -292,8 +292,10 @@ int wt_pass(wt_handle *h, const wt_gemv_desc *d, size_t n, void *stream);
 int wt_checksum(wt_handle *h, const void *const *ptr, const uint64_t *nbytes, size_t n,
                 uint64_t *out_dev, void *stream);
 
-/* Literal FNV-1a-64 of each device buffer (one serial chain per buffer; meant
- * for verification).  Buffers above 256 MiB are rejected with WT_EINVAL. */
+/* Literal FNV-1a-64 of each device buffer (meant for verification).  Buffers above 256 MiB
+ * are rejected with WT_EINVAL.  The serial chain of a buffer runs in parallel chunks with
+ * temporary stream-ordered storage (about 2 bytes for each 256 of input at most); where none
+ * is to be had, and inside a stream capture, one thread runs each buffer above 64 KiB. */
 int wt_checksum_plain(wt_handle *h, const void *const *ptr, const uint64_t *nbytes, size_t n,
                       uint64_t *out_dev, void *stream);
 

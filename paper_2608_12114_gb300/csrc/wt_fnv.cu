@@ -2,6 +2,7 @@
 // file's: the literal serial digest, and the tree digest (FNV-1a-64 of each 4 KiB leaf,
 // then FNV-1a-64 over the buffer's length and its leaf digests).  The second level of the
 // tree runs in parallel chunks, with the exact result of the serial chain.
+#include <algorithm>
 #include <cstring>
 
 #include "wt_device.cuh"
@@ -217,7 +218,9 @@ __global__ void __launch_bounds__(kFnvWarps * 32) fnv_leaf_kernel(const __grid_c
 // one chunk goes this way: 256-byte chunks keep the passes at a few microseconds each.
 // Measured on GB300 (whole calls, leaves included): 2.97 GB with two 1 GB tensors 1332 -> 814
 // us, 1253 tensors of 8 KiB to 8 MiB (1.56 GB) 1261 -> 457 us, against whole-byte tables over
-// 4096-byte chunks for buffers above 16 MiB and one thread per buffer below.
+// 4096-byte chunks for buffers above 16 MiB and one thread per buffer below; 797 and 443 us
+// with short streams in one block each and the tables of long ones loaded ahead.  The literal
+// digest of eight 16 MiB tensors, one thread each before: 276 ms -> 0.19 ms.
 
 // p^e mod 2^64 by square and multiply
 __host__ __device__ __forceinline__ uint64_t fnv_pow(uint64_t q, uint32_t e) {
@@ -294,30 +297,50 @@ __device__ __forceinline__ uint32_t through(uint32_t table, uint32_t s) {
 }
 // The table of `a` followed by `b`.
 __device__ __forceinline__ uint32_t then(uint32_t a, uint32_t b) {
-  uint32_t t = 0;
+  uint32_t t = a & 0x88888888u;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) t |= through(b, a >> (4 * j) & 15u) << (4 * j);
+  for (int j = 0; j < 8; ++j) t ^= (b >> ((a >> (4 * j) & 7u) << 2) & 15u) << (4 * j);
   return t;
 }
+constexpr uint32_t kIdentity = 0x76543210u;
 
-// State at the start of buffer t's serial stream, and the stream's bytes: the tree digest's
-// second level starts after LE64(nbytes) and runs over the leaf digests.
-template <class Tab>
+// Walks n tables f[0..n) from start s with one warp: start[k] becomes the state before table k.
+__device__ __forceinline__ void walk_tables(const uint32_t *f, uint32_t *start, uint32_t n, uint32_t s, int lane) {
+  const uint32_t per = (n + 31) / 32;
+  const uint32_t a = min(n, lane * per), e = min(n, a + per);
+  uint32_t g = kIdentity, mine = 0;
+  for (uint32_t k = a; k < e; ++k) g = then(g, f[k]);
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    if (k == lane) mine = s;
+    s = through(__shfl_sync(0xffffffffu, g, k), s);
+  }
+  for (uint32_t k = a; k < e; ++k) {
+    start[k] = mine;
+    mine = through(f[k], mine);
+  }
+}
+
+// A buffer's serial stream: its own bytes from FNV's offset basis (PLAIN, the literal digest),
+// or the leaf digests from the state after LE64(nbytes) (the tree digest's second level).
+template <bool PLAIN, class Tab>
 __device__ __forceinline__ uint64_t stream_head(const Tab &b, uint32_t t) {
   Fnv h;
-  h.le64(b.nbytes[t]);
+  if constexpr (!PLAIN) h.le64(b.nbytes[t]);
   return h.value();
 }
-template <class Tab>
+template <bool PLAIN, class Tab>
 __device__ __forceinline__ uint64_t stream_bytes(const Tab &b, uint32_t t) {
+  if constexpr (PLAIN) return b.nbytes[t];
   return 8ull * (b.leaf_prefix[t + 1] - b.leaf_prefix[t]);
 }
 
 // Passes 1, 3 and 5 (PASS 0, 1, 2): one thread per chunk.  Blocks of two warps spread a few
 // thousand chunks over the SMs.  The leaf digests of a batch lie in whole chunks one after
-// another (and up to a whole warp's), so every row may be read to its end.
+// another (and up to a whole warp's), so every row may be read to its end; a caller's bytes
+// take the coalesced copies where a warp's 32 chunks are whole, aligned and of one buffer.
 constexpr int kChunkWarps = 2;
-template <class Tab, int PASS>
+template <bool PLAIN, class Tab, int PASS>
 __global__ void __launch_bounds__(kChunkWarps * 32) fnv_chunk_kernel(const __grid_constant__ Tab b, FnvScratch sc) {
   __shared__ __align__(16) uint8_t buf[kChunkWarps][2][32][kSliceStride];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -328,88 +351,110 @@ __global__ void __launch_bounds__(kChunkWarps * 32) fnv_chunk_kernel(const __gri
   if (c < total) {
     t = find_in(b.chunk_prefix, b.n, c);
     nchunk = b.chunk_prefix[t + 1] - b.chunk_prefix[t];
-    len = (uint32_t)min((uint64_t)b.chunk, stream_bytes(b, t) - (uint64_t)(c - b.chunk_prefix[t]) * b.chunk);
+    len = (uint32_t)min((uint64_t)b.chunk, stream_bytes<PLAIN>(b, t) - (uint64_t)(c - b.chunk_prefix[t]) * b.chunk);
   }
   // a buffer of one chunk starts from a known state: it needs no table
   const bool mine = PASS == 2 ? nchunk > 0 : nchunk > 1;
   if (!mine) len = 0;
-  const uint8_t *wbase = reinterpret_cast<const uint8_t *>(sc.leaves) + (uint64_t)first * b.chunk;
-  const uint8_t *lp = wbase + (uint64_t)lane * b.chunk;
+  const uint8_t *wbase, *lp = nullptr;
+  bool fast = true;
+  if constexpr (PLAIN) {
+    if (mine) lp = b.ptr[t] + (uint64_t)(c - b.chunk_prefix[t]) * b.chunk;
+    wbase = reinterpret_cast<const uint8_t *>(__shfl_sync(0xffffffffu, (unsigned long long)lp, 0));
+    const uint32_t t0 = __shfl_sync(0xffffffffu, t, 0);
+    fast = __all_sync(0xffffffffu, mine && t == t0 && len == b.chunk && (reinterpret_cast<uintptr_t>(lp) & 15) == 0);
+  } else {
+    wbase = reinterpret_cast<const uint8_t *>(sc.leaves) + (uint64_t)first * b.chunk;
+    lp = wbase + (uint64_t)lane * b.chunk;
+  }
   if constexpr (PASS == 0) {
     LowNibble h;
-    run_rows(h, buf[warp], lp, len, true, wbase, b.chunk, lane);
+    run_rows(h, buf[warp], lp, len, fast, wbase, b.chunk, lane);
     if (mine) sc.tab[c] = h.table();
   } else if constexpr (PASS == 1) {
     HighNibble h(mine ? sc.lstart[c] : 0);
-    run_rows(h, buf[warp], lp, len, true, wbase, b.chunk, lane);
+    run_rows(h, buf[warp], lp, len, fast, wbase, b.chunk, lane);
     if (mine) sc.tab[c] = h.table();
   } else {
     uint32_t l = 0;
-    if (mine) l = nchunk > 1 ? sc.lstart[c] : (uint32_t)stream_head(b, t) & 0xffu;
+    if (mine) l = nchunk > 1 ? sc.lstart[c] : (uint32_t)stream_head<PLAIN>(b, t) & 0xffu;
     Fnv h;
     h.lo = l;
     h.hi = 0;
-    run_rows(h, buf[warp], lp, len, true, wbase, b.chunk, lane);
+    run_rows(h, buf[warp], lp, len, fast, wbase, b.chunk, lane);
     if (mine) sc.sum[c] = h.value() - (len == b.chunk ? b.chunk_pow : fnv_pow(kFnvPrime, len)) * l;
   }
 }
 
 // Passes 2 and 4 (HIGH): one block per buffer.  Each thread composes the tables of a run of
-// chunks, warp 0 composes and walks the threads' tables, and each thread walks its run.
-constexpr int kWalkThreads = 256;
-template <class Tab, bool HIGH>
+// chunks, warp 0 walks the threads' tables, and each thread walks its run.  The run's tables
+// are loaded eight at a time: loaded one by one by 256 threads, the L2 round trips made this
+// pass 21 us (ncu, cold, 8018 chunks) where it now takes 14.
+constexpr int kWalkThreads = 1024;
+template <bool PLAIN, class Tab, bool HIGH>
 __global__ void __launch_bounds__(kWalkThreads) fnv_walk_kernel(const __grid_constant__ Tab b, FnvScratch sc) {
   __shared__ uint32_t f[kWalkThreads];
   __shared__ uint32_t start[kWalkThreads];
-  constexpr uint32_t kIdentity = 0x76543210u;
+  constexpr uint32_t kAhead = 8;
   const uint32_t t = blockIdx.x, i = threadIdx.x;
   const uint32_t c0 = b.chunk_prefix[t], nc = b.chunk_prefix[t + 1] - c0;
   if (nc <= 1) return;
   const uint32_t run = (nc + kWalkThreads - 1) / kWalkThreads;
   const uint32_t a = min(nc, i * run), e = min(nc, a + run);
+  const uint32_t *tab = sc.tab + c0;
+  uint32_t *ls = sc.lstart + c0;
   uint32_t g = kIdentity;
-  for (uint32_t k = a; k < e; ++k) g = then(g, sc.tab[c0 + k]);
+  for (uint32_t k = a; k < e; k += kAhead) {
+    uint32_t v[kAhead];
+#pragma unroll
+    for (uint32_t j = 0; j < kAhead; ++j) v[j] = k + j < e ? tab[k + j] : kIdentity;
+#pragma unroll
+    for (uint32_t j = 0; j < kAhead; ++j) g = then(g, v[j]);
+  }
   f[i] = g;
   __syncthreads();
-  if (i < 32) {
-    constexpr uint32_t kPer = kWalkThreads / 32;
-    g = kIdentity;
-#pragma unroll
-    for (uint32_t k = 0; k < kPer; ++k) g = then(g, f[i * kPer + k]);
-    uint32_t s = (uint32_t)stream_head(b, t) >> (HIGH ? 4 : 0) & 15u, mine = 0;
-#pragma unroll
-    for (uint32_t k = 0; k < 32; ++k) {
-      if (k == i) mine = s;
-      s = through(__shfl_sync(0xffffffffu, g, k), s);
-    }
-#pragma unroll
-    for (uint32_t k = 0; k < kPer; ++k) {
-      start[i * kPer + k] = mine;
-      mine = through(f[i * kPer + k], mine);
-    }
-  }
+  if (i < 32) walk_tables(f, start, (nc + run - 1) / run, (uint32_t)stream_head<PLAIN>(b, t) >> (HIGH ? 4 : 0) & 15u, i);
   __syncthreads();
+  if (a >= e) return;
   uint32_t s = start[i];
-  for (uint32_t k = a; k < e; ++k) {
-    sc.lstart[c0 + k] = HIGH ? sc.lstart[c0 + k] | s << 4 : s;
-    s = through(sc.tab[c0 + k], s);
+  for (uint32_t k = a; k < e; k += kAhead) {
+    uint32_t v[kAhead], l[kAhead];
+#pragma unroll
+    for (uint32_t j = 0; j < kAhead; ++j) {
+      v[j] = k + j < e ? tab[k + j] : kIdentity;
+      l[j] = HIGH && k + j < e ? ls[k + j] : 0;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kAhead; ++j) {
+      if (k + j < e) ls[k + j] = HIGH ? l[j] | s << 4 : s;
+      s = through(v[j], s);
+    }
   }
 }
 
 // Pass 6: one block per buffer folds h = p^m h + D over its chunks: each thread its run of whole
 // chunks by Horner's rule, moved to the end of the whole chunks by a power of p^m; the sum of
 // those; then the last chunk.
-template <class Tab>
-__global__ void __launch_bounds__(kWalkThreads) fnv_fold_kernel(const __grid_constant__ Tab b, FnvScratch sc) {
-  __shared__ uint64_t part[kWalkThreads / 32];
+constexpr int kFoldThreads = 256;
+template <bool PLAIN, class Tab>
+__global__ void __launch_bounds__(kFoldThreads) fnv_fold_kernel(const __grid_constant__ Tab b, FnvScratch sc) {
+  __shared__ uint64_t part[kFoldThreads / 32];
   const uint32_t t = blockIdx.x, i = threadIdx.x;
   const uint32_t c0 = b.chunk_prefix[t], nc = b.chunk_prefix[t + 1] - c0;
   const uint32_t whole = nc ? nc - 1 : 0;
   uint64_t h = 0;
   if (whole) {
-    const uint32_t run = (whole + kWalkThreads - 1) / kWalkThreads;
+    const uint32_t run = (whole + kFoldThreads - 1) / kFoldThreads;
     const uint32_t a = min(whole, i * run), e = min(whole, a + run);
-    for (uint32_t k = a; k < e; ++k) h = h * b.chunk_pow + sc.sum[c0 + k];
+    constexpr uint32_t kAhead = 8;
+    for (uint32_t k = a; k < e; k += kAhead) {
+      uint64_t v[kAhead];
+#pragma unroll
+      for (uint32_t j = 0; j < kAhead; ++j) v[j] = k + j < e ? sc.sum[c0 + k + j] : 0;
+#pragma unroll
+      for (uint32_t j = 0; j < kAhead; ++j)
+        if (k + j < e) h = h * b.chunk_pow + v[j];
+    }
     if (a < e) h *= fnv_pow(b.chunk_pow, whole - e);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
@@ -417,20 +462,105 @@ __global__ void __launch_bounds__(kWalkThreads) fnv_fold_kernel(const __grid_con
     __syncthreads();
   }
   if (i != 0) return;
-  h = stream_head(b, t);
+  h = stream_head<PLAIN>(b, t);
   if (whole) {
     h *= fnv_pow(b.chunk_pow, whole);
-    for (int w = 0; w < kWalkThreads / 32; ++w) h += part[w];
+    for (int w = 0; w < kFoldThreads / 32; ++w) h += part[w];
   }
   if (nc) {
-    const uint32_t len = (uint32_t)(stream_bytes(b, t) - (uint64_t)whole * b.chunk);
+    const uint32_t len = (uint32_t)(stream_bytes<PLAIN>(b, t) - (uint64_t)whole * b.chunk);
     h = h * fnv_pow(kFnvPrime, len) + sc.sum[c0 + whole];
   }
   b.out[t] = h;
 }
 
-// One thread per buffer: the literal serial FNV-1a-64.
-__global__ void fnv_plain_kernel(const __grid_constant__ FnvBatch b) {
+// All six passes of a buffer of at most kBlockChunks chunks in one block: the stream is copied
+// to shared memory once, rows padded by 16 bytes so that the threads' reads of their own rows
+// fall in different banks, and each thread runs its chunk three times from there.
+constexpr uint32_t kBlockChunks = 256;
+constexpr uint32_t kRowPitch = kTreeChunk + 16;
+
+template <class H>
+__device__ __forceinline__ void run_row(H &h, const uint8_t *row, uint32_t len) {
+  uint32_t k = 0;
+  for (; k + 16 <= len; k += 16) h.vec(*reinterpret_cast<const uint4 *>(row + k));
+  for (; k < len; ++k) h.byte(row[k]);
+}
+
+template <bool PLAIN, class Tab>
+__global__ void __launch_bounds__(kBlockChunks) fnv_block_kernel(const __grid_constant__ Tab b, const uint64_t *leaves) {
+  extern __shared__ __align__(16) uint8_t rows[];
+  __shared__ uint32_t f[kBlockChunks], low[kBlockChunks], high[kBlockChunks];
+  __shared__ uint64_t part[kBlockChunks / 32];
+  const uint32_t t = blockIdx.x, i = threadIdx.x;
+  const uint32_t c0 = b.chunk_prefix[t], nc = b.chunk_prefix[t + 1] - c0;
+  const uint64_t head = stream_head<PLAIN>(b, t);
+  if (nc == 0) {
+    if (i == 0) b.out[t] = head;
+    return;
+  }
+  const uint32_t n = (uint32_t)stream_bytes<PLAIN>(b, t);
+  const uint8_t *src = PLAIN ? b.ptr[t] : reinterpret_cast<const uint8_t *>(leaves) + (uint64_t)c0 * kTreeChunk;
+  uint32_t k = 0;
+  if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    for (k = i * 16; k + 16 <= n; k += blockDim.x * 16)
+      *reinterpret_cast<uint4 *>(rows + k / kTreeChunk * kRowPitch + k % kTreeChunk) =
+          *reinterpret_cast<const uint4 *>(src + k);
+    k = n & ~15u;
+  }
+  for (k += i; k < n; k += blockDim.x) rows[k / kTreeChunk * kRowPitch + k % kTreeChunk] = src[k];
+  __syncthreads();
+  const uint8_t *row = rows + i * kRowPitch;
+  const uint32_t len = i < nc ? min(kTreeChunk, n - i * kTreeChunk) : 0;
+  uint32_t l = (uint32_t)head & 0xffu;
+  if (nc > 1) {
+    if (i < nc) {
+      LowNibble h;
+      run_row(h, row, len);
+      f[i] = h.table();
+    }
+    __syncthreads();
+    if (i < 32) walk_tables(f, low, nc, l & 15u, i);
+    __syncthreads();
+    if (i < nc) {
+      HighNibble h(low[i]);
+      run_row(h, row, len);
+      f[i] = h.table();
+    }
+    __syncthreads();
+    if (i < 32) walk_tables(f, high, nc, l >> 4, i);
+    __syncthreads();
+    if (i < nc) l = low[i] | high[i] << 4;
+  }
+  uint64_t sum = 0, last = 0;
+  if (i < nc) {
+    Fnv h;
+    h.lo = l;
+    h.hi = 0;
+    run_row(h, row, len);
+    const bool final_chunk = i == nc - 1;
+    sum = h.value() - (len == kTreeChunk ? b.chunk_pow : fnv_pow(kFnvPrime, len)) * l;
+    if (final_chunk) {
+      last = sum;
+      sum = 0;
+    } else {
+      sum *= fnv_pow(b.chunk_pow, nc - 2 - i);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((i & 31) == 0) part[i >> 5] = sum;
+  __syncthreads();
+  if (i == nc - 1) {
+    uint64_t h = head * fnv_pow(b.chunk_pow, nc - 1);
+    for (uint32_t w = 0; w < blockDim.x / 32; ++w) h += part[w];
+    b.out[t] = h * fnv_pow(kFnvPrime, len) + last;
+  }
+}
+
+// One thread per buffer: the literal serial FNV-1a-64, for short buffers and without scratch.
+template <class Tab>
+__global__ void fnv_plain_kernel(const __grid_constant__ Tab b) {
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= b.n) return;
   const uint8_t *p = b.ptr[t];
@@ -448,14 +578,21 @@ __global__ void fnv_plain_kernel(const __grid_constant__ FnvBatch b) {
 
 }  // namespace
 
+// Chunks a literal digest aims at: enough threads to fill the GPU, few enough that one block
+// per buffer composes their tables quickly.
+constexpr uint64_t kPlainChunks = 1 << 17;
+// A literal digest of buffers up to this length runs one thread per buffer: 6 us of call at 256
+// bytes, 10 at 512 and 16 at 1024, where a block takes 12 from 1 to 4 KiB and 17 at 64 KiB.
+constexpr uint64_t kSerialBytes = 640;
+
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Scratch layout of one batch: the leaf digests (whole chunks, up to a whole warp's), then the
-// per-chunk arrays, each 256-byte aligned.
-static FnvScratch fnv_layout(const FnvBatch &b, void *base, size_t *bytes) {
+// Scratch layout of one batch: the tree digest's leaf digests (whole chunks, up to a whole
+// warp's), then the per-chunk arrays, each 256-byte aligned.
+static FnvScratch fnv_layout(const FnvBatch &b, bool plain, void *base, size_t *bytes) {
   const size_t C = b.chunk_prefix[b.n];
   constexpr int kParts = 4;
-  const size_t len[kParts] = {((C + 31) & ~(size_t)31) * kTreeChunk, C * 4, C * 4, C * 8};
+  const size_t len[kParts] = {plain ? 0 : ((C + 31) & ~(size_t)31) * kTreeChunk, C * 4, C * 4, C * 8};
   size_t off[kParts];
   size_t o = 0;
   for (int i = 0; i < kParts; ++i) {
@@ -472,62 +609,93 @@ static FnvScratch fnv_layout(const FnvBatch &b, void *base, size_t *bytes) {
   return sc;
 }
 
+// Chunks of the batch's longest stream.
+static uint32_t longest_stream(const FnvBatch &b) {
+  uint32_t m = 0;
+  for (uint32_t t = 0; t < b.n; ++t) m = std::max(m, b.chunk_prefix[t + 1] - b.chunk_prefix[t]);
+  return m;
+}
+// One block takes a stream of up to kBlockChunks chunks of kTreeChunk bytes: a call of 12 to 17
+// us (64 KiB) where six launches take 32.  Longer streams need more than one SM.
+static bool in_blocks(const FnvBatch &b, uint32_t longest) { return longest <= kBlockChunks && b.chunk == kTreeChunk; }
+
 size_t fnv_fill_batch(FnvBatch &b, const void *const *ptr, const uint64_t *nbytes, uint64_t *out, size_t n, bool plain,
                       size_t *taken) {
-  uint64_t leaves = 0, chunks = 0;
-  b.out = out;
-  b.chunk = kTreeChunk;
+  uint64_t leaves = 0, chunks = 0, bytes = 0;
   size_t k = 0;
   for (; k < n && k < (size_t)kMaxFnv; ++k) {
     const uint64_t l = (nbytes[k] + kLeafBytes - 1) / kLeafBytes;
     if (k && leaves + l > 1ull << 31) break;
-    b.leaf_prefix[k] = (uint32_t)leaves;
-    b.chunk_prefix[k] = (uint32_t)chunks;
-    b.ptr[k] = static_cast<const uint8_t *>(ptr[k]);
-    b.nbytes[k] = nbytes[k];
     leaves += l;
-    chunks += (l + kChunkLeaves - 1) / kChunkLeaves;
+    bytes += nbytes[k];
   }
   b.n = (uint32_t)k;
+  b.out = out;
+  b.chunk = kTreeChunk;
+  if (plain)  // about kPlainChunks chunks a call, of 256 to 4096 bytes
+    while (b.chunk < kLeafBytes && bytes / b.chunk > kPlainChunks) b.chunk *= 2;
+  b.chunk_pow = fnv_pow(kFnvPrime, b.chunk);
+  leaves = 0;
+  for (size_t i = 0; i < k; ++i) {
+    const uint64_t l = (nbytes[i] + kLeafBytes - 1) / kLeafBytes;
+    b.leaf_prefix[i] = (uint32_t)leaves;
+    b.chunk_prefix[i] = (uint32_t)chunks;
+    b.ptr[i] = static_cast<const uint8_t *>(ptr[i]);
+    b.nbytes[i] = nbytes[i];
+    leaves += l;
+    chunks += plain ? (nbytes[i] + b.chunk - 1) / b.chunk : (l + kChunkLeaves - 1) / kChunkLeaves;
+  }
   b.leaf_prefix[k] = (uint32_t)leaves;
   b.chunk_prefix[k] = (uint32_t)chunks;
-  b.chunk_pow = fnv_pow(kFnvPrime, b.chunk);
   *taken = k;
-  size_t bytes = 0;
-  if (!plain) fnv_layout(b, nullptr, &bytes);
-  return bytes;
-}
-
-// A buffer of more than one chunk makes the table and walk passes necessary.
-static bool fnv_chained(const FnvBatch &b) {
-  for (uint32_t t = 0; t < b.n; ++t)
-    if (b.chunk_prefix[t + 1] - b.chunk_prefix[t] > 1) return true;
-  return false;
+  size_t need = 0;
+  if (!plain || !in_blocks(b, longest_stream(b))) fnv_layout(b, plain, nullptr, &need);
+  return need;
 }
 
 int fnv_tree_launches(const FnvBatch &b) {
   if (b.n == 0) return 0;
-  return (b.chunk_prefix[b.n] ? 2 : 0) + (fnv_chained(b) ? 4 : 0) + 1;
+  return (b.chunk_prefix[b.n] ? 1 : 0) + (in_blocks(b, longest_stream(b)) ? 1 : 6);
+}
+
+// The serial streams of a batch (passes 1 to 6).
+template <bool PLAIN, class Tab>
+static cudaError_t run_fnv_streams(const Tab &b, const FnvScratch &sc, bool blocks_do, uint32_t longest, cudaStream_t s) {
+  if (blocks_do) {
+    const uint32_t threads = std::max(32u, (longest + 31) / 32 * 32);
+    const size_t smem = (size_t)longest * kRowPitch;
+    const cudaError_t e = cudaFuncSetAttribute(fnv_block_kernel<PLAIN, Tab>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(kBlockChunks * kRowPitch));
+    if (e != cudaSuccess) return e;
+    fnv_block_kernel<PLAIN, Tab><<<b.n, threads, smem, s>>>(b, sc.leaves);
+    return cudaGetLastError();
+  }
+  const uint32_t blocks = (b.chunk_prefix[b.n] + kChunkWarps * 32 - 1) / (kChunkWarps * 32);
+  fnv_chunk_kernel<PLAIN, Tab, 0><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
+  fnv_walk_kernel<PLAIN, Tab, false><<<b.n, kWalkThreads, 0, s>>>(b, sc);
+  fnv_chunk_kernel<PLAIN, Tab, 1><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
+  fnv_walk_kernel<PLAIN, Tab, true><<<b.n, kWalkThreads, 0, s>>>(b, sc);
+  fnv_chunk_kernel<PLAIN, Tab, 2><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
+  fnv_fold_kernel<PLAIN, Tab><<<b.n, kFoldThreads, 0, s>>>(b, sc);
+  return cudaGetLastError();
 }
 
 template <class Tab>
-static cudaError_t run_fnv_tree(const Tab &b, const FnvScratch &sc, bool chained, cudaStream_t s) {
+static cudaError_t run_fnv_tree(const Tab &b, const FnvScratch &sc, bool blocks_do, uint32_t longest, cudaStream_t s) {
   const uint64_t total = b.leaf_prefix[b.n];
-  const uint32_t blocks = (b.chunk_prefix[b.n] + kChunkWarps * 32 - 1) / (kChunkWarps * 32);
   if (total > 0) {
     const uint64_t warps = (total + 31) / 32;
     const uint64_t want = (warps + kFnvWarps - 1) / kFnvWarps;
     const uint64_t cap = (uint64_t)num_sms() * 24;
     fnv_leaf_kernel<Tab><<<(int)(want < cap ? want : cap), kFnvWarps * 32, 0, s>>>(b, sc.leaves);
-    if (chained) {
-      fnv_chunk_kernel<Tab, 0><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
-      fnv_walk_kernel<Tab, false><<<b.n, kWalkThreads, 0, s>>>(b, sc);
-      fnv_chunk_kernel<Tab, 1><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
-      fnv_walk_kernel<Tab, true><<<b.n, kWalkThreads, 0, s>>>(b, sc);
-    }
-    fnv_chunk_kernel<Tab, 2><<<blocks, kChunkWarps * 32, 0, s>>>(b, sc);
   }
-  fnv_fold_kernel<Tab><<<b.n, kWalkThreads, 0, s>>>(b, sc);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : run_fnv_streams<false>(b, sc, blocks_do, longest, s);
+}
+
+template <class Tab>
+static cudaError_t run_fnv_serial(const Tab &b, cudaStream_t s) {
+  fnv_plain_kernel<Tab><<<(b.n + 63) / 64, 64, 0, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -550,16 +718,35 @@ using FnvSmall = FnvTab<32>;
 
 cudaError_t launch_fnv_tree(const FnvBatch &b, void *scratch, cudaStream_t s) {
   if (b.n == 0) return cudaSuccess;
-  const FnvScratch sc = fnv_layout(b, scratch, nullptr);
-  const bool chained = fnv_chained(b);
-  if (b.n <= (uint32_t)FnvSmall::kMax) return run_fnv_tree(shrink<FnvSmall>(b), sc, chained, s);
-  return run_fnv_tree(b, sc, chained, s);
+  const FnvScratch sc = fnv_layout(b, false, scratch, nullptr);
+  const uint32_t longest = longest_stream(b);
+  if (b.n <= (uint32_t)FnvSmall::kMax) return run_fnv_tree(shrink<FnvSmall>(b), sc, in_blocks(b, longest), longest, s);
+  return run_fnv_tree(b, sc, in_blocks(b, longest), longest, s);
 }
 
-cudaError_t launch_fnv_plain(const FnvBatch &b, cudaStream_t s) {
+// How a literal digest runs: serially (0), in blocks (1), or with all six passes (2).
+static int plain_way(const FnvBatch &b, bool scratch) {
+  if (in_blocks(b, longest_stream(b))) {
+    for (uint32_t t = 0; t < b.n; ++t)
+      if (b.nbytes[t] > kSerialBytes) return 1;
+    return 0;
+  }
+  return scratch ? 2 : 0;
+}
+
+int fnv_plain_launches(const FnvBatch &b, bool scratch) { return b.n == 0 ? 0 : plain_way(b, scratch) == 2 ? 6 : 1; }
+
+cudaError_t launch_fnv_plain(const FnvBatch &b, void *scratch, cudaStream_t s) {
   if (b.n == 0) return cudaSuccess;
-  fnv_plain_kernel<<<(b.n + 63) / 64, 64, 0, s>>>(b);
-  return cudaGetLastError();
+  const int way = plain_way(b, scratch != nullptr);
+  const uint32_t longest = longest_stream(b);
+  FnvScratch sc{};
+  if (way == 2) sc = fnv_layout(b, true, scratch, nullptr);
+  if (b.n <= (uint32_t)FnvSmall::kMax) {
+    const FnvSmall t = shrink<FnvSmall>(b);
+    return way ? run_fnv_streams<true>(t, sc, way == 1, longest, s) : run_fnv_serial(t, s);
+  }
+  return way ? run_fnv_streams<true>(b, sc, way == 1, longest, s) : run_fnv_serial(b, s);
 }
 
 }  // namespace wt

@@ -2395,17 +2395,22 @@ static int checksum_impl(wt_handle *h, const void *const *ptr, const uint64_t *n
   if (!b) return set_err(WT_ENOMEM, "wt_checksum: out of host memory");
   for (size_t i0 = 0, m = 0; i0 < n; i0 += m) {
     const size_t scratch = wt::fnv_fill_batch(*b, ptr + i0, nbytes + i0, out_dev + i0, n - i0, plain, &m);
+    void *sc = nullptr;
     if (plain) {
-      CU(wt::launch_fnv_plain(*b, s));
-      h->kernel_launches++;
+      // The literal digest needs no scratch: where none can be had, and inside a capture (the
+      // graph then holds no allocation), one thread runs each buffer.
+      cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+      if (scratch && cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+          cudaMallocAsync(&sc, scratch, s) != cudaSuccess)
+        sc = nullptr;
+      cudaGetLastError();
     } else {
-      void *sc = nullptr;
       CU(cudaMallocAsync(&sc, scratch, s));
-      const cudaError_t e = wt::launch_fnv_tree(*b, sc, s);
-      cudaFreeAsync(sc, s);
-      CU(e);
-      h->kernel_launches += wt::fnv_tree_launches(*b);
     }
+    const cudaError_t e = plain ? wt::launch_fnv_plain(*b, sc, s) : wt::launch_fnv_tree(*b, sc, s);
+    if (sc) cudaFreeAsync(sc, s);
+    CU(e);
+    h->kernel_launches += plain ? wt::fnv_plain_launches(*b, sc != nullptr) : wt::fnv_tree_launches(*b);
   }
   return WT_OK;
 }

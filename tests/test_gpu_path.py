@@ -333,6 +333,22 @@ def test_checksum_second_level_chunks(torch, leaves):
     assert got == [oracle.fnv_tree(data[o:o + n]) for o, n in zip(offs, sizes)]
 
 
+@pytest.mark.parametrize("sizes", [(639, 640), (641, 0, 3, 256 * 256), (256 * 257 + 1, 31 * 256, 8192, 5),
+                                   (1 << 22, (1 << 22) + 4095), (40 << 20,), (2000,) * 40])
+def test_plain_digest_chunks(torch, sizes):
+    """The literal digest around the serial line (640 bytes), one chunk per walking thread, and
+    the longer chunks of larger calls; aligned and unaligned starts."""
+    rng = np.random.default_rng(len(sizes) + sizes[0])
+    data = rng.integers(0, 256, max(sizes) + 64, dtype=np.uint8)
+    buf = torch.from_numpy(data).cuda()
+    for off in (0, 16, 5):
+        with wt.Handle([]) as h:
+            out = torch.zeros(len(sizes), dtype=torch.int64, device="cuda")
+            h.checksum([buf.data_ptr() + off] * len(sizes), sizes, out.data_ptr(), 0, plain=True)
+            got = [int(v) & (2 ** 64 - 1) for v in out.cpu().tolist()]
+        assert got == [oracle.fnv1a64(data[off:off + n]) for n in sizes]
+
+
 def test_unaligned_operands_take_the_generic_kernel(torch):
     """W and x 2 bytes past a 16-byte boundary (element-aligned only): the scalar fallback,
     checked against the oracle; one and several columns."""
