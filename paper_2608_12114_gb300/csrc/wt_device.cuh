@@ -29,6 +29,11 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
                : "memory");
 }
 
+// Raises the transaction count alone, without the arrival.
+__device__ __forceinline__ void mbar_expect_only(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -113,6 +118,30 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
 
 __device__ __forceinline__ uint4 lds_or_zero(uint32_t addr, bool ok) {
   return ok ? lds128(addr) : make_uint4(0, 0, 0, 0);
+}
+
+__device__ __forceinline__ void sts8(uint32_t addr, uint8_t v) {
+  asm volatile("st.shared.u8 [%0], %1;" ::"r"(addr), "r"((uint32_t)v) : "memory");
+}
+
+// The 16 bytes from byte `ph` (0..15) of the 32 bytes lo, hi on: two word selects and four
+// funnel shifts.
+__device__ __forceinline__ uint4 shift_bytes(const uint4 &lo, const uint4 &hi, uint32_t ph) {
+  uint32_t q0 = lo.x, q1 = lo.y, q2 = lo.z, q3 = lo.w, q4 = hi.x, q5 = hi.y;
+  if (ph & 8) q0 = lo.z, q1 = lo.w, q2 = hi.x, q3 = hi.y, q4 = hi.z, q5 = hi.w;
+  if (ph & 4) q0 = q1, q1 = q2, q2 = q3, q3 = q4, q4 = q5;
+  const uint32_t b = (ph & 3) * 8;
+  return make_uint4(__funnelshift_r(q0, q1, b), __funnelshift_r(q1, q2, b), __funnelshift_r(q2, q3, b),
+                    __funnelshift_r(q3, q4, b));
+}
+
+// 16 bytes of shared memory from any address: the two vectors that hold them.  Bytes past the
+// caller's data may be read (from the vector that holds its last byte, or the next).
+__device__ __forceinline__ uint4 lds_shifted(uint32_t addr) {
+  const uint32_t ph = addr & 15u;
+  const uint4 lo = lds128(addr - ph);
+  const uint4 hi = lds128(addr - ph + (ph ? 16 : 0));
+  return shift_bytes(lo, hi, ph);
 }
 
 // Two int8 weights as exact f16x2.  With u = b ^ 0x80 (0..255) in the low byte and 0x64 in

@@ -365,6 +365,7 @@ struct Plan {
     bool umma = false;           // multi-column launch on tcgen05 (wt_umma.cu)
     bool q8rows = false;         // int8 multi-column launch on the row-owner kernel (wt_q8rows.cu)
     bool mapped_cols = false;    // map endpoint with T columns
+    bool ragged = false;         // one-column kernel: some matrix has ragged rows
     int nt = 0;                  // warp-MMA multi-column launches: 8-column tiles (1 or 2)
     uint32_t nmat = 0, ntiles = 0;
   };
@@ -1138,7 +1139,7 @@ wt::MatDesc make_mat(const wt_gemv_desc &d) {
   m.y = d.y;
   m.s = static_cast<const uint8_t *>(d.scale);
   m.M = (uint32_t)d.M;
-  m.V = (uint32_t)(d.K * es / 16);
+  m.V = (uint32_t)((d.K * es + 15) / 16);
   m.rs = m.V;
   const uint32_t rowb = m.V * 16;
   // a consumer thread keeps at most 8 (bf16/f16/f32) or 2 (int8: 16 f16 activations per
@@ -1163,6 +1164,23 @@ wt::MatDesc make_mat(const wt_gemv_desc &d) {
   return m;
 }
 
+// Ragged rows for the one-column kernel: rows that are no whole number of 16-byte vectors, or
+// whose W or x does not lie on a 16-byte boundary.  A row's vectors count from the grid point
+// (16 bytes; int8: 8) at or before its start, so their number depends on the row's phase: G
+// is for the most.  A stage also holds the phases of its first and last row (whole
+// rows in one copy), or one more vector per row (column segments).
+constexpr uint32_t kRaggedSlack = 32;  // bytes of a stage
+uint32_t phase_vectors(uint64_t row_bytes, int dtype) { return (uint32_t)((row_bytes + (dtype == WT_I8 ? 7 : 15) + 15) / 16); }
+
+void make_ragged(wt::MatDesc &m, int dtype, uint64_t row_bytes, uint64_t pitch_bytes) {
+  const uint32_t nv = phase_vectors(row_bytes, dtype);
+  m.mode = wt::kModePhaseRows;
+  m.rb = (uint32_t)row_bytes;
+  m.rs = (uint32_t)pitch_bytes;
+  m.G = (uint16_t)(nv <= 32 ? pow2ceil(nv) : 32);
+  m.rt = (wt::kStageBytes - kRaggedSlack) / (row_bytes == pitch_bytes ? m.rb : (m.V + 1) * 16);
+}
+
 // Multi-column kernel: chunks of at most kColVecMax vectors per row, evened out over the row
 // and rounded up to 4 (mod 8): 448 vectors -> 5 chunks of 92 (the last box zero-filled past
 // the row's end).
@@ -1184,32 +1202,37 @@ wt::MatDesc make_cols_mat(const wt_gemv_desc &d) {
   return m;
 }
 
-// Segment length for rows of V vectors: ceil(V / seg_vectors) segments of nearly equal
-// length (a multiple of 8 vectors), so no segment is a sliver.  Depends on (V, dtype) only.
-uint32_t seg_length(uint32_t V, int dtype) {
-  const uint32_t S = wt::seg_vectors(dtype);
+// The longest row (and row segment) of the one-column kernel in vectors.
+uint32_t seg_max(int dtype, bool ragged) { return ragged ? wt::kPhaseVec(dtype) - 8 : wt::seg_vectors(dtype); }
+
+// Segment length for rows of V vectors: ceil(V / seg_max) segments of nearly equal
+// length (a multiple of 8 vectors), so no segment is a sliver.  Depends on (V, dtype, ragged)
+// only.
+uint32_t seg_length(uint32_t V, int dtype, bool ragged) {
+  const uint32_t S = seg_max(dtype, ragged);
   const uint32_t nseg = (V + S - 1) / S;
   return ((V + nseg - 1) / nseg + 7) / 8 * 8;
 }
 
-// Column segment k of a matrix whose rows exceed seg_vectors(dtype): vectors
+// Column segment k of a matrix whose rows exceed seg_max vectors: vectors
 // [k S, min((k + 1) S, V)) of every row, S = seg_length (row pitch: the full row), x
 // advanced to match, no scale, tile mode chosen by the segment's own length, y left for the
 // workspace patch.
-wt::MatDesc make_seg_mat(const wt_gemv_desc &d, uint32_t k) {
+wt::MatDesc make_seg_mat(const wt_gemv_desc &d, uint32_t k, bool ragged) {
   const int es = elem_bytes(d.dtype);
-  const uint32_t V = (uint32_t)(d.K * es / 16);
-  const uint32_t S = seg_length(V, d.dtype);
+  const uint32_t V = (uint32_t)((d.K * es + 15) / 16);
+  const uint32_t S = seg_length(V, d.dtype, ragged);
   const uint64_t xvb = d.dtype == WT_I8 ? 32 : 16;  // x bytes per 16-byte weight vector
   const uint32_t v0 = k * S;
   wt_gemv_desc sd = d;
   sd.W = static_cast<const uint8_t *>(d.W) + (uint64_t)v0 * 16;
   sd.x = static_cast<const uint8_t *>(d.x) + (uint64_t)v0 * xvb;
-  sd.K = (uint64_t)std::min(S, V - v0) * 16 / es;
+  sd.K = std::min<uint64_t>((uint64_t)S * 16 / es, d.K - (uint64_t)v0 * 16 / es);
   sd.scale = nullptr;
   wt::MatDesc m = make_mat(sd);
   m.s = nullptr;
-  m.rs = V;
+  if (ragged) make_ragged(m, d.dtype, sd.K * es, d.K * es);
+  else m.rs = V;
   return m;
 }
 
@@ -1601,29 +1624,36 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         q1.cols = 1;
         i8c[0].push_back(make_cols_mat(q1));
         i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
-      } else if (fast && q.K * es / 16 > wt::seg_vectors(q.dtype)) {
-        // long rows: column segments spread over CTAs, summed by the second pass
-        const uint32_t V = (uint32_t)(q.K * es / 16);
-        const uint32_t S = seg_length(V, q.dtype);
-        const uint32_t nseg = (V + S - 1) / S;
-        const size_t off = P->ws_floats;
-        P->ws_floats += (size_t)nseg * q.M;
-        for (uint32_t k = 0; k < nseg; ++k) {
-          by_dt[q.dtype].push_back(make_seg_mat(q, k));
-          seg_ws[q.dtype].push_back((int64_t)(off + (size_t)k * q.M));
+      } else if (q.cols == 0 && (fast || q.K * es < 0x7fffffffull)) {
+        // device memory, one column: whole 16-byte vectors per row, or ragged rows (any K, W
+        // and x at any byte), which the one-warp-per-row kernel streamed at 500 to 2500 GB/s
+        // and the phase rows stream at 4000 to 6900
+        const uint32_t V = (uint32_t)((q.K * es + 15) / 16);
+        if (V <= seg_max(q.dtype, !fast)) {
+          wt::MatDesc m = make_mat(q);
+          if (!fast) make_ragged(m, q.dtype, q.K * es, q.K * es);
+          by_dt[q.dtype].push_back(m);
+          seg_ws[q.dtype].push_back(-1);
+        } else {
+          // long rows: column segments spread over CTAs, summed by the second pass
+          const uint32_t S = seg_length(V, q.dtype, !fast);
+          const uint32_t nseg = (V + S - 1) / S;
+          const size_t off = P->ws_floats;
+          P->ws_floats += (size_t)nseg * q.M;
+          for (uint32_t k = 0; k < nseg; ++k) {
+            by_dt[q.dtype].push_back(make_seg_mat(q, k, !fast));
+            seg_ws[q.dtype].push_back((int64_t)(off + (size_t)k * q.M));
+          }
+          wt::SegReduce r;
+          memset(&r, 0, sizeof r);
+          r.y = q.y;
+          r.s = static_cast<const uint8_t *>(q.scale);
+          r.M = (uint32_t)q.M;
+          r.nseg = nseg;
+          reds.push_back(r);
+          red_ws.push_back(off);
+          g.reduce_rows = std::max(g.reduce_rows, (uint32_t)q.M);
         }
-        wt::SegReduce r;
-        memset(&r, 0, sizeof r);
-        r.y = q.y;
-        r.s = static_cast<const uint8_t *>(q.scale);
-        r.M = (uint32_t)q.M;
-        r.nseg = nseg;
-        reds.push_back(r);
-        red_ws.push_back(off);
-        g.reduce_rows = std::max(g.reduce_rows, (uint32_t)q.M);
-      } else if (fast) {
-        by_dt[q.dtype].push_back(make_mat(q));
-        seg_ws[q.dtype].push_back(-1);
       } else {
         g.generic.push_back({q.dtype, static_cast<const uint8_t *>(q.W), static_cast<const uint8_t *>(q.x), q.y, q.M, q.K,
                              static_cast<const uint8_t *>(q.scale), ncol});
@@ -1695,8 +1725,9 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         }
         if (pass == 0)
           for (const wt::MatDesc &m : ms)
-            if (m.mode != wt::kModeWarpRows && m.mode != wt::kModeBlockRows)
+            if (m.mode != wt::kModeWarpRows && m.mode != wt::kModeBlockRows && m.mode != wt::kModePhaseRows)
               return set_err(WT_ENOTSUP, "wt_pass: internal: a %u-vector row reached the TMA kernel unsegmented", m.V);
+        for (const wt::MatDesc &m : ms) L.ragged |= m.rb != 0;
         L.nt = pass == 2 ? 1 : pass == 5 ? 2 : 0;
         partition(ms, L.grid, pieces, begin, warp_mma ? (uint32_t)wt::kColTileRows : 1u,
                   pass == 0 ? one_col_slices(dt) : 1,
@@ -1819,6 +1850,7 @@ int run_plan(wt_handle *h, Plan *P, const wt_gemv_desc *d, cudaStream_t s, bool 
       gl.pieces = reinterpret_cast<const wt::Piece *>(P->dev + L.pieces);
       gl.begin = reinterpret_cast<const uint32_t *>(P->dev + L.begin);
       gl.status = h->status;
+      gl.ragged = L.ragged;
       gl.stall = wt::fault_injected("stall") ? 1 : 0;
       // Inside a captured graph of consecutive passes, each pass may start its launch and
       // prologue while the previous one finishes (a programmatic edge); a group gated on an

@@ -171,8 +171,17 @@ struct GemvGeo {
   static constexpr size_t kRedOff = kBarOff + 2 * kStages * sizeof(uint64_t);
   static constexpr size_t kFlagOff = kRedOff + 2 * kConsumerWarps * kRedRows * sizeof(float);
   static constexpr size_t kSmem = kFlagOff + 16;
+  // the ragged instantiation also stages x of one matrix: 16 zero bytes, its bytes, zeros up to
+  // the end of the last vector of any phase
+  static constexpr int kPhaseNJ = kPhaseVec(DT) / 32;
+  static constexpr size_t kXOff = kSmem;
+  static constexpr size_t kXBytes = 16 + (size_t)kPhaseNJ * 32 * (DT == 3 ? 32 : 16) + 64;
+  static constexpr size_t kSmemRagged = kXOff + kXBytes;
 };
 static_assert(GemvGeo<1>::kSmem <= 232448 && 2 * (GemvGeo<3>::kSmem + 1024) <= 233472, "GEMV shared memory");
+static_assert(GemvGeo<1>::kSmemRagged <= 232448 && 2 * (GemvGeo<3>::kSmemRagged + 1024) <= 233472 &&
+                  GemvGeo<1>::kXOff % 16 == 0 && GemvGeo<3>::kXOff % 16 == 0,
+              "ragged GEMV shared memory");
 
 // Two fp32 values in one 64-bit register; fma.rn.f32x2 performs two independent
 // round-to-nearest FMAs (the same arithmetic as two fmaf calls) in one instruction.
@@ -218,6 +227,19 @@ __device__ __forceinline__ float fma_h2(uint32_t a, uint32_t b, float c) {
       "mov.b32 {bl, bh}, %2;\n\t"
       "fma.rn.f32.f16 %0, al, bl, %3;\n\t"
       "fma.rn.f32.f16 %0, ah, bh, %0;\n\t}"
+      : "=f"(d)
+      : "r"(a), "r"(b), "f"(c));
+  return d;
+}
+
+// The same for bf16 operands.
+__device__ __forceinline__ float fma_b2(uint32_t a, uint32_t b, float c) {
+  float d;
+  asm("{\n\t.reg .b16 al, ah, bl, bh;\n\t"
+      "mov.b32 {al, ah}, %1;\n\t"
+      "mov.b32 {bl, bh}, %2;\n\t"
+      "fma.rn.f32.bf16 %0, al, bl, %3;\n\t"
+      "fma.rn.f32.bf16 %0, ah, bh, %0;\n\t}"
       : "=f"(d)
       : "r"(a), "r"(b), "f"(c));
   return d;
@@ -454,16 +476,282 @@ __device__ __forceinline__ void stamp_full(uint64_t *st, uint32_t it, int warp, 
   }
 }
 
+// ------------------------------------------------------------------ ragged rows
+// A row that is no whole number of 16-byte vectors starts at another phase of the 16-byte grid
+// than the row before it, but at the same phase as the row 8 before it (16 before it for int8,
+// whose grid here is 8 bytes).  So warp w (lane group c of shorter rows) takes the rows
+// r = w (mod 8): it reads them as aligned vectors and keeps x in registers shifted to its one
+// phase, with the bytes of neighbouring rows in the first and last vector masked off.  x stays
+// 16-bit and meets the weights in mixed FMAs (exact products, fp32 sums), which halves its
+// registers.  HBM bounds it: eight bf16 16384 x 2731 matrices take 103 us (6959 GB/s) and four
+// f32 ones 111 us; one warp per row with byte loads took 465 and 292 us, and a tile whose
+// vectors are each put together from the two that hold them (two loads, eleven selects, four
+// shifts) 201 and 158 us: twice the instructions, on CTAs of eight warps.
+
+// The mask of a vector's bytes [lo, hi).
+__device__ __forceinline__ uint4 byte_mask(int lo, int hi) {
+  uint32_t m[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int a = min(max(lo - 4 * i, 0), 4), b = min(max(hi - 4 * i, 0), 4);
+    m[i] = a >= b ? 0u : (0xffffffffu >> (32 - 8 * (b - a))) << (8 * a);
+  }
+  return make_uint4(m[0], m[1], m[2], m[3]);
+}
+
+__device__ __forceinline__ uint4 and4(const uint4 &a, const uint4 &b) {
+  return make_uint4(a.x & b.x, a.y & b.y, a.z & b.z, a.w & b.w);
+}
+
+// A weight vector: on the 16-byte grid, or (int8) on the 8-byte grid.
+template <int DT>
+__device__ __forceinline__ uint4 lds_vec(uint32_t addr) {
+  if constexpr (DT == 3) {
+    uint4 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.z), "=r"(v.w) : "r"(addr + 8));
+    return v;
+  }
+  return lds128(addr);
+}
+
+// 32-bit words of x per weight vector: 16 f16 for an int8 vector, else as many bytes.
+template <int DT>
+struct PhaseX {
+  static constexpr int N = DT == 3 ? 8 : 4;
+};
+
+// f[i] += the products of one weight vector and its x.
+template <int DT>
+__device__ __forceinline__ void phase_dot(const uint4 &w, const uint32_t (&x)[PhaseX<DT>::N], float (&f)[4]) {
+  const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if constexpr (DT == 0) {
+      f[i] = fmaf(__uint_as_float(ws[i]), __uint_as_float(x[i]), f[i]);
+    } else if constexpr (DT == 1) {
+      f[i] = fma_b2(ws[i], x[i], f[i]);
+    } else if constexpr (DT == 2) {
+      f[i] = fma_h2(ws[i], x[i], f[i]);
+    } else {
+      const uint32_t u = ws[i] ^ 0x80808080u;
+      f[i] = fma_h2(i8x2_to_f16x2(u, 0x4140u), x[2 * i], f[i]);
+      f[i] = fma_h2(i8x2_to_f16x2(u, 0x4342u), x[2 * i + 1], f[i]);
+    }
+  }
+}
+
+// Bytes [0, n) of x to shared memory at xs + 16, zeros before and behind them; all consumers.
+template <int DT>
+__device__ __forceinline__ void stage_x(uint32_t xs, const uint8_t *x, uint32_t n, int ct) {
+  constexpr uint32_t kVec = (uint32_t)(GemvGeo<DT>::kXBytes / 16);
+  for (uint32_t i = ct; i < kVec; i += kConsumers) {
+    const int64_t o = 16 * (int64_t)i - 16;  // x bytes [o, o + 16)
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (o >= 0 && o + 16 <= n && (reinterpret_cast<uint64_t>(x) & 15) == 0) {
+      v = __ldg(reinterpret_cast<const uint4 *>(x + o));
+    } else if (o >= 0 && o < n) {
+      uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int b = 0; b < 16; ++b)
+        if (o + b < n) w[b / 4] |= (uint32_t)__ldg(x + o + b) << (8 * (b % 4));
+      v = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(xs + 16 * i), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+  }
+}
+
+// Where a tile's rows lie: row q starts at byte ((ph + q * rl) & 15) of at + q * sp.  Whole rows
+// came in one copy (sp the row's length, rl 0, at on the first row's start); a column segment's
+// rows one by one, at a pitch of V vectors and one more.
+struct PhaseTile {
+  uint32_t at, ph, sp, rl;
+  __device__ __forceinline__ PhaseTile(const MatDesc &md, uint32_t stage, uint32_t r) {
+    const bool whole = md.rs == md.rb;
+    ph = (uint32_t)(reinterpret_cast<uint64_t>(md.W) + (uint64_t)r * md.rs) & 15u;
+    at = stage + (whole ? ph : 0);
+    sp = whole ? md.rs : (md.V + 1) * 16;
+    rl = whole ? 0 : md.rs & 15u;
+    if (whole) ph = 0;
+  }
+  __device__ __forceinline__ uint32_t row(uint32_t q) const { return at + q * sp + ((ph + q * rl) & 15u); }
+};
+
+struct StageRing {
+  uint32_t stage0, full0, empty0;
+  volatile int *abort_flag;
+  int *status;
+};
+
+// One piece of a ragged matrix: NJ vectors per lane, G lanes per row (G < 32: NJ = 1).
+template <int DT, int NJ, int G>
+__device__ __forceinline__ void phase_rows(const MatDesc &md, const Piece &pc, const StageRing &R, uint32_t xs,
+                                           uint32_t &it, int warp, int lane, uint64_t *st) {
+  constexpr uint32_t kStages = GemvGeo<DT>::kStages;
+  constexpr uint32_t kGrid = DT == 3 ? 8 : 16;
+  constexpr int NX = PhaseX<DT>::N;
+  constexpr uint32_t RPW = 32 / G;                // rows a warp takes at once
+  constexpr uint32_t step = kConsumerWarps * RPW;  // a multiple of 8
+  constexpr int U = NJ == 1 ? 8 : NJ == 2 ? 4 : (NJ <= 4 ? 2 : 1);
+  static_assert(kConsumerWarps % 8 == 0, "one phase per lane group");
+  const uint32_t gl = lane & (G - 1);
+  const uint32_t cls = warp * RPW + lane / G;  // rows cls, cls + step, ... of the matrix
+  const uint32_t ph = (uint32_t)(reinterpret_cast<uint64_t>(md.W) + (uint64_t)cls * md.rs) & (kGrid - 1);
+  const uint32_t nv = (ph + md.rb + 15) / 16;  // vectors of a row of this phase, from its grid point on
+
+  uint32_t x[NJ][NX];
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    const uint32_t v = gl + j * G;
+    const bool ok = v < nv;
+#pragma unroll
+    for (int k = 0; k < NX / 4; ++k) {
+      // x bytes from 16 v - ph on (int8: twice that), staged 16 bytes further on
+      const uint4 t = lds_shifted(xs + 16 + (ok ? (NX / 4) * (16 * v - ph) + 16 * k : -16u));
+      x[j][4 * k] = ok ? t.x : 0, x[j][4 * k + 1] = ok ? t.y : 0;
+      x[j][4 * k + 2] = ok ? t.z : 0, x[j][4 * k + 3] = ok ? t.w : 0;
+    }
+  }
+  // masks of this lane's first vector (the row before ends in it) and last one
+  const uint32_t vl = gl + (NJ - 1) * G;
+  const uint4 m0 = byte_mask(gl == 0 ? (int)ph : 0, NJ > 1 ? 16 : (int)(ph + md.rb) - 16 * (int)gl);
+  const uint4 m1 = byte_mask(0, (int)(ph + md.rb) - 16 * (int)vl);
+
+  for (uint32_t r = pc.r0; r < pc.r1; r += md.rt) {
+    const uint32_t nr = min(md.rt, pc.r1 - r);
+    const uint32_t s = it % kStages;
+    bounded_wait(R.full0 + 8 * s, (it / kStages) & 1, R.abort_flag, R.status);
+    if (st) stamp_full(st, it, warp, lane);
+    const PhaseTile tile(md, R.stage0 + s * kStageBytes, r);
+    float *y = md.y + r;
+    const uint8_t *sr = md.s ? md.s + 2ull * r : nullptr;
+    // first row of this lane group in the tile; the loop runs for the whole warp
+    const uint32_t q0 = (cls - r) & (step - 1);
+    const uint32_t qw = RPW == 1 ? q0 : 0;
+    for (uint32_t b = qw; b < nr; b += U * step) {
+      const uint32_t qb = RPW == 1 ? b : b + q0;
+      uint32_t a[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t q = qb + u * step;
+        a[u] = tile.row(q < nr ? q : 0) & ~(kGrid - 1);
+      }
+      float t[U];
+      uint4 w[U][NJ];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          const uint32_t v = gl + j * G;
+          w[u][j] = lds_vec<DT>(a[u] + (j + 1 < NJ || v < nv ? v * 16 : 0));
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        float f[4] = {0.f, 0.f, 0.f, 0.f};
+        w[u][0] = and4(w[u][0], m0);
+        if (NJ > 1) w[u][NJ - 1] = and4(w[u][NJ - 1], m1);
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) phase_dot<DT>(w[u][j], x[j], f);
+        t[u] = (f[0] + f[1]) + (f[2] + f[3]);
+      }
+      if constexpr (G == 32) {
+        const float sum = transpose_reduce<U>(t, lane);
+        constexpr int L = Log2<U>::value;
+        const uint32_t q = qb + (uint32_t)(lane >> (5 - L)) * step;
+        if ((lane & ((32 >> L) - 1)) == 0 && q < nr) y[q] = sum * row_scale<DT>(sr, q);
+      } else {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) t[u] += __shfl_xor_sync(0xffffffffu, t[u], o);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const uint32_t q = qb + u * step;
+          if (gl == 0 && q < nr) y[q] = t[u] * row_scale<DT>(sr, q);
+        }
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(R.empty0 + 8 * s);
+    ++it;
+  }
+}
+
+// Lanes per row by the matrix, vectors per lane by the warp's own phase (its rows may have one
+// vector less than others, and the last one needs its mask).
+template <int DT>
+__device__ __forceinline__ void phase_dispatch(const MatDesc &md, const Piece &pc, const StageRing &R, uint32_t xs,
+                                               uint32_t &it, int warp, int lane, uint64_t *st) {
+  constexpr int kNJ = GemvGeo<DT>::kPhaseNJ;
+#define WT_PH(NJ) case NJ: phase_rows<DT, (NJ <= kNJ ? NJ : 1), 32>(md, pc, R, xs, it, warp, lane, st); break;
+  switch (md.G) {
+    case 1: phase_rows<DT, 1, 1>(md, pc, R, xs, it, warp, lane, st); return;
+    case 2: phase_rows<DT, 1, 2>(md, pc, R, xs, it, warp, lane, st); return;
+    case 4: phase_rows<DT, 1, 4>(md, pc, R, xs, it, warp, lane, st); return;
+    case 8: phase_rows<DT, 1, 8>(md, pc, R, xs, it, warp, lane, st); return;
+    case 16: phase_rows<DT, 1, 16>(md, pc, R, xs, it, warp, lane, st); return;
+  }
+  const uint32_t ph = (uint32_t)(reinterpret_cast<uint64_t>(md.W) + (uint64_t)warp * md.rs) & (DT == 3 ? 7u : 15u);
+  switch ((ph + md.rb + 511) / 512) {
+    WT_PH(1) WT_PH(2) WT_PH(3) WT_PH(4) WT_PH(5) WT_PH(6) WT_PH(7) WT_PH(8)
+    WT_PH(9) WT_PH(10) WT_PH(11) WT_PH(12) WT_PH(13) WT_PH(14) WT_PH(15) WT_PH(16)
+  }
+#undef WT_PH
+}
+
+// The copies of rows [r, r + nr) of a ragged matrix to their stage, by the whole producer warp:
+// whole rows are one range, the rows of a column segment one range each (lane q takes rows
+// q, q + 32, ...: one thread's address arithmetic alone held the copies to 3.5 TB/s).  A range
+// arrives with its byte src at dst + (src & 15): a bulk copy brings the whole 16-byte vectors
+// that hold it and lie inside the matrix; bytes of the matrix's first or last vector that no
+// such vector holds go one by one.
+__device__ __forceinline__ void ragged_tile(const MatDesc &md, uint32_t r, uint32_t nr, uint32_t dst, uint32_t bar,
+                                            uint64_t pol, int lane) {
+  const uint64_t w0 = reinterpret_cast<uint64_t>(md.W), wend = w0 + (uint64_t)(md.M - 1) * md.rs + md.rb;
+  const uint64_t wlo = (w0 + 15) & ~15ull, whi = wend & ~15ull;
+  const bool whole = md.rs == md.rb;
+  const uint32_t ranges = whole ? 1 : nr, len = whole ? nr * md.rb : md.rb;
+  for (uint32_t q0 = 0; q0 < ranges; q0 += 32) {
+    const uint32_t q = q0 + lane;
+    const uint64_t src = w0 + (uint64_t)(r + q) * md.rs, a = src & ~15ull, end = src + len;
+    uint64_t lo = max(a, wlo), hi = min((end + 15) & ~(uint64_t)15, whi);
+    const uint32_t d = dst + q * (md.V + 1) * 16;
+    uint32_t bulk = 0;
+    if (q < ranges) {
+      if (hi > lo) bulk = (uint32_t)(hi - lo);
+      else lo = hi = end;
+      if (src < lo || hi < end) {
+        for (uint64_t p = src; p < lo; ++p) sts8(d + (uint32_t)(p - a), *reinterpret_cast<const uint8_t *>(p));
+        for (uint64_t p = max(hi, src); p < end; ++p)
+          sts8(d + (uint32_t)(p - a), *reinterpret_cast<const uint8_t *>(p));
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+    }
+    const uint32_t tx = __reduce_add_sync(0xffffffffu, bulk);
+    // the stage's one arrival comes with its last bytes announced, after every lane's stores
+    if (lane == 0) {
+      if (q0 + 32 < ranges) mbar_expect_only(bar, tx);
+      else mbar_expect_tx(bar, tx);
+    }
+    __syncwarp();
+    if (bulk) bulk_g2s(d + (uint32_t)(lo - a), reinterpret_cast<const void *>(lo), bulk, bar, pol);
+  }
+}
+
 // ST: the stamping instantiation, which also writes the per-CTA times of StampField to
-// stamps[blockIdx.x * kStampFields ...]; otherwise identical.
-template <int DT, bool ST>
+// stamps[blockIdx.x * kStampFields ...]; otherwise identical.  RAG: also takes matrices with
+// ragged rows (kModePhaseRows), and stamps if stamps is non-null.
+template <int DT, bool ST, bool RAG>
 __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
     gemv_tma_kernel(const MatDesc *__restrict__ mats, const Piece *__restrict__ pieces,
                     const uint32_t *__restrict__ begin, int *status, int stall, uint64_t *stamps) {
   constexpr int NP = Pairs<DT>::N;
   constexpr int kStages = GemvGeo<DT>::kStages;
-  uint64_t *const st = ST ? stamps + (uint64_t)blockIdx.x * kStampFields : nullptr;
-  if (ST && threadIdx.x == 0) {
+  const bool stamping = ST && (!RAG || stamps != nullptr);
+  uint64_t *const st = stamping ? stamps + (uint64_t)blockIdx.x * kStampFields : nullptr;
+  if (stamping && threadIdx.x == 0) {
     st[kStEntry] = globaltimer_ns();
     st[kStFirstCopy] = st[kStFirstFull] = st[kStLastFull] = 0;
   }
@@ -488,7 +776,7 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
     mbar_fence_init();
   }
   __syncthreads();
-  if (ST && threadIdx.x == 0) st[kStPrologue] = globaltimer_ns();
+  if (stamping && threadIdx.x == 0) st[kStPrologue] = globaltimer_ns();
   // Up to here only the plan tables (written once, by the upload before the first launch) and
   // shared memory are touched, so under a programmatic launch this prologue may overlap the
   // previous kernel of the stream; W, x, y and the scales are read or written only after that
@@ -496,11 +784,12 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
   // only as this grid leaves it.  Without a programmatic launch both are no-ops.
   griddep_wait();
   griddep_launch();
-  if (ST && threadIdx.x == 0) st[kStOperands] = globaltimer_ns();
+  if (stamping && threadIdx.x == 0) st[kStOperands] = globaltimer_ns();
 
   if (warp == kConsumerWarps) {
-    // ---------------- producer: one thread issues every bulk copy of the CTA
-    if (lane == 0 && !stall) {
+    // ---------------- producer: one thread issues every bulk copy of the CTA; the ragged
+    // instantiation keeps the whole warp, whose lanes share out a column segment's rows
+    if ((RAG || lane == 0) && !stall) {
       const uint64_t pol = l2_evict_first_policy();
       uint32_t it = 0;
       bool live = true;
@@ -514,21 +803,29 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
           const uint32_t s = it % kStages;
           if (it >= kStages && !bounded_wait(empty0 + 8 * s, ((it / kStages) - 1) & 1, abort_flag, status)) {
             live = false;
-            break;
+            if (!RAG) break;
+          }
+          if (RAG) {
+            live = __all_sync(0xffffffffu, live);
+            if (!live) break;
           }
           const uint32_t dst = stage0 + s * kStageBytes;
           const uint32_t bar = full0 + 8 * s;
-          if (ST && it == 0) st[kStFirstCopy] = globaltimer_ns();
-          mbar_expect_tx(bar, nr * vb);
-          if (md.rs == md.V) {
-            bulk_g2s(dst, md.W + (uint64_t)r * rowb, nr * vb, bar, pol);  // contiguous rows: one copy
-          } else {
-            for (uint32_t q = 0; q < nr; ++q) bulk_g2s(dst + q * vb, md.W + (uint64_t)(r + q) * rowb, vb, bar, pol);
+          if (stamping && it == 0 && (!RAG || lane == 0)) st[kStFirstCopy] = globaltimer_ns();
+          if (RAG && md.rb) {
+            ragged_tile(md, r, nr, dst, bar, pol, lane);
+          } else if (!RAG || lane == 0) {
+            mbar_expect_tx(bar, nr * vb);
+            if (md.rs == md.V) {
+              bulk_g2s(dst, md.W + (uint64_t)r * rowb, nr * vb, bar, pol);  // contiguous rows: one copy
+            } else {
+              for (uint32_t q = 0; q < nr; ++q) bulk_g2s(dst + q * vb, md.W + (uint64_t)(r + q) * rowb, vb, bar, pol);
+            }
           }
           ++it;
         }
       }
-      if (!live || *abort_flag) {
+      if ((!RAG || lane == 0) && (!live || *abort_flag)) {
         // drain: the copies of the last (up to kStages) issued stages may still be in flight
         const uint32_t first = it > (uint32_t)kStages ? it - kStages : 0;
         for (uint32_t j = first; j < it; ++j) {
@@ -550,6 +847,14 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
       const Piece pc = pieces[pi];
       const MatDesc md = mats[pc.mat];
       const uint32_t V = md.V;
+      if (RAG && md.mode == kModePhaseRows) {
+        const uint32_t xs = smem_u32(smem + GemvGeo<DT>::kXOff);
+        named_bar(1, kConsumers);  // every warp has taken the last matrix's x into registers
+        stage_x<DT>(xs, md.x, DT == 3 ? 2 * md.rb : md.rb, ct);
+        named_bar(1, kConsumers);
+        phase_dispatch<DT>(md, pc, {stage0, full0, empty0, abort_flag, status}, xs, it, warp, lane, st);
+        continue;
+      }
       if (md.mode == kModeWarpRows) {
         const uint32_t G = md.G;
         const uint32_t gl = lane & (G - 1);
@@ -565,7 +870,7 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
           const uint32_t nr = min(md.rt, pc.r1 - r);
           const uint32_t s = it % kStages;
           bounded_wait(full0 + 8 * s, (it / kStages) & 1, abort_flag, status);
-          if (ST) stamp_full(st, it, warp, lane);
+          if (stamping) stamp_full(st, it, warp, lane);
           const uint32_t tile = stage0 + s * kStageBytes;
           float *y = md.y + r;
           const uint8_t *sr = md.s ? md.s + 2ull * r : nullptr;  // f16 row scales (int8 weights)
@@ -606,7 +911,7 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
           const uint32_t nr = min(md.rt, pc.r1 - r);
           const uint32_t s = it % kStages;
           bounded_wait(full0 + 8 * s, (it / kStages) & 1, abort_flag, status);
-          if (ST) stamp_full(st, it, warp, lane);
+          if (stamping) stamp_full(st, it, warp, lane);
           const uint32_t tile = stage0 + s * kStageBytes;
           float *rb = red + par * (kConsumerWarps * kRedRows) + gn * kConsumerWarps;
           if (!block_rows_dispatch<DT>(nj, nr, tile, V, ct, warp, lane, xp, rb) && ct == 0)
@@ -628,7 +933,7 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
     }
   }
   __syncthreads();
-  if (ST && threadIdx.x == 0) {
+  if (stamping && threadIdx.x == 0) {
     st[kStExit] = globaltimer_ns();
     st[kStSm] = sm_id();
   }
@@ -824,10 +1129,12 @@ int gemv_ctas_per_sm(int dtype) { return dtype == 3 ? GemvGeo<3>::kCtasPerSm : G
 
 template <int DT>
 static cudaError_t gemv_attr() {
-  const cudaError_t e =
-      cudaFuncSetAttribute(gemv_tma_kernel<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemvGeo<DT>::kSmem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(gemv_tma_kernel<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemvGeo<DT>::kSmem);
+  constexpr cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(gemv_tma_kernel<DT, false, false>, a, (int)GemvGeo<DT>::kSmem)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(gemv_tma_kernel<DT, true, false>, a, (int)GemvGeo<DT>::kSmem)) != cudaSuccess)
+    return e;
+  return cudaFuncSetAttribute(gemv_tma_kernel<DT, true, true>, a, (int)GemvGeo<DT>::kSmemRagged);
 }
 
 cudaError_t gemv_prepare() {
@@ -845,17 +1152,16 @@ static cudaError_t gemv_launch(const GemvLaunch &L, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)L.grid);
   cfg.blockDim = dim3(kGemvThreads);
-  cfg.dynamicSmemBytes = GemvGeo<DT>::kSmem;
+  cfg.dynamicSmemBytes = L.ragged ? GemvGeo<DT>::kSmemRagged : GemvGeo<DT>::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = L.pdl ? 1 : 0;
-  if (L.stamps)
-    return cudaLaunchKernelEx(&cfg, gemv_tma_kernel<DT, true>, L.mats, L.pieces, L.begin, L.status, L.stall, L.stamps);
-  return cudaLaunchKernelEx(&cfg, gemv_tma_kernel<DT, false>, L.mats, L.pieces, L.begin, L.status, L.stall,
-                            (uint64_t *)nullptr);
+  const auto k = L.ragged ? gemv_tma_kernel<DT, true, true>
+                          : L.stamps ? gemv_tma_kernel<DT, true, false> : gemv_tma_kernel<DT, false, false>;
+  return cudaLaunchKernelEx(&cfg, k, L.mats, L.pieces, L.begin, L.status, L.stall, L.stamps);
 }
 
 cudaError_t launch_gemv(const GemvLaunch &L, cudaStream_t s) {

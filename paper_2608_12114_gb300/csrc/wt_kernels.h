@@ -37,6 +37,7 @@ enum GemvMode : uint16_t {
   kModeBlockRows = 1,  // 256 < vectors <= kStageBytes/16: whole CTA per row, full-row tiles
   kModeLongRows = 2,   // rows longer than one stage: split into column segments before any TMA launch
   kModeCols = 3,       // multi-column kernel (G = T columns): 16-row tiles x vc-vector chunks
+  kModePhaseRows = 4,  // ragged rows (one-column kernel): G lanes per row, one 16-byte phase per warp
 };
 
 // Multi-column kernel: at most kColVecMax 16-byte vectors of a row per stage, and a chunk
@@ -60,7 +61,8 @@ struct alignas(16) MatDesc {
   uint32_t rs;    // row pitch in 16-byte vectors: V, or the full row of a column segment
                   // (segments are split-K only); s == nullptr then means "no scale yet"
   uint32_t cols;  // map endpoint with T activation columns: T (X [T, K], Y [T, M]); else 0
-  uint32_t pad;
+  uint32_t rb;    // ragged rows (one-column kernel: rows, W or x off the 16-byte grid): bytes of a
+                  // row or row segment, V = ceil(rb / 16), and rs is the row pitch in bytes; else 0
 };
 static_assert(sizeof(MatDesc) == 64, "MatDesc is one 64-byte record");
 
@@ -71,6 +73,9 @@ static_assert(sizeof(MatDesc) == 64, "MatDesc is one 64-byte record");
 // segments of each row in segment order and applies the row scale.  Segment boundaries
 // depend only on the matrix, so a row's result never depends on how rows and segments were
 // spread over CTAs.
+// Ragged rows: at most this many vectors, counted from the grid point at or before the row's
+// start (the x registers of a lane: 64, or 48 for int8, which runs two CTAs per SM).
+constexpr uint32_t kPhaseVec(int dtype) { return dtype == 3 ? 192 : 512; }
 constexpr uint32_t kSegVec = 2048;  // bf16 / f16 / f32: 32 KB per segment row
 constexpr uint32_t seg_vectors(int dtype) { return dtype == 3 ? kSegVec / 4 : kSegVec; }  // int8: 8 KB
 
@@ -105,6 +110,7 @@ struct GemvLaunch {
   int stall = 0;  // failure test (host fault site "stall"): the producer issues no copy, so
                   // every consumer wait runs out, reports WT_ETIMEDOUT and the CTA exits
   int nt = 0;     // multi-column kernel: 8-column MMA tiles of every matrix (T <= 8 nt)
+  int ragged = 0;  // one-column kernel: some matrix has ragged rows (MatDesc.rb > 0)
   int pdl = 0;    // one-column kernel: launch with programmatic stream serialization (the
                   // launch and prologue may overlap the previous kernel of the stream)
   uint64_t *stamps = nullptr;  // one-column kernel: non-null runs the stamping instantiation,
@@ -168,9 +174,9 @@ struct UmmaLaunch {
 cudaError_t gemm_cols_umma_prepare();
 cudaError_t launch_gemm_cols_umma(const UmmaLaunch &L, cudaStream_t s);
 
-// Fallback for operands the tiled kernels cannot take (unaligned W/x, rows whose byte length
-// is not a multiple of 16, or multi-column W read in place from a mapping): one warp per
-// row, scalar loads.  cols = 0 or 1: y = W x; cols = T > 1: Y [T, M] from X [T, K].
+// Fallback for operands the tiled kernels cannot take (W read in place from host memory, or
+// several columns, with unaligned W/x or rows whose byte length is not a multiple of 16; rows
+// of 2^31 bytes and more): one warp per row, scalar loads.  cols = 0 or 1: y = W x; cols = T > 1: Y [T, M] from X [T, K].
 cudaError_t launch_gemv_generic(int dtype, const uint8_t *W, const uint8_t *x, float *y,
                                 uint64_t M, uint64_t K, const uint8_t *scale, uint32_t cols,
                                 cudaStream_t s);

@@ -1,0 +1,84 @@
+"""Rows off the 16-byte grid: K of any length, W and x at any byte, in every element type, on
+the tiled kernels; against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2608_12114_gb300 import build, synth, wt
+
+pytestmark = pytest.mark.gpu
+F32, BF16, F16, I8 = wt.WT_F32, wt.WT_BF16, wt.WT_F16, wt.WT_I8
+ES = {F32: 4, BF16: 2, F16: 2, I8: 1}
+
+# (M, bytes of a row, bytes past a 16-byte boundary of W and of x): matrices and rows smaller
+# than a vector; rows of one phase that fill 16 and 32 lanes and of another that need one more;
+# every row count of a stage; 8 rows and fewer; the longest unsegmented row (504 vectors; int8:
+# 184) and the first segmented one; a partial last segment; aligned rows at unaligned addresses
+SHAPES = [(1, 4, 0, 0), (5, 4, 4, 4), (3, 20, 0, 0), (1000, 12, 8, 0), (33, 232, 4, 8), (33, 244, 0, 4), (40, 256, 4, 0),
+          (70, 496, 12, 0), (70, 508, 4, 0), (90, 516, 4, 0), (65, 1012, 0, 0), (65, 1028, 8, 0), (300, 2940, 0, 0),
+          (300, 2948, 4, 4), (41, 4084, 0, 0), (41, 4100, 0, 0), (129, 5460, 0, 0), (7, 6132, 0, 0), (50, 8060, 4, 0),
+          (50, 8064, 4, 0), (50, 8068, 0, 0), (37, 8192, 0, 8), (37, 8196, 4, 0), (19, 12300, 0, 0), (9, 32636, 0, 0),
+          (5, 65540, 4, 0), (3, 131076, 0, 12)]
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch
+    assert torch.cuda.is_available()
+    build.build()
+    wt.lib()
+    return torch
+
+
+def weights(rng, dtype, n):
+    if dtype == I8:
+        return rng.integers(-128, 128, n).astype(np.int8).view(np.uint8)
+    v = rng.standard_normal(n).astype(np.float32)
+    return synth.f32_to_bf16_bits(v).view(np.uint8) if dtype == BF16 else \
+        v.astype(np.float16 if dtype == F16 else np.float32).view(np.uint8)
+
+
+def at(torch, data, off):
+    """`data` on the device, `off` bytes past a 16-byte boundary, among bytes of 0xff (NaN in
+    every float type: a value read past an operand shows)."""
+    buf = torch.full((data.size + 64,), 255, dtype=torch.uint8, device="cuda")
+    buf[16 + off:16 + off + data.size] = torch.from_numpy(np.ascontiguousarray(data)).cuda()
+    return buf, buf.data_ptr() + 16 + off
+
+
+def bound(K):
+    """|fp32 sum of K products - exact| <= K u sum|w x|, and the row scale's rounding."""
+    return (K + 4) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("dtype", [F32, BF16, F16, I8])
+@pytest.mark.parametrize("odd", [0, 1])
+def test_ragged_rows_against_oracle(torch, dtype, odd):
+    """Every shape in one pass with an aligned matrix, then alone (the same bits).  odd: one
+    element fewer per row, so that rows of 1- and 2-byte types start at every phase."""
+    rng = np.random.default_rng(100 * dtype + odd)
+    es = ES[dtype]
+    shapes = [(M, max(1, kb // es - odd), wo - wo % es, xo - xo % (2 if dtype == I8 else es))
+              for M, kb, wo, xo in SHAPES] + [(64, 1024, 0, 0)]
+    cs = []
+    for M, K, wo, xo in shapes:
+        W, x = weights(rng, dtype, M * K), weights(rng, F16 if dtype == I8 else dtype, K)
+        s = rng.uniform(0.001, 0.02, M).astype(np.float16).view(np.uint8) if dtype == I8 else None
+        wb, wp = at(torch, W, wo)
+        xb, xp = at(torch, x, xo)
+        sb, sp = at(torch, s, 0) if s is not None else (None, 0)
+        y = torch.full((M,), float("nan"), dtype=torch.float32, device="cuda")
+        ref = oracle.gemv_q8(W, s, M, K, x) if dtype == I8 else oracle.gemv(W, dtype, M, K, x)
+        cs.append((M, K, wp, xp, sp, y, ref, (wb, xb, sb)))
+    with wt.Handle([]) as h:
+        h.pass_([wt.gemv_desc(wp, dtype, M, K, xp, y.data_ptr(), scale=sp) for M, K, wp, xp, sp, y, _, _ in cs], 0)
+        torch.cuda.synchronize()
+        assert h.device_status() == 0
+        for M, K, wp, xp, sp, y, (yhat, a), _ in cs:
+            err = oracle.gemv_error(y.cpu().numpy(), yhat, a)
+            assert err <= bound(K), (dtype, M, K, err)
+        for M, K, wp, xp, sp, y, _, _ in cs:
+            y2 = torch.full_like(y, float("nan"))
+            h.pass_([wt.gemv_desc(wp, dtype, M, K, xp, y2.data_ptr(), scale=sp)], 0)
+            assert torch.equal(y2, y), (dtype, M, K)
+        assert h.device_status() == 0
