@@ -23,6 +23,16 @@
 // the end of a super block the warps' partial tiles meet in shared memory and are summed in
 // warp order (deterministic; rows never depend on the partition across CTAs).
 //
+// Ragged operands (RAG: rows of W or X that are no whole number of 16-byte vectors, or W or X
+// off a 16-byte boundary): no tensor map can describe such rows, so each lane of the producer
+// warp brings one row's share of a chunk by a 1-D copy, and every weight and X vector is put
+// together from the two 16-byte vectors that hold it.  Each vector's MMAs start from zero and
+// meet the fp32 sums in ordinary additions: the tensor cores' own accumulation truncates, and
+// these calls had fp32 FMAs before (error against 64 bits, rows of 2731: 9.6e-8 bf16, 9.8e-8 int8,
+// 1.1e-7 f16 at T = 16, against 8.5e-8, 8.7e-8 and 1.7e-7).  Eight bf16 16384 x 2731 matrices at
+// T = 8 take 250 us (2884 GB/s; bound by the instructions of putting vectors together), and took
+// 1940 us with byte loads, one warp per row and the row read again for every column.
+//
 // Why warp-level MMAs and not tcgen05: the A operand is decoded from int8 in registers and
 // goes to the MMA from there; tcgen05 takes A only from shared or tensor memory, which would
 // add a store and a fence per decoded tile, and for T <= 16 the tensor rate is far from the
@@ -42,6 +52,10 @@ constexpr int kColConsumers = kColWarps * 32;
 constexpr int kColThreads = kColConsumers + 32;  // + one producer warp
 constexpr int kColRows = kColTileRows;           // rows of one stage (one MMA tile)
 constexpr int kColGroups = (kColVecMax / 4 + kColWarps - 1) / kColWarps;  // 4-vector groups per warp
+// a ragged row's chunk sits at its 16-byte phase: the pitch is this many vectors past the chunk
+// (a multiple of 8: still 64 bytes past a multiple of 128)
+constexpr uint32_t kColRagPad = 8;
+static_assert(kColRagPad == kColVecMax - kColVecMaxRagged, "a padded chunk fills a stage row");
 constexpr uint32_t kColStageBytes = kColRows * kColVecMax * 16;
 static_assert(kColVecMax % 8 == 4, "row pitch 64 bytes past a multiple of 128");
 static_assert(kColStageBytes % 128 == 0, "stages stay 128-byte aligned for the tensor copies");
@@ -50,7 +64,7 @@ static_assert(kColStageBytes % 128 == 0, "stages stay 128-byte aligned for the t
 // CTAs per SM with half the ring each (the same bytes in flight per SM, twice the warps; the
 // int8 path is latency-bound on its decode).  The cross-warp partials of one 16-row tile take
 // 16 x 8 NT floats per warp, in two alternating halves.
-template <int DT, int NT>
+template <int DT, int NT, bool RAG = false>
 struct ColGeo {
   static constexpr int kCtasPerSm = DT == 3 ? 2 : 1;
   static constexpr int kStages = kCtasPerSm == 2 ? 3 : 6;
@@ -60,7 +74,7 @@ struct ColGeo {
   static constexpr int kBlocks = DT == 3 && NT == 2 ? 2 : 4;
   // accumulator sets per tile (even / odd k16 steps: shorter MMA chains); int8 with 16
   // columns keeps one, its two column tiles already give two independent chains per A
-  static constexpr int kAcc = DT == 3 && NT == 2 ? 1 : 2;
+  static constexpr int kAcc = RAG || (DT == 3 && NT == 2) ? 1 : 2;
   static constexpr int kSuper = kColRows * kBlocks;
   static constexpr uint32_t kRedStride = 128 * NT;  // floats per (tile, warp)
   static constexpr size_t kRedFloats = (size_t)kBlocks * kColWarps * kRedStride;  // one half
@@ -120,6 +134,42 @@ __device__ __forceinline__ void load_xvec(const uint8_t *X, uint64_t vec, bool o
   }
 }
 
+// Bytes [o, o + 16) of X, which has `total` bytes at any address, those from `end` on zero.
+__device__ __forceinline__ uint4 ldg_shifted(const uint8_t *X, uint64_t o, uint64_t end, uint64_t total) {
+  if (o >= end) return make_uint4(0, 0, 0, 0);
+  const uint64_t a = reinterpret_cast<uint64_t>(X) + o, x0 = reinterpret_cast<uint64_t>(X);
+  const uint32_t ph = (uint32_t)a & 15u;
+  uint4 r;
+  if (a - ph >= x0 && a - ph + (ph ? 32 : 16) <= x0 + total) {
+    const uint4 *p = reinterpret_cast<const uint4 *>(a - ph);
+    const uint4 lo = __ldg(p), hi = ph ? __ldg(p + 1) : lo;
+    r = shift_bytes(lo, hi, ph);
+  } else {  // the first or last vector of X
+    uint64_t lo = 0, hi = 0;
+#pragma unroll 1
+    for (int i = 15; i >= 0; --i) {
+      hi = (hi << 8) | (lo >> 56);
+      lo = (lo << 8) | (o + i < total ? __ldg(X + o + i) : 0);
+    }
+    r = make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+  }
+  return o + 16 <= end ? r : and4(r, byte_mask(0, (int)(end - o)));
+}
+
+// load_xvec for ragged operands: weight vector v (of the whole row) of column `col`.
+template <int DT>
+__device__ __forceinline__ void load_xvec_ragged(const MatDesc &md, uint32_t col, uint32_t v, bool ok,
+                                                 uint32_t (&xr)[ColX<DT>::W]) {
+  constexpr uint32_t kXB = DT == 3 ? 32 : 16;  // X bytes of a weight vector
+  const uint64_t xp = (uint64_t)md.rb * (kXB / 16);
+  const uint64_t o = col * xp + (uint64_t)v * kXB, end = (col + 1) * xp, total = md.G * xp;
+#pragma unroll
+  for (uint32_t k = 0; k < kXB / 16; ++k) {
+    const uint4 a = ldg_shifted(md.x, o + 16 * k, ok ? end : 0, total);
+    xr[4 * k] = a.x, xr[4 * k + 1] = a.y, xr[4 * k + 2] = a.z, xr[4 * k + 3] = a.w;
+  }
+}
+
 // 2-D tensor copy of one box into this CTA's shared memory, completion counted on `bar`.
 // x (in 8-byte elements) is always a multiple of 2: 16-byte aligned.
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int32_t x, int32_t y, uint32_t bar,
@@ -135,19 +185,37 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int3
 // Thread (g, t) takes vector (q * warps + warp) * 4 + t of group q.
 // The box holds vc vectors per row at pitch vc * 16; rows and vectors past the matrix are
 // zeros, so only whole groups past vc are skipped.
-template <int DT, int NT, int H>
+// RAG: row g starts ph0 bytes past its pitch's start, row g + 8 ph1 bytes; of vector v only the
+// row's own bytes count (left: those from the chunk's start on; an int8 neighbour meets a zero
+// of X and is a finite number, so only the 2-byte types mask it).
+template <int DT, int NT, int H, bool RAG>
 __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, int warp, uint32_t g, uint32_t t,
-                                           const uint32_t (&xr)[kColGroups][NT][ColX<DT>::W], float (&acc)[H][NT][4]) {
-  const uint32_t pitch = vc * 16;
+                                           const uint32_t (&xr)[kColGroups][NT][ColX<DT>::W], float (&acc)[H][NT][4],
+                                           uint32_t ph0, uint32_t ph1, uint32_t left) {
+  const uint32_t pitch = RAG ? (vc + kColRagPad) * 16 : vc * 16;
 #pragma unroll
   for (int q = 0; q < kColGroups; ++q) {
     const uint32_t v0 = (uint32_t)(q * kColWarps + warp) * 4;
     if (v0 >= vc) continue;  // warp-uniform: the box ends before this group
     const uint32_t v = v0 + t;
-    const uint4 w0 = lds128(tile + g * pitch + v * 16);
-    const uint4 w1 = lds128(tile + (g + 8) * pitch + v * 16);
+    uint4 w0, w1;
+    if constexpr (RAG) {
+      w0 = lds_shifted(tile + g * pitch + ph0 + v * 16);
+      w1 = lds_shifted(tile + (g + 8) * pitch + ph1 + v * 16);
+      if (DT != 3 && left < vc * 16) {  // uniform: the row's last chunk
+        const uint4 m = byte_mask(0, (int)left - (int)(v * 16));
+        w0 = and4(w0, m);
+        w1 = and4(w1, m);
+      }
+    } else {
+      w0 = lds128(tile + g * pitch + v * 16);
+      w1 = lds128(tile + (g + 8) * pitch + v * 16);
+    }
     const uint32_t ra[4] = {w0.x, w0.y, w0.z, w0.w};
     const uint32_t rb[4] = {w1.x, w1.y, w1.z, w1.w};
+    float part[NT][4];  // RAG: this vector's products
+#pragma unroll
+    for (int n = 0; n < NT; ++n) part[n][0] = part[n][1] = part[n][2] = part[n][3] = 0.f;
     if constexpr (DT == 3) {
       // word j = weights k 4j..4j+3 of the vector; its activations are x words 2j, 2j+1
 #pragma unroll
@@ -157,7 +225,7 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, int warp,
         const uint32_t a1 = i8x2_to_f16x2(u1, 0x4140u), a3 = i8x2_to_f16x2(u1, 0x4342u);
 #pragma unroll
         for (int n = 0; n < NT; ++n)
-          mma16816<2>(acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
+          mma16816<2>(RAG ? part[n] : acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
       }
     } else {
       // words 2s, 2s+1 = elements 4s..4s+3 of the vector
@@ -165,9 +233,15 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, int warp,
       for (int s = 0; s < 2; ++s) {
 #pragma unroll
         for (int n = 0; n < NT; ++n)
-          mma16816<DT>(acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
+          mma16816<DT>(RAG ? part[n] : acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
                        xr[q][n][2 * s + 1]);
       }
+    }
+    if constexpr (RAG) {
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[0][n][i] += part[n][i];
     }
   }
 }
@@ -179,19 +253,19 @@ struct Ring {
 };
 
 // Consumer side of one piece (rows [r0, r1) of one matrix), NT = 8-column MMA tiles.
-template <int DT, int NT>
+template <int DT, int NT, bool RAG>
 __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, const Ring &R, float *red_base,
                                            uint32_t &it, uint32_t &par, int warp, int lane) {
   const uint32_t V = md.V, vc = md.vc, T = md.G;
   const uint32_t nchunk = (V + vc - 1) / vc;
   const uint32_t g = lane >> 2, t = lane & 3;
   const int ct = threadIdx.x;
-  constexpr int kColBlocks = ColGeo<DT, NT>::kBlocks;
-  constexpr int kColSuper = ColGeo<DT, NT>::kSuper;
+  constexpr int kColBlocks = ColGeo<DT, NT, RAG>::kBlocks;
+  constexpr int kColSuper = ColGeo<DT, NT, RAG>::kSuper;
   for (uint32_t sb = pc.r0; sb < pc.r1; sb += kColSuper) {
     const uint32_t rows = min((uint32_t)kColSuper, pc.r1 - sb);
     const uint32_t nrb = (rows + kColRows - 1) / kColRows;
-    constexpr int H = ColGeo<DT, NT>::kAcc;
+    constexpr int H = ColGeo<DT, NT, RAG>::kAcc;
     float acc[kColBlocks][H][NT][4];
 #pragma unroll
     for (int b = 0; b < kColBlocks; ++b)
@@ -208,15 +282,18 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
           const uint32_t col = g + 8 * n;
-          load_xvec<DT>(md.x, (uint64_t)col * V + (uint64_t)c * vc + v, v < nv && col < T, xr[q][n]);
+          if constexpr (RAG) load_xvec_ragged<DT>(md, col, c * vc + v, v < nv && col < T, xr[q][n]);
+          else load_xvec<DT>(md.x, (uint64_t)col * V + (uint64_t)c * vc + v, v < nv && col < T, xr[q][n]);
         }
       }
 #pragma unroll
       for (int b = 0; b < kColBlocks; ++b) {
         if ((uint32_t)b < nrb) {
-          const uint32_t s = it % ColGeo<DT, NT>::kStages;
-          bounded_wait(R.full0 + 8 * s, (it / ColGeo<DT, NT>::kStages) & 1, R.abort_flag, R.status);
-          cols_stage<DT, NT, H>(R.stage0 + s * kColStageBytes, vc, warp, g, t, xr, acc[b]);
+          const uint32_t s = it % ColGeo<DT, NT, RAG>::kStages;
+          bounded_wait(R.full0 + 8 * s, (it / ColGeo<DT, NT, RAG>::kStages) & 1, R.abort_flag, R.status);
+          const uint64_t row = reinterpret_cast<uint64_t>(md.W) + (uint64_t)(sb + b * kColRows + g) * md.rb;
+          cols_stage<DT, NT, H, RAG>(R.stage0 + s * kColStageBytes, vc, warp, g, t, xr, acc[b], (uint32_t)row & 15u,
+                                     (uint32_t)(row + 8ull * md.rb) & 15u, md.rb - c * vc * 16);
           __syncwarp();
           if (lane == 0) mbar_arrive(R.empty0 + 8 * s);
           ++it;
@@ -226,8 +303,8 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
     // warp partials -> red[b][warp][col][row]; C fragment: (g, 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1).
     // Two halves alternate, so one barrier per super block suffices: a half is rewritten
     // only after every thread has passed the next super block's barrier.
-    constexpr uint32_t kStride = ColGeo<DT, NT>::kRedStride;
-    float *red = red_base + par * ColGeo<DT, NT>::kRedFloats;
+    constexpr uint32_t kStride = ColGeo<DT, NT, RAG>::kRedStride;
+    float *red = red_base + par * ColGeo<DT, NT, RAG>::kRedFloats;
     par ^= 1;
 #pragma unroll
     for (int b = 0; b < kColBlocks; ++b) {
@@ -257,11 +334,11 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
   }
 }
 
-template <int DT, int NT>
-__global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT>::kCtasPerSm))
+template <int DT, int NT, bool RAG>
+__global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG>::kCtasPerSm))
     gemm_cols_kernel(const MatDesc *__restrict__ mats, const Piece *__restrict__ pieces,
                      const uint32_t *__restrict__ begin, int *status, const uint8_t *__restrict__ maps) {
-  using Geo = ColGeo<DT, NT>;
+  using Geo = ColGeo<DT, NT, RAG>;
   constexpr int kColStages = Geo::kStages;
   extern __shared__ __align__(128) uint8_t smem[];
   Ring R;
@@ -287,8 +364,9 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT>::kCtasPerSm))
   __syncthreads();
 
   if (warp == kColWarps) {
-    // ---------------- producer: one thread issues every bulk copy of the CTA
-    if (lane == 0) {
+    // ---------------- producer: one thread issues every tensor copy of the CTA (ragged rows:
+    // sixteen threads a row's copy each)
+    if (RAG || lane == 0) {
       const uint64_t pol = l2_evict_first_policy();
       uint32_t it = 0;
       bool live = true;
@@ -304,11 +382,19 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT>::kCtasPerSm))
             for (uint32_t b = 0; b < nrb; ++b) {
               const uint32_t s = it % kColStages;
               if (it >= kColStages &&
-                  !bounded_wait(R.empty0 + 8 * s, ((it / kColStages) - 1) & 1, R.abort_flag, status)) {
+                  !bounded_wait(R.empty0 + 8 * s, ((it / kColStages) - 1) & 1, R.abort_flag, status))
                 live = false;
-                break;
-              }
+              if (RAG) live = __all_sync(0xffffffffu, live);
+              if (!live) break;
               const uint32_t bar = R.full0 + 8 * s;
+              if constexpr (RAG) {
+                const uint32_t row0 = sb + b * kColRows;
+                ragged_rows(md, row0, min((uint32_t)kColRows, pc.r1 - row0), c * md.vc * 16,
+                            min(md.vc * 16, md.rb - c * md.vc * 16), R.stage0 + s * kColStageBytes,
+                            (md.vc + kColRagPad) * 16, bar, pol, lane);
+                ++it;
+                continue;
+              }
               mbar_expect_tx(bar, kColRows * md.vc * 16);  // the whole box, zero fill included
               tma_load_2d(R.stage0 + s * kColStageBytes, tmap, (int32_t)(2 * c * md.vc),
                           (int32_t)(sb + b * kColRows), bar, pol);
@@ -317,7 +403,7 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT>::kCtasPerSm))
           }
         }
       }
-      if (!live || *R.abort_flag) {
+      if ((!live || *R.abort_flag) && lane == 0) {
         // drain: the copies of the last (up to kColStages) issued stages may still be in flight
         const uint32_t first = it > (uint32_t)kColStages ? it - kColStages : 0;
         for (uint32_t j = first; j < it; ++j) {
@@ -335,7 +421,7 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT>::kCtasPerSm))
     for (uint32_t pi = p0; pi < p1; ++pi) {
       const Piece pc = pieces[pi];
       const MatDesc md = mats[pc.mat];
-      cols_piece<DT, NT>(md, pc, R, red, it, par, warp, lane);
+      cols_piece<DT, NT, RAG>(md, pc, R, red, it, par, warp, lane);
     }
   }
   __syncthreads();
@@ -347,7 +433,11 @@ int gemm_cols_ctas_per_sm(int dtype, int nt) { return dtype == 3 ? 2 : 1; }
 
 template <int DT, int NT>
 static cudaError_t cols_attr() {
-  return cudaFuncSetAttribute(gemm_cols_kernel<DT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  static_assert(ColGeo<DT, NT>::kSmem == ColGeo<DT, NT, true>::kSmem, "one geometry");
+  const cudaError_t e = cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ColGeo<DT, NT>::kSmem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)ColGeo<DT, NT>::kSmem);
 }
 
@@ -362,12 +452,15 @@ cudaError_t gemm_cols_prepare() {
 
 template <int DT, int NT>
 static void cols_launch(const GemvLaunch &L, cudaStream_t s) {
-  gemm_cols_kernel<DT, NT><<<L.grid, kColThreads, ColGeo<DT, NT>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status,
-                                                                             L.maps);
+  constexpr size_t smem = ColGeo<DT, NT>::kSmem;
+  if (L.ragged)
+    gemm_cols_kernel<DT, NT, true><<<L.grid, kColThreads, smem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
+  else
+    gemm_cols_kernel<DT, NT, false><<<L.grid, kColThreads, smem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
 }
 
 cudaError_t launch_gemm_cols(const GemvLaunch &L, cudaStream_t s) {
-  if (L.maps == nullptr || (L.nt != 1 && L.nt != 2)) return cudaErrorInvalidValue;
+  if ((L.maps == nullptr && !L.ragged) || (L.nt != 1 && L.nt != 2)) return cudaErrorInvalidValue;
   switch (L.dtype * 4 + L.nt) {
     case 1 * 4 + 1: cols_launch<1, 1>(L, s); break;
     case 1 * 4 + 2: cols_launch<1, 2>(L, s); break;

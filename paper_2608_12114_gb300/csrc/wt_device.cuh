@@ -5,6 +5,8 @@
 
 #include <cstdint>
 
+#include "wt_kernels.h"
+
 namespace wt {
 namespace {
 
@@ -142,6 +144,58 @@ __device__ __forceinline__ uint4 lds_shifted(uint32_t addr) {
   const uint4 lo = lds128(addr - ph);
   const uint4 hi = lds128(addr - ph + (ph ? 16 : 0));
   return shift_bytes(lo, hi, ph);
+}
+
+// The mask of a vector's bytes [lo, hi).
+__device__ __forceinline__ uint4 byte_mask(int lo, int hi) {
+  uint32_t m[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int a = min(max(lo - 4 * i, 0), 4), b = min(max(hi - 4 * i, 0), 4);
+    m[i] = a >= b ? 0u : (0xffffffffu >> (32 - 8 * (b - a))) << (8 * a);
+  }
+  return make_uint4(m[0], m[1], m[2], m[3]);
+}
+
+__device__ __forceinline__ uint4 and4(const uint4 &a, const uint4 &b) {
+  return make_uint4(a.x & b.x, a.y & b.y, a.z & b.z, a.w & b.w);
+}
+
+// Bytes [off, off + len) of rows [r, r + n) of a ragged matrix to its stage, by the whole
+// producer warp (lane q takes rows q, q + 32, ...: one thread's address arithmetic alone held
+// such copies to 3.5 TB/s).  Row q arrives with its byte src at dst + q * pitch + (src & 15): a
+// bulk copy brings the whole 16-byte vectors that hold the range and lie inside the matrix;
+// bytes of the matrix's first or last vector that no such vector holds go one by one.
+__device__ __forceinline__ void ragged_rows(const MatDesc &md, uint32_t r, uint32_t n, uint32_t off, uint32_t len,
+                                            uint32_t dst, uint32_t pitch, uint32_t bar, uint64_t pol, int lane) {
+  const uint64_t w0 = reinterpret_cast<uint64_t>(md.W), wend = w0 + (uint64_t)(md.M - 1) * md.rs + md.rb;
+  const uint64_t wlo = (w0 + 15) & ~(uint64_t)15, whi = wend & ~(uint64_t)15;
+  for (uint32_t q0 = 0; q0 < n; q0 += 32) {
+    const uint32_t q = q0 + lane;
+    const uint64_t src = w0 + (uint64_t)(r + q) * md.rs + off, a = src & ~(uint64_t)15, end = src + len;
+    uint64_t lo = max(a, wlo), hi = min((end + 15) & ~(uint64_t)15, whi);
+    const uint32_t d = dst + q * pitch;
+    uint32_t bulk = 0;
+    if (q < n) {
+      if (hi > lo) bulk = (uint32_t)(hi - lo);
+      else lo = hi = end;
+      if (src < lo || hi < end) {
+        for (uint64_t p = src; p < lo; ++p) sts8(d + (uint32_t)(p - a), *reinterpret_cast<const uint8_t *>(p));
+        for (uint64_t p = max(hi, src); p < end; ++p)
+          sts8(d + (uint32_t)(p - a), *reinterpret_cast<const uint8_t *>(p));
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+    }
+    const uint32_t tx = __reduce_add_sync(0xffffffffu, bulk);
+    __syncwarp();
+    // the stage's one arrival comes with its last bytes announced, after every lane's stores
+    if (lane == 0) {
+      if (q0 + 32 < n) mbar_expect_only(bar, tx);
+      else mbar_expect_tx(bar, tx);
+    }
+    __syncwarp();
+    if (bulk) bulk_g2s(d + (uint32_t)(lo - a), reinterpret_cast<const void *>(lo), bulk, bar, pol);
+  }
 }
 
 // Two int8 weights as exact f16x2.  With u = b ^ 0x80 (0..255) in the low byte and 0x64 in

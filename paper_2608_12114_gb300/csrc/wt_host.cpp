@@ -365,7 +365,7 @@ struct Plan {
     bool umma = false;           // multi-column launch on tcgen05 (wt_umma.cu)
     bool q8rows = false;         // int8 multi-column launch on the row-owner kernel (wt_q8rows.cu)
     bool mapped_cols = false;    // map endpoint with T columns
-    bool ragged = false;         // one-column kernel: some matrix has ragged rows
+    bool ragged = false;         // some matrix has ragged rows (multi-column launches: every one)
     int nt = 0;                  // warp-MMA multi-column launches: 8-column tiles (1 or 2)
     uint32_t nmat = 0, ntiles = 0;
   };
@@ -1184,7 +1184,7 @@ void make_ragged(wt::MatDesc &m, int dtype, uint64_t row_bytes, uint64_t pitch_b
 // Multi-column kernel: chunks of at most kColVecMax vectors per row, evened out over the row
 // and rounded up to 4 (mod 8): 448 vectors -> 5 chunks of 92 (the last box zero-filled past
 // the row's end).
-wt::MatDesc make_cols_mat(const wt_gemv_desc &d) {
+wt::MatDesc make_cols_mat(const wt_gemv_desc &d, bool ragged = false) {
   wt::MatDesc m;
   memset(&m, 0, sizeof m);
   m.W = static_cast<const uint8_t *>(d.W);
@@ -1192,12 +1192,15 @@ wt::MatDesc make_cols_mat(const wt_gemv_desc &d) {
   m.y = d.y;
   m.s = static_cast<const uint8_t *>(d.scale);
   m.M = (uint32_t)d.M;
-  m.V = (uint32_t)(d.K * elem_bytes(d.dtype) / 16);
-  m.rs = m.V;
+  const uint64_t row_bytes = d.K * elem_bytes(d.dtype);
+  m.V = (uint32_t)((row_bytes + 15) / 16);
+  m.rs = ragged ? (uint32_t)row_bytes : m.V;
+  m.rb = ragged ? (uint32_t)row_bytes : 0;
   m.mode = wt::kModeCols;
   m.G = (uint16_t)d.cols;
   m.rt = 16;
-  const uint32_t nchunk = (m.V + wt::kColVecMax - 1) / wt::kColVecMax;
+  const uint32_t most = ragged ? wt::kColVecMaxRagged : wt::kColVecMax;
+  const uint32_t nchunk = (m.V + most - 1) / most;
   m.vc = ((m.V + nchunk - 1) / nchunk + 3) / 8 * 8 + 4;
   return m;
 }
@@ -1551,6 +1554,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
     g.first = mem.front();
     // cols_dt: warp-MMA multi-column with T <= 8, colsw_dt: with 8 < T <= 16
     std::vector<wt::MatDesc> by_dt[4], mapped_dt[4], cols_dt[4], umma_dt[4], mcols_dt[4], colsw_dt[4], q8r_dt[4],
+        ragc_dt[4], ragcw_dt[4],  // warp-MMA with ragged operands, T <= 8 and T > 8
         q8r1_dt[4];  // row-owner int8 launches with two 8-column tiles (T > 8) and with one
     std::vector<wt::MatDesc> i8c[2];  // int8 on the tensor cores, T <= 8 and T > 8: kernel chosen below
     uint64_t i8_blocks = 0;           // their 128-row blocks
@@ -1624,6 +1628,8 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         q1.cols = 1;
         i8c[0].push_back(make_cols_mat(q1));
         i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
+      } else if (q.cols > 0 && q.dtype != WT_F32 && q.K * es < 0x7fffffffull) {
+        (q.cols > 8 ? ragcw_dt : ragc_dt)[q.dtype].push_back(make_cols_mat(q, true));
       } else if (q.cols == 0 && (fast || q.K * es < 0x7fffffffull)) {
         // device memory, one column: whole 16-byte vectors per row, or ragged rows (any K, W
         // and x at any byte), which the one-warp-per-row kernel streamed at 500 to 2500 GB/s
@@ -1666,7 +1672,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
       lo.insert(lo.end(), i8c[0].begin(), i8c[0].end());
       hi.insert(hi.end(), i8c[1].begin(), i8c[1].end());
     }
-    for (int pass = 0; pass < 8; ++pass) {
+    for (int pass = 0; pass < 10; ++pass) {
       for (int dt = 0; dt < 4; ++dt) {
         std::vector<wt::MatDesc> &ms = pass == 0   ? by_dt[dt]
                                        : pass == 1 ? mapped_dt[dt]
@@ -1674,9 +1680,11 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
                                        : pass == 3 ? umma_dt[dt]
                                        : pass == 4 ? mcols_dt[dt]
                                        : pass == 5 ? colsw_dt[dt]
-                                       : pass == 6 ? q8r_dt[dt]
+                                       : pass == 6 ? ragc_dt[dt]
+                                       : pass == 7 ? ragcw_dt[dt]
+                                       : pass == 8 ? q8r_dt[dt]
                                                    : q8r1_dt[dt];
-        const bool warp_mma = pass == 2 || pass == 5;
+        const bool warp_mma = pass == 2 || pass >= 5;
         if (ms.empty()) continue;
         Plan::Launch L;
         L.dtype = dt;
@@ -1706,10 +1714,10 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           g.cols.push_back(L);
           continue;
         }
-        if (pass >= 6) {
+        if (pass >= 8) {
           // row-owner int8 launch: pieces cut at 128-row blocks, two tensor maps per matrix
           L.q8rows = true;
-          L.nt = pass == 6 ? 2 : 1;
+          L.nt = pass == 8 ? 2 : 1;
           partition(ms, L.grid, pieces, begin, (uint32_t)wt::kQ8RowsBlock, 1, 2);
           L.mats = append(P->table, ms);
           L.pieces = append(P->table, pieces);
@@ -1728,7 +1736,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
             if (m.mode != wt::kModeWarpRows && m.mode != wt::kModeBlockRows && m.mode != wt::kModePhaseRows)
               return set_err(WT_ENOTSUP, "wt_pass: internal: a %u-vector row reached the TMA kernel unsegmented", m.V);
         for (const wt::MatDesc &m : ms) L.ragged |= m.rb != 0;
-        L.nt = pass == 2 ? 1 : pass == 5 ? 2 : 0;
+        L.nt = pass == 2 || pass == 6 ? 1 : pass == 5 || pass == 7 ? 2 : 0;
         partition(ms, L.grid, pieces, begin, warp_mma ? (uint32_t)wt::kColTileRows : 1u,
                   pass == 0 ? one_col_slices(dt) : 1,
                   pass == 0 ? wt::gemv_ctas_per_sm(dt) : warp_mma ? wt::gemm_cols_ctas_per_sm(dt, L.nt) : 1);
@@ -1740,7 +1748,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
               P->ws_patches.push_back({L.mats + k * sizeof(wt::MatDesc) + offsetof(wt::MatDesc, y), (size_t)seg_ws[dt][k]});
         L.pieces = append(P->table, pieces);
         L.begin = append(P->table, begin);
-        if (warp_mma) {
+        if (warp_mma && !L.ragged) {
           L.maps = (P->table.size() + 127) & ~(size_t)127;
           P->table.resize(L.maps + ms.size() * wt::kTensorMapBytes);
           for (size_t k = 0; k < ms.size(); ++k) {
@@ -1900,7 +1908,8 @@ int run_plan(wt_handle *h, Plan *P, const wt_gemv_desc *d, cudaStream_t s, bool 
       gl.pieces = reinterpret_cast<const wt::Piece *>(P->dev + L.pieces);
       gl.begin = reinterpret_cast<const uint32_t *>(P->dev + L.begin);
       gl.status = h->status;
-      gl.maps = P->dev + L.maps;
+      gl.maps = L.ragged ? nullptr : P->dev + L.maps;
+      gl.ragged = L.ragged;
       gl.nt = L.nt;
       if (L.q8rows) {
         CU(wt::launch_gemm_q8_rows(gl, s));

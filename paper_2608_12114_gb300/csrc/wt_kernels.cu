@@ -488,21 +488,6 @@ __device__ __forceinline__ void stamp_full(uint64_t *st, uint32_t it, int warp, 
 // vectors are each put together from the two that hold them (two loads, eleven selects, four
 // shifts) 201 and 158 us: twice the instructions, on CTAs of eight warps.
 
-// The mask of a vector's bytes [lo, hi).
-__device__ __forceinline__ uint4 byte_mask(int lo, int hi) {
-  uint32_t m[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int a = min(max(lo - 4 * i, 0), 4), b = min(max(hi - 4 * i, 0), 4);
-    m[i] = a >= b ? 0u : (0xffffffffu >> (32 - 8 * (b - a))) << (8 * a);
-  }
-  return make_uint4(m[0], m[1], m[2], m[3]);
-}
-
-__device__ __forceinline__ uint4 and4(const uint4 &a, const uint4 &b) {
-  return make_uint4(a.x & b.x, a.y & b.y, a.z & b.z, a.w & b.w);
-}
-
 // A weight vector: on the 16-byte grid, or (int8) on the 8-byte grid.
 template <int DT>
 __device__ __forceinline__ uint4 lds_vec(uint32_t addr) {
@@ -701,45 +686,6 @@ __device__ __forceinline__ void phase_dispatch(const MatDesc &md, const Piece &p
 #undef WT_PH
 }
 
-// The copies of rows [r, r + nr) of a ragged matrix to their stage, by the whole producer warp:
-// whole rows are one range, the rows of a column segment one range each (lane q takes rows
-// q, q + 32, ...: one thread's address arithmetic alone held the copies to 3.5 TB/s).  A range
-// arrives with its byte src at dst + (src & 15): a bulk copy brings the whole 16-byte vectors
-// that hold it and lie inside the matrix; bytes of the matrix's first or last vector that no
-// such vector holds go one by one.
-__device__ __forceinline__ void ragged_tile(const MatDesc &md, uint32_t r, uint32_t nr, uint32_t dst, uint32_t bar,
-                                            uint64_t pol, int lane) {
-  const uint64_t w0 = reinterpret_cast<uint64_t>(md.W), wend = w0 + (uint64_t)(md.M - 1) * md.rs + md.rb;
-  const uint64_t wlo = (w0 + 15) & ~15ull, whi = wend & ~15ull;
-  const bool whole = md.rs == md.rb;
-  const uint32_t ranges = whole ? 1 : nr, len = whole ? nr * md.rb : md.rb;
-  for (uint32_t q0 = 0; q0 < ranges; q0 += 32) {
-    const uint32_t q = q0 + lane;
-    const uint64_t src = w0 + (uint64_t)(r + q) * md.rs, a = src & ~15ull, end = src + len;
-    uint64_t lo = max(a, wlo), hi = min((end + 15) & ~(uint64_t)15, whi);
-    const uint32_t d = dst + q * (md.V + 1) * 16;
-    uint32_t bulk = 0;
-    if (q < ranges) {
-      if (hi > lo) bulk = (uint32_t)(hi - lo);
-      else lo = hi = end;
-      if (src < lo || hi < end) {
-        for (uint64_t p = src; p < lo; ++p) sts8(d + (uint32_t)(p - a), *reinterpret_cast<const uint8_t *>(p));
-        for (uint64_t p = max(hi, src); p < end; ++p)
-          sts8(d + (uint32_t)(p - a), *reinterpret_cast<const uint8_t *>(p));
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      }
-    }
-    const uint32_t tx = __reduce_add_sync(0xffffffffu, bulk);
-    // the stage's one arrival comes with its last bytes announced, after every lane's stores
-    if (lane == 0) {
-      if (q0 + 32 < ranges) mbar_expect_only(bar, tx);
-      else mbar_expect_tx(bar, tx);
-    }
-    __syncwarp();
-    if (bulk) bulk_g2s(d + (uint32_t)(lo - a), reinterpret_cast<const void *>(lo), bulk, bar, pol);
-  }
-}
-
 // ST: the stamping instantiation, which also writes the per-CTA times of StampField to
 // stamps[blockIdx.x * kStampFields ...]; otherwise identical.  RAG: also takes matrices with
 // ragged rows (kModePhaseRows), and stamps if stamps is non-null.
@@ -813,7 +759,9 @@ __global__ void __launch_bounds__(kGemvThreads, GemvGeo<DT>::kCtasPerSm)
           const uint32_t bar = full0 + 8 * s;
           if (stamping && it == 0 && (!RAG || lane == 0)) st[kStFirstCopy] = globaltimer_ns();
           if (RAG && md.rb) {
-            ragged_tile(md, r, nr, dst, bar, pol, lane);
+            // whole rows are one range
+            if (md.rs == md.rb) ragged_rows(md, r, 1, 0, nr * md.rb, dst, 0, bar, pol, lane);
+            else ragged_rows(md, r, nr, 0, md.rb, dst, (md.V + 1) * 16, bar, pol, lane);
           } else if (!RAG || lane == 0) {
             mbar_expect_tx(bar, nr * vb);
             if (md.rs == md.V) {

@@ -44,6 +44,7 @@ enum GemvMode : uint16_t {
 // length vc = 4 (mod 8) so that the stage's row pitch vc * 16 is 64 bytes past a multiple
 // of 128 (the two rows a quarter-warp reads fall in different banks).
 constexpr int kColVecMax = 92;
+constexpr int kColVecMaxRagged = 84;  // ragged operands: the pitch is 8 vectors past the chunk
 constexpr int kColTileRows = 16;
 constexpr int kTensorMapBytes = 128;  // one CUtensorMap
 
@@ -61,8 +62,8 @@ struct alignas(16) MatDesc {
   uint32_t rs;    // row pitch in 16-byte vectors: V, or the full row of a column segment
                   // (segments are split-K only); s == nullptr then means "no scale yet"
   uint32_t cols;  // map endpoint with T activation columns: T (X [T, K], Y [T, M]); else 0
-  uint32_t rb;    // ragged rows (one-column kernel: rows, W or x off the 16-byte grid): bytes of a
-                  // row or row segment, V = ceil(rb / 16), and rs is the row pitch in bytes; else 0
+  uint32_t rb;    // ragged rows (rows, W or x off the 16-byte grid): bytes of a row or row segment,
+                  // V = ceil(rb / 16), and rs is the row pitch in bytes; else 0
 };
 static_assert(sizeof(MatDesc) == 64, "MatDesc is one 64-byte record");
 
@@ -110,7 +111,8 @@ struct GemvLaunch {
   int stall = 0;  // failure test (host fault site "stall"): the producer issues no copy, so
                   // every consumer wait runs out, reports WT_ETIMEDOUT and the CTA exits
   int nt = 0;     // multi-column kernel: 8-column MMA tiles of every matrix (T <= 8 nt)
-  int ragged = 0;  // one-column kernel: some matrix has ragged rows (MatDesc.rb > 0)
+  int ragged = 0;  // one-column kernel: some matrix has ragged rows (MatDesc.rb > 0);
+                   // multi-column kernel: every matrix has (maps stays null)
   int pdl = 0;    // one-column kernel: launch with programmatic stream serialization (the
                   // launch and prologue may overlap the previous kernel of the stream)
   uint64_t *stamps = nullptr;  // one-column kernel: non-null runs the stamping instantiation,
@@ -174,9 +176,9 @@ struct UmmaLaunch {
 cudaError_t gemm_cols_umma_prepare();
 cudaError_t launch_gemm_cols_umma(const UmmaLaunch &L, cudaStream_t s);
 
-// Fallback for operands the tiled kernels cannot take (W read in place from host memory, or
-// several columns, with unaligned W/x or rows whose byte length is not a multiple of 16; rows
-// of 2^31 bytes and more): one warp per row, scalar loads.  cols = 0 or 1: y = W x; cols = T > 1: Y [T, M] from X [T, K].
+// Fallback for operands the tiled kernels cannot take (W read in place from host memory with
+// unaligned W/x or rows whose byte length is not a multiple of 16, and such rows of 2^31 bytes
+// and more): one warp per row, scalar loads.  cols = 0 or 1: y = W x; cols = T > 1: Y [T, M] from X [T, K].
 cudaError_t launch_gemv_generic(int dtype, const uint8_t *W, const uint8_t *x, float *y,
                                 uint64_t M, uint64_t K, const uint8_t *scale, uint32_t cols,
                                 cudaStream_t s);

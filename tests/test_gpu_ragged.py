@@ -82,3 +82,44 @@ def test_ragged_rows_against_oracle(torch, dtype, odd):
             h.pass_([wt.gemv_desc(wp, dtype, M, K, xp, y2.data_ptr(), scale=sp)], 0)
             assert torch.equal(y2, y), (dtype, M, K)
         assert h.device_status() == 0
+
+
+# (M, bytes of a row, bytes past a 16-byte boundary of W and of X): a 16-row tile and a 64-row
+# super block and one more row; one 4-vector group; 84 vectors (one chunk) and one more; several
+# uneven chunks; aligned rows, also at unaligned addresses; the longest short rows (2048 bytes;
+# int8: 1024) and one byte or element either way; 32-row groups and several stages of them
+COL_SHAPES = [(1, 4, 0, 0), (17, 20, 4, 4), (64, 64, 4, 0), (65, 132, 0, 0), (33, 1340, 0, 4), (16, 1344, 4, 0),
+              (80, 1348, 0, 0), (130, 2732, 8, 8), (40, 5460, 0, 0), (23, 20004, 4, 4), (1100, 32, 0, 0), (600, 48, 0, 0),
+              (70, 1024, 0, 0), (33, 1028, 4, 0), (200, 2048, 0, 0), (35, 2052, 0, 0)]
+
+
+@pytest.mark.parametrize("dtype", [BF16, F16, I8])
+@pytest.mark.parametrize("T", [1, 8, 9, 16])
+def test_ragged_columns_against_oracle(torch, dtype, T):
+    """As above with T activation columns.  The tensor cores truncate where fp32 additions
+    round, so each of a sum's K additions may lose twice as much."""
+    rng = np.random.default_rng(1000 * dtype + T)
+    es = ES[dtype]
+    cs = []
+    for odd in (0, 1):
+        for M, kb, wo, xo in COL_SHAPES:
+            K = max(1, kb // es - odd)
+            W, X = weights(rng, dtype, M * K), weights(rng, F16 if dtype == I8 else dtype, T * K)
+            s = rng.uniform(0.001, 0.02, M).astype(np.float16).view(np.uint8) if dtype == I8 else None
+            wb, wp = at(torch, W, wo - wo % es)
+            xb, xp = at(torch, X, xo)
+            sb, sp = at(torch, s, 0) if s is not None else (None, 0)
+            y = torch.full((T * M,), float("nan"), dtype=torch.float32, device="cuda")
+            cs.append((M, K, wp, xp, sp, y, oracle.gemv_cols(W, dtype, M, K, X, T, scale=s), (wb, xb, sb)))
+    with wt.Handle([]) as h:
+        h.pass_([wt.gemv_desc(wp, dtype, M, K, xp, y.data_ptr(), scale=sp, cols=T) for M, K, wp, xp, sp, y, _, _ in cs], 0)
+        torch.cuda.synchronize()
+        assert h.device_status() == 0
+        for M, K, wp, xp, sp, y, (yhat, a), _ in cs:
+            err = oracle.gemv_error(y.cpu().numpy(), yhat.reshape(-1), a.reshape(-1))
+            assert err <= 2 * bound(K), (dtype, M, K, T, err)
+        for M, K, wp, xp, sp, y, _, _ in cs:
+            y2 = torch.full_like(y, float("nan"))
+            h.pass_([wt.gemv_desc(wp, dtype, M, K, xp, y2.data_ptr(), scale=sp, cols=T)], 0)
+            assert torch.equal(y2, y), (dtype, M, K, T)
+        assert h.device_status() == 0
