@@ -364,6 +364,7 @@ struct Plan {
     size_t maps = SIZE_MAX;      // multi-column launches: tensor maps (128-byte aligned)
     bool umma = false;           // multi-column launch on tcgen05 (wt_umma.cu)
     bool q8rows = false;         // int8 multi-column launch on the row-owner kernel (wt_q8rows.cu)
+    bool short_rows = false;     // multi-column launch on the short-row kernel (wt_colshort.cu)
     bool mapped_cols = false;    // map endpoint with T columns
     bool ragged = false;         // some matrix has ragged rows (multi-column launches: every one)
     int nt = 0;                  // warp-MMA multi-column launches: 8-column tiles (1 or 2)
@@ -622,6 +623,7 @@ int prepare_device(int dev) {
     CU(wt::gemm_cols_prepare());
     CU(wt::gemm_cols_umma_prepare());
     CU(wt::gemm_q8_rows_prepare());
+    CU(wt::gemm_short_prepare());
     g_prepared[dev] = true;
   }
   return WT_OK;
@@ -1169,7 +1171,6 @@ wt::MatDesc make_mat(const wt_gemv_desc &d) {
 // (16 bytes; int8: 8) at or before its start, so their number depends on the row's phase: G
 // is for the most.  A stage also holds the phases of its first and last row (whole
 // rows in one copy), or one more vector per row (column segments).
-constexpr uint32_t kRaggedSlack = 32;  // bytes of a stage
 uint32_t phase_vectors(uint64_t row_bytes, int dtype) { return (uint32_t)((row_bytes + (dtype == WT_I8 ? 7 : 15) + 15) / 16); }
 
 void make_ragged(wt::MatDesc &m, int dtype, uint64_t row_bytes, uint64_t pitch_bytes) {
@@ -1178,7 +1179,7 @@ void make_ragged(wt::MatDesc &m, int dtype, uint64_t row_bytes, uint64_t pitch_b
   m.rb = (uint32_t)row_bytes;
   m.rs = (uint32_t)pitch_bytes;
   m.G = (uint16_t)(nv <= 32 ? pow2ceil(nv) : 32);
-  m.rt = (wt::kStageBytes - kRaggedSlack) / (row_bytes == pitch_bytes ? m.rb : (m.V + 1) * 16);
+  m.rt = (wt::kStageBytes - wt::kRaggedSlack) / (row_bytes == pitch_bytes ? m.rb : (m.V + 1) * 16);
 }
 
 // Multi-column kernel: chunks of at most kColVecMax vectors per row, evened out over the row
@@ -1202,6 +1203,25 @@ wt::MatDesc make_cols_mat(const wt_gemv_desc &d, bool ragged = false) {
   const uint32_t most = ragged ? wt::kColVecMaxRagged : wt::kColVecMax;
   const uint32_t nchunk = (m.V + most - 1) / most;
   m.vc = ((m.V + nchunk - 1) / nchunk + 3) / 8 * 8 + 4;
+  return m;
+}
+
+// Multi-column matrices whose rows the short-row kernel takes: up to 1024 bytes (128 MiB in
+// bf16, T = 8 / 16, by row bytes: 64: 38 / 52 us against 334 / 107 us on the warp-MMA kernel
+// and tcgen05; 1024: 25.5 / 29.3 against 28.5 / 29.2; 2048: 32 / 39 against 26 / 31).  int8
+// rows of 65 to 512 weights go there only where the row-owner kernel has too few blocks
+// (T = 8: 64 weights 72 us against 68, 128: 48 against 41, 512: 28 against 25; but 153 and 45 us
+// on the warp-MMA kernel, which such small launches took), shorter ones always (32: 132 us
+// against 246).  WT_COLS_KERNEL, which names one of the other kernels, keeps the aligned ones
+// away from it.
+constexpr uint64_t kI8ShortK = 64;
+bool cols_on_short(const wt_gemv_desc &d, bool ragged) {
+  return d.K * elem_bytes(d.dtype) <= wt::short_row_bytes(d.dtype) && (ragged || !getenv("WT_COLS_KERNEL"));
+}
+
+wt::MatDesc make_short_mat(const wt_gemv_desc &d, bool ragged) {
+  wt::MatDesc m = make_cols_mat(d, ragged);
+  m.rt = ragged ? (wt::kStageBytes - wt::kRaggedSlack) / m.rb : wt::kStageBytes / (m.V * 16);
   return m;
 }
 
@@ -1350,10 +1370,13 @@ int encode_q8rows_maps(const wt::MatDesc &m, uint8_t *out) {
 // CUDA-core kernel's cross-CTA split-K, since the MMA kernels give a whole row to one CTA.
 // WT_I8_ONECOL=cuda keeps every int8 one-column matrix on the CUDA-core kernel (its parity
 // tests run both ways).
+// Rows of up to 64 weights stay on the CUDA cores too: an MMA's k is mostly padding there
+// (128 MiB of 32-weight rows: 53 us against 108 us on the short-row kernel and 167 us on the
+// row-owner kernel; 64 weights: 45, 52, 53 us; 128: 48, 38, 32 us).
 bool i8_onecol_on_mma(uint32_t V) {
   const char *e = getenv("WT_I8_ONECOL");
   if (e && strcmp(e, "cuda") == 0) return false;
-  return V <= wt::seg_vectors(WT_I8);
+  return (V > 4 || getenv("WT_COLS_KERNEL")) && V <= wt::seg_vectors(WT_I8);
 }
 
 // The two tensor maps of a tcgen05 multi-column matrix (2-byte weights; see wt::UmmaLaunch).
@@ -1387,19 +1410,34 @@ int encode_umma_maps(const wt::MatDesc &m, uint8_t *out) {
   return WT_OK;
 }
 
+// What a matrix costs a kernel, in bytes of weights.  Where kernels work in blocks, a partial
+// block costs a whole one; rows of the short-row kernel cost their outputs and, in int8, the
+// decoding of a padded vector besides (measured per row at T = 8 / 16: bf16 7 / 12 ps over
+// 0.18 ps a byte, int8 31 / 31 ps).  Sets of one row length are cut the same either way; the
+// many-small set in int8 took 611 us cut by bytes alone, the CTAs with the shortest rows last.
+struct CostModel {
+  uint32_t block = 1;     // rows of a block
+  uint32_t vecs = 1;      // 16-byte vectors of a row's step
+  uint32_t row_extra = 0;  // bytes a row costs besides
+  uint64_t row(const wt::MatDesc &m) const { return (uint64_t)(m.V + vecs - 1) / vecs * vecs * 16 + row_extra; }
+  uint64_t rows(const wt::MatDesc &m) const { return ((uint64_t)m.M + block - 1) / block * block; }
+};
+
 // Split the rows of `mats` (in order) into grid * slices contiguous slices of nearly
-// equal bytes, cut at row boundaries; slice j goes to CTA j % grid, so every CTA streams
+// equal cost (bytes, unless cost says otherwise), cut at row boundaries; slice j goes to CTA j % grid, so every CTA streams
 // `slices` slices spread over the whole set and gets a similar mix of shapes.  The grid is
 // at most ctas_per_sm CTAs per SM (all resident at once: the launch is persistent).
 void partition(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<wt::Piece> &pieces,
-               std::vector<uint32_t> &begin, uint32_t row_align = 1, int slices = 1, int ctas_per_sm = 1) {
-  uint64_t B = 0;
+               std::vector<uint32_t> &begin, uint32_t row_align = 1, int slices = 1, int ctas_per_sm = 1,
+               const CostModel &cost = CostModel()) {
+  uint64_t B = 0, C = 0;
   std::vector<uint64_t> start(mats.size() + 1, 0);
   for (size_t i = 0; i < mats.size(); ++i) {
-    start[i] = B;
+    start[i] = C;
     B += (uint64_t)mats[i].M * mats[i].V * 16;
+    C += cost.rows(mats[i]) * cost.row(mats[i]);
   }
-  start[mats.size()] = B;
+  start[mats.size()] = C;
   constexpr uint64_t kMinCtaBytes = 64 << 10;
   grid = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((uint64_t)wt::num_sms() * ctas_per_sm, (B + kMinCtaBytes - 1) / kMinCtaBytes));
@@ -1413,14 +1451,14 @@ void partition(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<wt::
   }
   slices = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)slices, B / ((uint64_t)grid * min_slice)));
   const int nslice = grid * slices;
-  // cut c (1..nslice-1) at the row boundary nearest byte B*c/nslice
+  // cut c (1..nslice-1) at the row boundary nearest cost C*c/nslice
   std::vector<std::pair<uint32_t, uint32_t>> cuts;  // (mat, row)
   cuts.push_back({0, 0});
   size_t m = 0;
   for (int c = 1; c < nslice; ++c) {
-    const uint64_t T = (uint64_t)((unsigned __int128)B * c / nslice);
+    const uint64_t T = (uint64_t)((unsigned __int128)C * c / nslice);
     while (m + 1 < mats.size() && start[m + 1] <= T) ++m;
-    const uint64_t rb = (uint64_t)mats[m].V * 16;
+    const uint64_t rb = cost.row(mats[m]);
     uint64_t row = (T - start[m] + rb / 2) / rb;
     row = (row + row_align / 2) / row_align * row_align;  // whole tiles per slice
     std::pair<uint32_t, uint32_t> cut = {(uint32_t)m, (uint32_t)std::min<uint64_t>(row, mats[m].M)};
@@ -1555,8 +1593,9 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
     // cols_dt: warp-MMA multi-column with T <= 8, colsw_dt: with 8 < T <= 16
     std::vector<wt::MatDesc> by_dt[4], mapped_dt[4], cols_dt[4], umma_dt[4], mcols_dt[4], colsw_dt[4], q8r_dt[4],
         ragc_dt[4], ragcw_dt[4],  // warp-MMA with ragged operands, T <= 8 and T > 8
+        short_dt[4][4],           // [dtype][T > 8, + 2 if ragged]: short rows
         q8r1_dt[4];  // row-owner int8 launches with two 8-column tiles (T > 8) and with one
-    std::vector<wt::MatDesc> i8c[2];  // int8 on the tensor cores, T <= 8 and T > 8: kernel chosen below
+    std::vector<wt_gemv_desc> i8c[2];  // int8 on the tensor cores, T <= 8 and T > 8: kernel chosen below
     uint64_t i8_blocks = 0;           // their 128-row blocks
     std::vector<int64_t> seg_ws[4];  // per by_dt entry: workspace float offset of its partials, or -1
     std::vector<wt::SegReduce> reds;
@@ -1617,8 +1656,10 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           g.generic.push_back({q.dtype, static_cast<const uint8_t *>(q.W), static_cast<const uint8_t *>(q.x), q.y, q.M, q.K,
                                static_cast<const uint8_t *>(q.scale), ncol});
         }
+      } else if (q.cols > 0 && q.dtype != WT_F32 && cols_on_short(q, !fast) && (!fast || q.dtype != WT_I8 || q.K <= kI8ShortK)) {
+        short_dt[q.dtype][(q.cols > 8) + 2 * !fast].push_back(make_short_mat(q, !fast));
       } else if (fast && q.cols > 0 && q.dtype == WT_I8) {
-        i8c[q.cols > 8 ? 1 : 0].push_back(make_cols_mat(q));
+        i8c[q.cols > 8 ? 1 : 0].push_back(q);
         i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
       } else if (fast && q.cols > 0) {
         (cols_on_umma(q.dtype, q.cols) ? umma_dt : q.cols > 8 ? colsw_dt : cols_dt)[q.dtype].push_back(make_cols_mat(q));
@@ -1626,7 +1667,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         // y[M] is Y[1, M] and x[K] is X[1, K]: the one-column GEMV as a T = 1 tensor-core GEMV
         wt_gemv_desc q1 = q;
         q1.cols = 1;
-        i8c[0].push_back(make_cols_mat(q1));
+        i8c[0].push_back(q1);
         i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
       } else if (q.cols > 0 && q.dtype != WT_F32 && q.K * es < 0x7fffffffull) {
         (q.cols > 8 ? ragcw_dt : ragc_dt)[q.dtype].push_back(make_cols_mat(q, true));
@@ -1667,12 +1708,13 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
     }
     if (!i8c[0].empty() || !i8c[1].empty()) {
       const bool rows = i8_on_q8rows(i8_blocks);
-      auto &lo = rows ? q8r1_dt[WT_I8] : cols_dt[WT_I8];
-      auto &hi = rows ? q8r_dt[WT_I8] : colsw_dt[WT_I8];
-      lo.insert(lo.end(), i8c[0].begin(), i8c[0].end());
-      hi.insert(hi.end(), i8c[1].begin(), i8c[1].end());
+      for (int w = 0; w < 2; ++w)
+        for (const wt_gemv_desc &q : i8c[w]) {
+          if (!rows && cols_on_short(q, false)) short_dt[WT_I8][w].push_back(make_short_mat(q, false));
+          else (rows ? (w ? q8r_dt : q8r1_dt) : (w ? colsw_dt : cols_dt))[WT_I8].push_back(make_cols_mat(q));
+        }
     }
-    for (int pass = 0; pass < 10; ++pass) {
+    for (int pass = 0; pass < 14; ++pass) {
       for (int dt = 0; dt < 4; ++dt) {
         std::vector<wt::MatDesc> &ms = pass == 0   ? by_dt[dt]
                                        : pass == 1 ? mapped_dt[dt]
@@ -1683,8 +1725,9 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
                                        : pass == 6 ? ragc_dt[dt]
                                        : pass == 7 ? ragcw_dt[dt]
                                        : pass == 8 ? q8r_dt[dt]
-                                                   : q8r1_dt[dt];
-        const bool warp_mma = pass == 2 || pass >= 5;
+                                       : pass == 9 ? q8r1_dt[dt]
+                                                   : short_dt[dt][pass - 10];
+        const bool warp_mma = pass == 2 || (pass >= 5 && pass < 8);
         if (ms.empty()) continue;
         Plan::Launch L;
         L.dtype = dt;
@@ -1714,11 +1757,28 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           g.cols.push_back(L);
           continue;
         }
+        if (pass >= 10) {
+          // short rows: pieces cut at 32-row groups
+          L.short_rows = true;
+          L.nt = (pass - 10) % 2 + 1;
+          L.ragged = pass >= 12;
+          CostModel cm;
+          cm.row_extra = 4 * 8 * L.nt + (dt == WT_I8 ? 160 : 16);
+          partition(ms, L.grid, pieces, begin, 32, 1, 1, cm);
+          L.mats = append(P->table, ms);
+          L.pieces = append(P->table, pieces);
+          L.begin = append(P->table, begin);
+          g.cols.push_back(L);
+          continue;
+        }
         if (pass >= 8) {
           // row-owner int8 launch: pieces cut at 128-row blocks, two tensor maps per matrix
           L.q8rows = true;
           L.nt = pass == 8 ? 2 : 1;
-          partition(ms, L.grid, pieces, begin, (uint32_t)wt::kQ8RowsBlock, 1, 2);
+          CostModel cm;
+          cm.block = wt::kQ8RowsBlock;
+          cm.vecs = 192 / 16;
+          partition(ms, L.grid, pieces, begin, (uint32_t)wt::kQ8RowsBlock, 1, 2, cm);
           L.mats = append(P->table, ms);
           L.pieces = append(P->table, pieces);
           L.begin = append(P->table, begin);
@@ -1908,10 +1968,12 @@ int run_plan(wt_handle *h, Plan *P, const wt_gemv_desc *d, cudaStream_t s, bool 
       gl.pieces = reinterpret_cast<const wt::Piece *>(P->dev + L.pieces);
       gl.begin = reinterpret_cast<const uint32_t *>(P->dev + L.begin);
       gl.status = h->status;
-      gl.maps = L.ragged ? nullptr : P->dev + L.maps;
+      gl.maps = L.maps == SIZE_MAX ? nullptr : P->dev + L.maps;
       gl.ragged = L.ragged;
       gl.nt = L.nt;
-      if (L.q8rows) {
+      if (L.short_rows) {
+        CU(wt::launch_gemm_short(gl, s));
+      } else if (L.q8rows) {
         CU(wt::launch_gemm_q8_rows(gl, s));
       } else if (L.umma) {
         wt::UmmaLaunch ul;

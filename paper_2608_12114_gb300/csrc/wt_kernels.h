@@ -74,6 +74,9 @@ static_assert(sizeof(MatDesc) == 64, "MatDesc is one 64-byte record");
 // segments of each row in segment order and applies the row scale.  Segment boundaries
 // depend only on the matrix, so a row's result never depends on how rows and segments were
 // spread over CTAs.
+// What a stage of whole ragged rows needs besides them: the phases of its two ends.
+constexpr uint32_t kRaggedSlack = 32;
+
 // Ragged rows: at most this many vectors, counted from the grid point at or before the row's
 // start (the x registers of a lane: 64, or 48 for int8, which runs two CTAs per SM).
 constexpr uint32_t kPhaseVec(int dtype) { return dtype == 3 ? 192 : 512; }
@@ -157,6 +160,13 @@ cudaError_t launch_gemv_mapped_cols(const GemvLaunch &L, cudaStream_t s);
 cudaError_t gemm_cols_prepare();
 cudaError_t launch_gemm_cols(const GemvLaunch &L, cudaStream_t s);
 int gemm_cols_ctas_per_sm(int dtype, int nt);
+
+// The same for short rows (wt_colshort.cu), at most short_row_bytes each: stages of whole rows,
+// rt of them (32 KB, less kRaggedSlack for ragged ones).  One launch
+// holds matrices of one dtype and one nt, all ragged (MatDesc.rb > 0, GemvLaunch.ragged) or none.
+constexpr uint32_t short_row_bytes(int dtype) { return dtype == 3 ? 512 : 1024; }
+cudaError_t gemm_short_prepare();
+cudaError_t launch_gemm_short(const GemvLaunch &L, cudaStream_t s);
 
 // The same multi-column GEMV on tcgen05 for 2-byte weights (wt_umma.cu): row tiles of 128
 // rows, K in chunks of 64 elements, accumulators in tensor memory.  pieces[m] = {m, first
