@@ -64,6 +64,13 @@ static_assert(kColStageBytes % 128 == 0, "stages stay 128-byte aligned for the t
 // CTAs per SM with half the ring each (the same bytes in flight per SM, twice the warps; the
 // int8 path is latency-bound on its decode).  The cross-warp partials of one 16-row tile take
 // 16 x 8 NT floats per warp, in two alternating halves.
+// Where a partial sum of (column, row) sits among its tile's: a pair of columns takes 32 floats,
+// turned by 8 per pair, so that neither the stores of a fragment (rows g of the columns 2t; in
+// plain order the four shared a bank) nor the sums over a pair meet in a bank.
+__device__ __forceinline__ uint32_t red_at(uint32_t col, uint32_t row) {
+  return (col >> 1) * 32 + ((((col & 1) << 4) + row + 8 * (col >> 1)) & 31);
+}
+
 template <int DT, int NT, bool RAG = false>
 struct ColGeo {
   static constexpr int kCtasPerSm = DT == 3 ? 2 : 1;
@@ -183,20 +190,21 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int3
 
 // One stage: rows g and g + 8 of the tile against this warp's vectors of the chunk.
 // Thread (g, t) takes vector (q * warps + warp) * 4 + t of group q.
-// The box holds vc vectors per row at pitch vc * 16; rows and vectors past the matrix are
-// zeros, so only whole groups past vc are skipped.
+// The box holds vc vectors per row at pitch vc * 16, nv of them the row's; rows and vectors past
+// the matrix are zeros, so only whole groups past nv are skipped (at K = 1024 the 17th group of
+// a chunk is padding, and was warp 0's third).
 // RAG: row g starts ph0 bytes past its pitch's start, row g + 8 ph1 bytes; of vector v only the
 // row's own bytes count (left: those from the chunk's start on; an int8 neighbour meets a zero
 // of X and is a finite number, so only the 2-byte types mask it).
 template <int DT, int NT, int H, bool RAG>
-__device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, int warp, uint32_t g, uint32_t t,
+__device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t nv, int warp, uint32_t g, uint32_t t,
                                            const uint32_t (&xr)[kColGroups][NT][ColX<DT>::W], float (&acc)[H][NT][4],
                                            uint32_t ph0, uint32_t ph1, uint32_t left) {
   const uint32_t pitch = RAG ? (vc + kColRagPad) * 16 : vc * 16;
 #pragma unroll
   for (int q = 0; q < kColGroups; ++q) {
     const uint32_t v0 = (uint32_t)(q * kColWarps + warp) * 4;
-    if (v0 >= vc) continue;  // warp-uniform: the box ends before this group
+    if (v0 >= nv) continue;  // warp-uniform: the row ends before this group
     const uint32_t v = v0 + t;
     uint4 w0, w1;
     if constexpr (RAG) {
@@ -292,7 +300,7 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
           const uint32_t s = it % ColGeo<DT, NT, RAG>::kStages;
           bounded_wait(R.full0 + 8 * s, (it / ColGeo<DT, NT, RAG>::kStages) & 1, R.abort_flag, R.status);
           const uint64_t row = reinterpret_cast<uint64_t>(md.W) + (uint64_t)(sb + b * kColRows + g) * md.rb;
-          cols_stage<DT, NT, H, RAG>(R.stage0 + s * kColStageBytes, vc, warp, g, t, xr, acc[b], (uint32_t)row & 15u,
+          cols_stage<DT, NT, H, RAG>(R.stage0 + s * kColStageBytes, vc, nv, warp, g, t, xr, acc[b], (uint32_t)row & 15u,
                                      (uint32_t)(row + 8ull * md.rb) & 15u, md.rb - c * vc * 16);
           __syncwarp();
           if (lane == 0) mbar_arrive(R.empty0 + 8 * s);
@@ -313,10 +321,10 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
           const uint32_t c0 = 2 * t + 8 * n;
-          r[c0 * 16 + g] = acc[b][0][n][0] + (H == 2 ? acc[b][H - 1][n][0] : 0.f);
-          r[(c0 + 1) * 16 + g] = acc[b][0][n][1] + (H == 2 ? acc[b][H - 1][n][1] : 0.f);
-          r[c0 * 16 + g + 8] = acc[b][0][n][2] + (H == 2 ? acc[b][H - 1][n][2] : 0.f);
-          r[(c0 + 1) * 16 + g + 8] = acc[b][0][n][3] + (H == 2 ? acc[b][H - 1][n][3] : 0.f);
+          r[red_at(c0, g)] = acc[b][0][n][0] + (H == 2 ? acc[b][H - 1][n][0] : 0.f);
+          r[red_at(c0 + 1, g)] = acc[b][0][n][1] + (H == 2 ? acc[b][H - 1][n][1] : 0.f);
+          r[red_at(c0, g + 8)] = acc[b][0][n][2] + (H == 2 ? acc[b][H - 1][n][2] : 0.f);
+          r[red_at(c0 + 1, g + 8)] = acc[b][0][n][3] + (H == 2 ? acc[b][H - 1][n][3] : 0.f);
         }
       }
     }
@@ -324,7 +332,7 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
     for (uint32_t o = ct; o < nrb * kStride; o += kColConsumers) {
       const uint32_t b = o / kStride, e = o % kStride, col = e >> 4, row = b * kColRows + (e & 15);
       if (col < T && row < rows) {
-        const float *r = red + b * kColWarps * kStride + e;
+        const float *r = red + b * kColWarps * kStride + red_at(col, e & 15);
         float sum = 0.f;
 #pragma unroll
         for (int w = 0; w < kColWarps; ++w) sum += r[w * kStride];
