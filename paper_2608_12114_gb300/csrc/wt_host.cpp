@@ -1206,17 +1206,23 @@ wt::MatDesc make_cols_mat(const wt_gemv_desc &d, bool ragged = false) {
   return m;
 }
 
+// The multi-column kernel that WT_COLS_KERNEL names: 1 umma, 2 mma, 3 q8rows, 0 none.
+int cols_forced() {
+  const char *e = getenv("WT_COLS_KERNEL");
+  return !e ? 0 : strcmp(e, "umma") == 0 ? 1 : strcmp(e, "mma") == 0 ? 2 : strcmp(e, "q8rows") == 0 ? 3 : 0;
+}
+
 // Multi-column matrices whose rows the short-row kernel takes: up to 1024 bytes (128 MiB in
 // bf16, T = 8 / 16, by row bytes: 64: 38 / 52 us against 334 / 107 us on the warp-MMA kernel
 // and tcgen05; 1024: 25.5 / 29.3 against 28.5 / 29.2; 2048: 32 / 39 against 26 / 31).  int8
-// rows of 65 to 512 weights go there only where the row-owner kernel has too few blocks
-// (T = 8: 64 weights 72 us against 68, 128: 48 against 41, 512: 28 against 25; but 153 and 45 us
+// rows of 64 to 512 weights go there only where the row-owner kernel's blocks leave the CTAs
+// uneven (T = 8: 64 weights 72 us against 68, 128: 48 against 41, 512: 28 against 25; but 153 and 45 us
 // on the warp-MMA kernel, which such small launches took), shorter ones always (32: 132 us
 // against 246).  WT_COLS_KERNEL, which names one of the other kernels, keeps the aligned ones
 // away from it.
-constexpr uint64_t kI8ShortK = 64;
+constexpr uint64_t kI8ShortK = 63;
 bool cols_on_short(const wt_gemv_desc &d, bool ragged) {
-  return d.K * elem_bytes(d.dtype) <= wt::short_row_bytes(d.dtype) && (ragged || !getenv("WT_COLS_KERNEL"));
+  return d.K * elem_bytes(d.dtype) <= wt::short_row_bytes(d.dtype) && (ragged || !cols_forced());
 }
 
 wt::MatDesc make_short_mat(const wt_gemv_desc &d, bool ragged) {
@@ -1305,32 +1311,6 @@ int encode_cols_map(const wt::MatDesc &m, uint8_t *out) {
 // costs an exposed reload of x.
 int one_col_slices(int dtype) { return dtype == WT_I8 ? 1 : 16; }
 
-// Which multi-column kernel runs a matrix: tcgen05 (wt_umma.cu) for 2-byte weights with more
-// than 8 columns, where its T-independent tensor time wins (bf16 protocol, T = 16: 6529
-// against 6370 GB/s); the warp-level MMA kernel (wt_cols.cu) otherwise (T = 1: 6958 against
-// 6580; int8 decodes in registers there).  WT_COLS_KERNEL=mma or =umma forces one kernel
-// (umma still only for 2-byte weights).
-bool cols_on_umma(int dtype, int cols) {
-  const char *e = getenv("WT_COLS_KERNEL");
-  const int force = e && strcmp(e, "umma") == 0 ? 1 : e && strcmp(e, "mma") == 0 ? 2 : 0;
-  if (dtype != WT_BF16 && dtype != WT_F16) return false;
-  return force == 1 || (force == 0 && cols > 8);
-}
-
-// int8 weights on the tensor cores (T columns, and one column with rows up to K = 8192) run
-// the row-owner kernel (wt_q8rows.cu) when its 128-row blocks fill the GPU (at least two per
-// CTA slot over the launch): its warps keep no activation registers and meet in no reduction.
-// The matched protocol: T = 1 / 8 / 16 at 6663 / 6581 / 6502 GB/s against 6565 / 6250 / 5004
-// on the warp-MMA kernel.  Launches of fewer rows keep the warp-MMA kernel's 16-row tiles,
-// which spread over 8 times as many CTAs.  WT_COLS_KERNEL=mma or =q8rows forces one kernel
-// for every int8 matrix (the parity tests run each routing).
-bool i8_on_q8rows(uint64_t blocks) {
-  const char *e = getenv("WT_COLS_KERNEL");
-  if (e && strcmp(e, "mma") == 0) return false;
-  if (e && strcmp(e, "q8rows") == 0) return true;
-  return blocks >= 2ull * wt::num_sms();
-}
-
 // The two tensor maps of a row-owner int8 matrix (see wt::launch_gemm_q8_rows).
 int encode_q8rows_maps(const wt::MatDesc &m, uint8_t *out) {
   EncodeTiledFn fn = encode_tiled();
@@ -1376,7 +1356,7 @@ int encode_q8rows_maps(const wt::MatDesc &m, uint8_t *out) {
 bool i8_onecol_on_mma(uint32_t V) {
   const char *e = getenv("WT_I8_ONECOL");
   if (e && strcmp(e, "cuda") == 0) return false;
-  return (V > 4 || getenv("WT_COLS_KERNEL")) && V <= wt::seg_vectors(WT_I8);
+  return (V > 4 || cols_forced()) && V <= wt::seg_vectors(WT_I8);
 }
 
 // The two tensor maps of a tcgen05 multi-column matrix (2-byte weights; see wt::UmmaLaunch).
@@ -1423,10 +1403,30 @@ struct CostModel {
   uint64_t rows(const wt::MatDesc &m) const { return ((uint64_t)m.M + block - 1) / block * block; }
 };
 
+CostModel q8rows_cost() {
+  CostModel c;
+  c.block = wt::kQ8RowsBlock;
+  c.vecs = 192 / 16;
+  return c;
+}
+
+CostModel warp_mma_cost() {
+  CostModel c;
+  c.block = wt::kColTileRows;
+  return c;
+}
+
+// CTAs for B bytes of weights: all that are resident at once (the launch is persistent), and
+// at least 64 KB each.
+int max_grid(uint64_t B, int ctas_per_sm) {
+  constexpr uint64_t kMinCtaBytes = 64 << 10;
+  return (int)std::max<uint64_t>(
+      1, std::min<uint64_t>((uint64_t)wt::num_sms() * ctas_per_sm, (B + kMinCtaBytes - 1) / kMinCtaBytes));
+}
+
 // Split the rows of `mats` (in order) into grid * slices contiguous slices of nearly
 // equal cost (bytes, unless cost says otherwise), cut at row boundaries; slice j goes to CTA j % grid, so every CTA streams
-// `slices` slices spread over the whole set and gets a similar mix of shapes.  The grid is
-// at most ctas_per_sm CTAs per SM (all resident at once: the launch is persistent).
+// `slices` slices spread over the whole set and gets a similar mix of shapes.
 void partition(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<wt::Piece> &pieces,
                std::vector<uint32_t> &begin, uint32_t row_align = 1, int slices = 1, int ctas_per_sm = 1,
                const CostModel &cost = CostModel()) {
@@ -1438,9 +1438,7 @@ void partition(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<wt::
     C += cost.rows(mats[i]) * cost.row(mats[i]);
   }
   start[mats.size()] = C;
-  constexpr uint64_t kMinCtaBytes = 64 << 10;
-  grid = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>((uint64_t)wt::num_sms() * ctas_per_sm, (B + kMinCtaBytes - 1) / kMinCtaBytes));
+  grid = max_grid(B, ctas_per_sm);
   // slices of at least 2 MiB: a slice costs the consumers a reload of x, and a slice shorter
   // than a tile makes its stages partial.  WT_MIN_SLICE_BYTES (>= 4096) lowers the floor so
   // that tests reach the many-slices-per-CTA partition on sets far smaller than a decoder.
@@ -1480,6 +1478,116 @@ void partition(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<wt::
     }
     begin.push_back((uint32_t)pieces.size());
   }
+}
+
+// Deal the tiles (cost.block rows) of `mats` to the CTAs of a tiled kernel, equal cost to each:
+// matrices with the dearest tiles first, every CTA as many as fit its share, so that the cheaper
+// tiles of later matrices fill what whole tiles leave open; the cheapest in contiguous runs cut
+// nearest to what each CTA lacks (a set of one tile cost is thus cut as partition cuts it).  A tile of long rows is a large part
+// of a share (two decoder layers in bf16: 458 KB of 5.7 MB; one mid layer in int8: 110 of
+// 259 KB), and contiguous shares cut at tiles left some CTAs one tile over.
+// Returns the largest CTA's cost over an even share of the weights' bytes.
+double deal_tiles(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<wt::Piece> &pieces,
+                  std::vector<uint32_t> &begin, int ctas_per_sm, const CostModel &cost) {
+  uint64_t B = 0, C = 0;
+  std::vector<uint32_t> order(mats.size());
+  for (size_t i = 0; i < mats.size(); ++i) {
+    order[i] = (uint32_t)i;
+    B += (uint64_t)mats[i].M * mats[i].V * 16;
+    C += cost.rows(mats[i]) * cost.row(mats[i]);
+  }
+  std::stable_sort(order.begin(), order.end(),
+                   [&](uint32_t a, uint32_t b) { return cost.row(mats[a]) > cost.row(mats[b]); });
+  grid = max_grid(B, ctas_per_sm);
+  std::vector<int64_t> left(grid, (int64_t)((C + grid - 1) / grid));
+  std::vector<std::pair<int, wt::Piece>> dealt;
+  const uint64_t cheapest = cost.row(mats[order.back()]) * cost.block;
+  uint64_t last = 0;  // tile cost of the previous matrix: its CTAs are full up to `c` for this one
+  int c = 0;
+  int64_t lack = 0;  // cheapest tiles: what CTAs up to c lack beyond the tiles dealt so far
+  for (const uint32_t i : order) {
+    const wt::MatDesc &m = mats[i];
+    const uint64_t tc = cost.row(m) * cost.block;
+    if (tc != last) c = 0;
+    if (tc == cheapest && last != tc) lack = left[0];
+    last = tc;
+    uint32_t r = 0;
+    const auto give = [&](int to, uint64_t tiles) {
+      const uint32_t r1 = (uint32_t)std::min<uint64_t>(m.M, r + tiles * cost.block);
+      dealt.push_back({to, {i, r, r1, 0}});
+      left[to] -= (int64_t)(tiles * tc);
+      r = r1;
+    };
+    if (tc == cheapest) {
+      while (r < m.M) {
+        const uint64_t run = lack > 0 ? ((uint64_t)lack + tc / 2) / tc : 0;
+        if (run > 0 || c == grid - 1) {
+          const uint64_t tiles = (m.M - r + cost.block - 1) / cost.block;
+          const uint64_t k = c == grid - 1 ? tiles : std::min(run, tiles);
+          give(c, k);
+          lack -= (int64_t)(k * tc);
+          if (k < run) break;  // the matrix has ended; the next one goes on here
+        }
+        if (c < grid - 1) lack += left[++c];
+      }
+      continue;
+    }
+    for (; r < m.M; ++c) {
+      if (c == grid) break;
+      const uint64_t fit = left[c] > 0 ? (uint64_t)left[c] / tc : 0;
+      if (fit == 0) continue;
+      give(c, std::min<uint64_t>(fit, (m.M - r + cost.block - 1) / cost.block));
+      if (r == m.M) break;  // the next matrix of this tile cost goes on here
+    }
+    if (r < m.M) {  // no CTA has room for a whole tile: one each to those with the most left
+      std::vector<std::pair<int64_t, int>> by_left(grid);
+      for (int k = 0; k < grid; ++k) by_left[k] = {-left[k], k};
+      std::make_heap(by_left.begin(), by_left.end(), std::greater<std::pair<int64_t, int>>());
+      while (r < m.M) {
+        std::pop_heap(by_left.begin(), by_left.end(), std::greater<std::pair<int64_t, int>>());
+        give(by_left.back().second, 1);
+        by_left.back().first += (int64_t)tc;
+        std::push_heap(by_left.begin(), by_left.end(), std::greater<std::pair<int64_t, int>>());
+      }
+    }
+  }
+  begin.assign(grid + 1, 0);
+  for (const auto &d : dealt) ++begin[d.first + 1];
+  for (int k = 0; k < grid; ++k) begin[k + 1] += begin[k];
+  pieces.resize(dealt.size());
+  std::vector<uint32_t> at(begin.begin(), begin.end() - 1);
+  for (const auto &d : dealt) pieces[at[d.first]++] = d.second;
+  const int64_t most = (int64_t)((C + grid - 1) / grid) - *std::min_element(left.begin(), left.end());
+  return (double)most * grid / (double)std::max<uint64_t>(1, B);
+}
+
+// 2-byte weights with more than 8 columns run on the warp-level MMA kernel (wt_cols.cu), or on
+// tcgen05 (wt_umma.cu) where a launch has at least 16 of its 128-row tiles per SM.  tcgen05 keeps
+// the rate of HBM at any T but deals whole tiles, and a launch waits for the CTA with one more
+// (T = 16, bf16, us on tcgen05 / warp-MMA: the large decoder, 84 tiles per SM: 2441 / 2533;
+// 65536 x 1024 x 8, 27: 170 / 211; 8192 x 4096 x 16, 6.7: 167 / 165; two large layers, 4.4:
+// 173 / 141; four mid layers 137 / 105; 4096 x 4096: 27 / 12).  Up to 8 columns the warp-MMA
+// kernel is the faster throughout.  WT_COLS_KERNEL=mma or =umma forces one kernel (umma still
+// only for 2-byte weights).
+bool cols_on_umma(const std::vector<wt::MatDesc> &ms) {
+  const int f = cols_forced();
+  uint64_t tiles = 0;
+  for (const wt::MatDesc &m : ms) tiles += (m.M + 127) / 128;
+  return f != 2 && tiles >= 16ull * wt::num_sms();
+}
+
+// int8 weights on the tensor cores (T columns, and one column with rows up to K = 8192) run
+// the row-owner kernel (wt_q8rows.cu) unless its 128-row blocks leave the CTAs uneven: its
+// warps keep no activation registers and meet in no reduction, but a launch waits for the CTA
+// with one block more, where the warp-MMA kernel cuts at 16 rows.  Even, it is the faster by
+// 2, 5 and 30 % at T = 1, 8 and 16 (6663 / 6581 / 6502 GB/s against 6565 / 6250 / 5004); with
+// the largest CTA at 1.2 times an even share (128 MiB of 2048-weight rows) by 18 and 60 % at
+// T = 8 and 16; at 1.8 times (one large decoder layer, 336 blocks for 304 CTAs) it takes 51 /
+// 51 / 56 us and the warp-MMA kernel 39 / 40 / 55.  WT_COLS_KERNEL=mma or =q8rows forces one kernel for every int8 matrix
+// (the parity tests run each routing).
+bool i8_on_q8rows(double share, bool wide) {
+  const int f = cols_forced();
+  return f == 3 || (f != 2 && share < (wide ? 1.6 : 1.35));
 }
 
 size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
@@ -1596,7 +1704,6 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         short_dt[4][4],           // [dtype][T > 8, + 2 if ragged]: short rows
         q8r1_dt[4];  // row-owner int8 launches with two 8-column tiles (T > 8) and with one
     std::vector<wt_gemv_desc> i8c[2];  // int8 on the tensor cores, T <= 8 and T > 8: kernel chosen below
-    uint64_t i8_blocks = 0;           // their 128-row blocks
     std::vector<int64_t> seg_ws[4];  // per by_dt entry: workspace float offset of its partials, or -1
     std::vector<wt::SegReduce> reds;
     std::vector<size_t> red_ws;      // per reds entry: workspace float offset
@@ -1660,15 +1767,13 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         short_dt[q.dtype][(q.cols > 8) + 2 * !fast].push_back(make_short_mat(q, !fast));
       } else if (fast && q.cols > 0 && q.dtype == WT_I8) {
         i8c[q.cols > 8 ? 1 : 0].push_back(q);
-        i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
-      } else if (fast && q.cols > 0) {
-        (cols_on_umma(q.dtype, q.cols) ? umma_dt : q.cols > 8 ? colsw_dt : cols_dt)[q.dtype].push_back(make_cols_mat(q));
+      } else if (fast && q.cols > 0 && q.dtype != WT_F32) {
+        (cols_forced() == 1 ? umma_dt : q.cols > 8 ? colsw_dt : cols_dt)[q.dtype].push_back(make_cols_mat(q));
       } else if (fast && q.dtype == WT_I8 && i8_onecol_on_mma((uint32_t)(q.K / 16))) {
         // y[M] is Y[1, M] and x[K] is X[1, K]: the one-column GEMV as a T = 1 tensor-core GEMV
         wt_gemv_desc q1 = q;
         q1.cols = 1;
         i8c[0].push_back(q1);
-        i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
       } else if (q.cols > 0 && q.dtype != WT_F32 && q.K * es < 0x7fffffffull) {
         (q.cols > 8 ? ragcw_dt : ragc_dt)[q.dtype].push_back(make_cols_mat(q, true));
       } else if (q.cols == 0 && (fast || q.K * es < 0x7fffffffull)) {
@@ -1706,14 +1811,26 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
                              static_cast<const uint8_t *>(q.scale), ncol});
       }
     }
-    if (!i8c[0].empty() || !i8c[1].empty()) {
-      const bool rows = i8_on_q8rows(i8_blocks);
-      for (int w = 0; w < 2; ++w)
-        for (const wt_gemv_desc &q : i8c[w]) {
-          if (!rows && cols_on_short(q, false)) short_dt[WT_I8][w].push_back(make_short_mat(q, false));
-          else (rows ? (w ? q8r_dt : q8r1_dt) : (w ? colsw_dt : cols_dt))[WT_I8].push_back(make_cols_mat(q));
-        }
+    for (int w = 0; w < 2; ++w) {
+      if (i8c[w].empty()) continue;
+      std::vector<wt::MatDesc> ms;
+      for (const wt_gemv_desc &q : i8c[w]) ms.push_back(make_cols_mat(q));
+      int grid = 0;
+      std::vector<wt::Piece> pieces;
+      std::vector<uint32_t> begin;
+      CostModel blocks;
+      blocks.block = wt::kQ8RowsBlock;
+      if (i8_on_q8rows(deal_tiles(ms, grid, pieces, begin, 2, blocks), w == 1)) {
+        (w ? q8r_dt : q8r1_dt)[WT_I8] = std::move(ms);
+        continue;
+      }
+      for (size_t k = 0; k < ms.size(); ++k) {
+        if (cols_on_short(i8c[w][k], false)) short_dt[WT_I8][w].push_back(make_short_mat(i8c[w][k], false));
+        else (w ? colsw_dt : cols_dt)[WT_I8].push_back(ms[k]);
+      }
     }
+    for (const int dt : {WT_BF16, WT_F16})
+      if (cols_on_umma(colsw_dt[dt])) std::swap(colsw_dt[dt], umma_dt[dt]);
     for (int pass = 0; pass < 14; ++pass) {
       for (int dt = 0; dt < 4; ++dt) {
         std::vector<wt::MatDesc> &ms = pass == 0   ? by_dt[dt]
@@ -1775,10 +1892,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           // row-owner int8 launch: pieces cut at 128-row blocks, two tensor maps per matrix
           L.q8rows = true;
           L.nt = pass == 8 ? 2 : 1;
-          CostModel cm;
-          cm.block = wt::kQ8RowsBlock;
-          cm.vecs = 192 / 16;
-          partition(ms, L.grid, pieces, begin, (uint32_t)wt::kQ8RowsBlock, 1, 2, cm);
+          deal_tiles(ms, L.grid, pieces, begin, 2, q8rows_cost());
           L.mats = append(P->table, ms);
           L.pieces = append(P->table, pieces);
           L.begin = append(P->table, begin);
@@ -1797,9 +1911,12 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
               return set_err(WT_ENOTSUP, "wt_pass: internal: a %u-vector row reached the TMA kernel unsegmented", m.V);
         for (const wt::MatDesc &m : ms) L.ragged |= m.rb != 0;
         L.nt = pass == 2 || pass == 6 ? 1 : pass == 5 || pass == 7 ? 2 : 0;
-        partition(ms, L.grid, pieces, begin, warp_mma ? (uint32_t)wt::kColTileRows : 1u,
-                  pass == 0 ? one_col_slices(dt) : 1,
-                  pass == 0 ? wt::gemv_ctas_per_sm(dt) : warp_mma ? wt::gemm_cols_ctas_per_sm(dt, L.nt) : 1);
+        if (warp_mma) {
+          deal_tiles(ms, L.grid, pieces, begin, wt::gemm_cols_ctas_per_sm(dt, L.nt), warp_mma_cost());
+        } else {
+          partition(ms, L.grid, pieces, begin, 1, pass == 0 ? one_col_slices(dt) : 1,
+                    pass == 0 ? wt::gemv_ctas_per_sm(dt) : 1);
+        }
         L.mapped_cols = pass == 4;
         L.mats = append(P->table, ms);
         if (pass == 0)
