@@ -349,6 +349,24 @@ def test_plain_digest_chunks(torch, sizes):
         assert got == [oracle.fnv1a64(data[off:off + n]) for n in sizes]
 
 
+@pytest.mark.parametrize("off", [0, 3])
+@pytest.mark.parametrize("leaves", [8192, 8193])
+def test_tree_digest_leaves_by_warps_and_by_threads(torch, off, leaves):
+    """Calls of 8192 leaves and fewer take a warp per leaf, larger ones a thread: lengths that end
+    in and around the 128-byte shares of a warp's lanes, and one buffer that makes up the count."""
+    rng = np.random.default_rng(21)
+    sizes = [1, 15, 16, 127, 128, 129, 255, 1000, 3968, 3969, 4095, 4096, 4097, 8191, 12288 + 130]
+    sizes.append(4096 * (leaves - sum(-(-n // 4096) for n in sizes)) - 77)
+    data = rng.integers(0, 256, sizes[-1], dtype=np.uint8)
+    buf = torch.zeros(data.size + 16, dtype=torch.uint8, device="cuda")
+    buf[off:off + data.size] = torch.from_numpy(data).cuda()
+    with wt.Handle([]) as h:
+        out = torch.zeros(len(sizes), dtype=torch.int64, device="cuda")
+        h.checksum([buf.data_ptr() + off] * len(sizes), sizes, out.data_ptr(), 0)
+        got = [int(v) & (2 ** 64 - 1) for v in out.cpu().tolist()]
+    assert got == [oracle.fnv_tree(data[:n]) for n in sizes]
+
+
 def test_unaligned_operands_take_the_generic_kernel(torch):
     """W and x 2 bytes past a 16-byte boundary (element-aligned only): the scalar fallback,
     checked against the oracle; one and several columns."""
