@@ -2528,9 +2528,11 @@ int wt_pass(wt_handle *h, const wt_gemv_desc *d, size_t n, void *stream) {
   if (h->host_only) return set_err(WT_ENOTSUP, "wt_pass: handle was opened host-only");
   if (n == 0) return WT_OK;
   if (!d) return set_err(WT_EINVAL, "wt_pass: NULL descriptors");
+  bool events = false;
   for (size_t i = 0; i < n; ++i) {
     int rc = validate_desc(d[i], i);
     if (rc) return rc;
+    events |= d[i].wait_event != nullptr;
     if (d[i].M && inside_mapping(h, d[i].y, d[i].M * std::max<int32_t>(1, d[i].cols) * sizeof(float)))
       return set_err(WT_EINVAL, "wt_pass: y of desc %zu lies inside a read-only mapping", i);
   }
@@ -2544,8 +2546,20 @@ int wt_pass(wt_handle *h, const wt_gemv_desc *d, size_t n, void *stream) {
   try {
     // Plans are keyed by the descriptors with each wait_event replaced by the ordinal of its
     // first appearance: calls that differ only in which events they wait on share one plan.
+    // Descriptors without events are their own key, and most calls repeat a recent plan's: those
+    // are compared in place.
+    if (!events)
+      for (auto it = h->plans.begin(); it != h->plans.end(); ++it) {
+        Plan *P = *it;
+        if (P->key.size() != n * sizeof(wt_gemv_desc) || memcmp(P->key.data(), d, P->key.size()) != 0) continue;
+        if (it != h->plans.begin()) {
+          h->plans.erase(it);
+          h->plans.push_front(P);
+        }
+        return run_plan(h, P, d, static_cast<cudaStream_t>(stream), capturing);
+      }
     std::vector<wt_gemv_desc> kd(d, d + n);
-    {
+    if (events) {
       std::vector<std::pair<uintptr_t, uintptr_t>> seen;  // (event, ordinal), sorted by event
       for (size_t i = 0; i < n; ++i) {
         const uintptr_t e = reinterpret_cast<uintptr_t>(d[i].wait_event);

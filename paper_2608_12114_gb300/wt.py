@@ -85,6 +85,7 @@ assert DESC_DTYPE.itemsize == C.sizeof(GemvDesc)
 
 
 _lib = None
+_pass_at = None
 ABI_VERSION = 4  # wt_abi_version() of the include/wt.h this binding follows
 
 
@@ -114,6 +115,9 @@ def lib(path: str = LIB_PATH):
     L.wt_file_registration.argtypes = [vp, sz, C.POINTER(C.c_uint)]
     L.wt_adopt.argtypes = [vp, vp, vp, sz, C.c_uint, vp, vp]
     L.wt_pass.argtypes = [vp, C.POINTER(GemvDesc), sz, vp]
+    global _pass_at
+    _pass_at = L["wt_pass"]  # a function object of its own: the descriptors' address as an integer
+    _pass_at.argtypes = [vp, vp, sz, vp]
     L.wt_checksum.argtypes = [vp, C.POINTER(vp), u64p, sz, vp, vp]
     L.wt_checksum_plain.argtypes = [vp, C.POINTER(vp), u64p, sz, vp, vp]
     L.wt_checksum_noalloc.argtypes = [C.POINTER(vp), u64p, sz, vp, vp]
@@ -289,14 +293,18 @@ class Handle:
     def pass_(self, descs, stream: int = 0):
         """wt_pass over a list of GemvDesc or a contiguous numpy array of DESC_DTYPE records."""
         if isinstance(descs, np.ndarray):
-            if descs.dtype != DESC_DTYPE or not descs.flags.c_contiguous:
+            # no ctypes objects on this path: a pass of small matrices is bound by its call
+            # (8 fp32 256 x 256 matrices: 5.1 us in this method with a cast pointer, 4.1 now)
+            t = descs.dtype
+            if (t is not DESC_DTYPE and t != DESC_DTYPE) or not descs.flags.c_contiguous:
                 raise ValueError("descriptor array must be a contiguous DESC_DTYPE array")
             n = descs.size
-            arr = C.cast(descs.ctypes.data if n else 0, C.POINTER(GemvDesc))
+            rc = _pass_at(self.ptr, descs.ctypes.data if n else 0, n, stream)
         else:
             n = len(descs)
-            arr = (GemvDesc * max(1, n))(*descs)
-        _check(lib().wt_pass(self.ptr, arr, n, C.c_void_p(stream)))
+            rc = lib().wt_pass(self.ptr, (GemvDesc * max(1, n))(*descs), n, C.c_void_p(stream))
+        if rc:
+            _check(rc)
 
     def checksum(self, ptrs: Sequence[int], nbytes: Sequence[int], out_dev: int, stream: int = 0,
                  plain: bool = False):
