@@ -102,7 +102,7 @@ struct ColX {
 
 template <int DT>
 __device__ __forceinline__ float col_scale(const uint8_t *s, uint64_t row) {
-  if constexpr (DT == 3) return __half2float(reinterpret_cast<const __half *>(s)[row]);
+  if constexpr (DT == 3) return s ? __half2float(reinterpret_cast<const __half *>(s)[row]) : 1.f;
   return 1.f;
 }
 
@@ -291,7 +291,7 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
         for (int n = 0; n < NT; ++n) {
           const uint32_t col = g + 8 * n;
           if constexpr (RAG) load_xvec_ragged<DT>(md, col, c * vc + v, v < nv && col < T, xr[q][n]);
-          else load_xvec<DT>(md.x, (uint64_t)col * V + (uint64_t)c * vc + v, v < nv && col < T, xr[q][n]);
+          else load_xvec<DT>(md.x, (uint64_t)col * md.rs + (uint64_t)c * vc + v, v < nv && col < T, xr[q][n]);
         }
       }
 #pragma unroll

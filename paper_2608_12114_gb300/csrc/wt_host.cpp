@@ -1265,6 +1265,33 @@ wt::MatDesc make_seg_mat(const wt_gemv_desc &d, uint32_t k, bool ragged) {
   return m;
 }
 
+// Multi-column matrices of few long rows (aligned): the warp-MMA kernel gives a 16-row tile to
+// one CTA, so 64 rows of 32768 elements kept 4 of 152 busy.  They run in column segments as the
+// one-column kernel's long rows do, as many as leave a CTA each a tile and 256 vectors or more.
+// The number depends on the matrix alone, so where a group has many of them the second pass comes
+// on top of full CTAs; from 3072 vectors on that costs nothing (bf16, T = 8, us without / with:
+// 64 x 32768 21 / 9.9, 64 of those 55 / 49, 1024 x 32768 25 / 22; but 16 of 128 x 16384 17.8 /
+// 20.0, 1024 x 8192 10.3 / 12.0).
+uint32_t cols_segments(const wt_gemv_desc &d) {
+  const uint64_t V = d.K * elem_bytes(d.dtype) / 16, tiles = (d.M + wt::kColTileRows - 1) / wt::kColTileRows;
+  if (V < 3072 || cols_forced() == 1 || cols_forced() == 3) return 1;
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(V / 256, (uint64_t)wt::num_sms() / tiles));
+}
+
+// Segment k of nseg (of nearly equal length, whole vectors) of such a matrix.
+wt::MatDesc make_cols_seg(const wt_gemv_desc &d, uint32_t k, uint32_t nseg) {
+  const int es = elem_bytes(d.dtype);
+  const uint64_t V = d.K * es / 16, v0 = V * k / nseg, v1 = V * (k + 1) / nseg;
+  wt_gemv_desc sd = d;
+  sd.W = static_cast<const uint8_t *>(d.W) + v0 * 16;
+  sd.x = static_cast<const uint8_t *>(d.x) + v0 * (d.dtype == WT_I8 ? 32 : 16);
+  sd.K = (v1 - v0) * 16 / es;
+  sd.scale = nullptr;
+  wt::MatDesc m = make_cols_mat(sd);
+  m.rs = (uint32_t)V;
+  return m;
+}
+
 // cuTensorMapEncodeTiled, looked up once through the runtime (no link against libcuda).
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                    const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -1290,7 +1317,7 @@ int encode_cols_map(const wt::MatDesc &m, uint8_t *out) {
   EncodeTiledFn fn = encode_tiled();
   if (!fn) return set_err(WT_ECUDA, "wt_pass: cuTensorMapEncodeTiled is not available from the driver");
   const cuuint64_t dims[2] = {(cuuint64_t)m.V * 2, (cuuint64_t)m.M};
-  const cuuint64_t strides[1] = {(cuuint64_t)m.V * 16};
+  const cuuint64_t strides[1] = {(cuuint64_t)m.rs * 16};
   const cuuint32_t box[2] = {m.vc * 2, (cuuint32_t)wt::kColTileRows};
   const cuuint32_t estr[2] = {1, 1};
   CUtensorMap map;
@@ -1705,6 +1732,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         q8r1_dt[4];  // row-owner int8 launches with two 8-column tiles (T > 8) and with one
     std::vector<wt_gemv_desc> i8c[2];  // int8 on the tensor cores, T <= 8 and T > 8: kernel chosen below
     std::vector<int64_t> seg_ws[4];  // per by_dt entry: workspace float offset of its partials, or -1
+    std::vector<std::pair<wt::MatDesc, size_t>> cseg_dt[4][2];  // multi-column segments [dtype][T > 8], likewise
     std::vector<wt::SegReduce> reds;
     std::vector<size_t> red_ws;      // per reds entry: workspace float offset
     RangeCache rcw, rcx, rcy, rcs;
@@ -1765,6 +1793,22 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         }
       } else if (q.cols > 0 && q.dtype != WT_F32 && cols_on_short(q, !fast) && (!fast || q.dtype != WT_I8 || q.K <= kI8ShortK)) {
         short_dt[q.dtype][(q.cols > 8) + 2 * !fast].push_back(make_short_mat(q, !fast));
+      } else if (fast && q.cols > 0 && q.dtype != WT_F32 && cols_segments(q) > 1) {
+        const uint32_t nseg = cols_segments(q);
+        const uint64_t outs = q.M * ncol;
+        const size_t off = P->ws_floats;
+        P->ws_floats += (size_t)nseg * outs;
+        for (uint32_t k = 0; k < nseg; ++k) cseg_dt[q.dtype][q.cols > 8].push_back({make_cols_seg(q, k, nseg), off + k * outs});
+        wt::SegReduce r;
+        memset(&r, 0, sizeof r);
+        r.y = q.y;
+        r.s = static_cast<const uint8_t *>(q.scale);
+        r.M = (uint32_t)outs;
+        r.nseg = nseg;
+        r.rows = (uint32_t)q.M;
+        reds.push_back(r);
+        red_ws.push_back(off);
+        g.reduce_rows = std::max(g.reduce_rows, (uint32_t)outs);
       } else if (fast && q.cols > 0 && q.dtype == WT_I8) {
         i8c[q.cols > 8 ? 1 : 0].push_back(q);
       } else if (fast && q.cols > 0 && q.dtype != WT_F32) {
@@ -1802,6 +1846,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           r.s = static_cast<const uint8_t *>(q.scale);
           r.M = (uint32_t)q.M;
           r.nseg = nseg;
+          r.rows = r.M;
           reds.push_back(r);
           red_ws.push_back(off);
           g.reduce_rows = std::max(g.reduce_rows, (uint32_t)q.M);
@@ -1829,8 +1874,18 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         else (w ? colsw_dt : cols_dt)[WT_I8].push_back(ms[k]);
       }
     }
+    std::vector<int64_t> cseg_ws[4][2];
     for (const int dt : {WT_BF16, WT_F16})
       if (cols_on_umma(colsw_dt[dt])) std::swap(colsw_dt[dt], umma_dt[dt]);
+    for (int dt = 0; dt < 4; ++dt)  // segments join their warp-MMA launch last
+      for (int w = 0; w < 2; ++w) {
+        std::vector<wt::MatDesc> &ms = (w ? colsw_dt : cols_dt)[dt];
+        cseg_ws[dt][w].assign(ms.size(), -1);
+        for (const auto &sg : cseg_dt[dt][w]) {
+          ms.push_back(sg.first);
+          cseg_ws[dt][w].push_back((int64_t)sg.second);
+        }
+      }
     for (int pass = 0; pass < 14; ++pass) {
       for (int dt = 0; dt < 4; ++dt) {
         std::vector<wt::MatDesc> &ms = pass == 0   ? by_dt[dt]
@@ -1919,10 +1974,10 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         }
         L.mapped_cols = pass == 4;
         L.mats = append(P->table, ms);
-        if (pass == 0)
-          for (size_t k = 0; k < ms.size(); ++k)
-            if (seg_ws[dt][k] >= 0)
-              P->ws_patches.push_back({L.mats + k * sizeof(wt::MatDesc) + offsetof(wt::MatDesc, y), (size_t)seg_ws[dt][k]});
+        const std::vector<int64_t> *ws = pass == 0 ? &seg_ws[dt] : pass == 2 || pass == 5 ? &cseg_ws[dt][pass == 5] : nullptr;
+        for (size_t k = 0; ws && k < ms.size(); ++k)
+          if ((*ws)[k] >= 0)
+            P->ws_patches.push_back({L.mats + k * sizeof(wt::MatDesc) + offsetof(wt::MatDesc, y), (size_t)(*ws)[k]});
         L.pieces = append(P->table, pieces);
         L.begin = append(P->table, begin);
         if (warp_mma && !L.ragged) {
@@ -2062,10 +2117,6 @@ int run_plan(wt_handle *h, Plan *P, const wt_gemv_desc *d, cudaStream_t s, bool 
       CU(wt::launch_gemv(gl, s));
       h->kernel_launches++;
     }
-    if (g.n_reduce) {
-      CU(wt::launch_seg_reduce(reinterpret_cast<const wt::SegReduce *>(P->dev + g.reduce), g.n_reduce, g.reduce_rows, s));
-      h->kernel_launches++;
-    }
     for (const Plan::Launch &L : g.mapped) {
       wt::GemvLaunch gl;
       gl.dtype = L.dtype;
@@ -2106,6 +2157,10 @@ int run_plan(wt_handle *h, Plan *P, const wt_gemv_desc *d, cudaStream_t s, bool 
       } else {
         CU(wt::launch_gemm_cols(gl, s));
       }
+      h->kernel_launches++;
+    }
+    if (g.n_reduce) {
+      CU(wt::launch_seg_reduce(reinterpret_cast<const wt::SegReduce *>(P->dev + g.reduce), g.n_reduce, g.reduce_rows, s));
       h->kernel_launches++;
     }
     for (const Plan::Generic &q : g.generic) {

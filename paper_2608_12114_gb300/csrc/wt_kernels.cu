@@ -1049,7 +1049,7 @@ __global__ void seg_reduce_kernel(const SegReduce *__restrict__ tab) {
   if (row >= r.M) return;
   float sum = 0.f;
   for (uint32_t k = 0; k < r.nseg; ++k) sum += r.ws[(uint64_t)k * r.M + row];
-  r.y[row] = r.s ? sum * __half2float(reinterpret_cast<const __half *>(r.s)[row]) : sum;
+  r.y[row] = r.s ? sum * __half2float(reinterpret_cast<const __half *>(r.s)[row % r.rows]) : sum;
 }
 
 }  // namespace

@@ -87,8 +87,10 @@ struct alignas(16) SegReduce {
   const float *ws;   // nseg x M partial sums (segment-major)
   float *y;          // M outputs
   const uint8_t *s;  // f16 row scales (int8 weights) or null
-  uint32_t M;
+  uint32_t M;        // outputs: rows, or rows x T columns
   uint32_t nseg;
+  uint32_t rows;     // rows (outputs M = rows x T, one column after another)
+  uint32_t pad[3];
 };
 
 // y[row] = (sum over segments of ws[seg * M + row], in segment order) * scale[row], for

@@ -257,3 +257,24 @@ def test_cols_map_endpoint_bf16_and_f16(torch, tmp_path):
                 assert oracle.gemv_error(Y.cpu().numpy().astype(np.float64), Yhat.reshape(-1), A.reshape(-1)) <= TOL
             assert h.device_status() == 0
         co.close()
+
+
+@pytest.mark.parametrize("T", [1, 8, 9, 16])
+def test_cols_few_long_rows(torch, T):
+    """Rows of 3072 vectors and more in few tiles (column segments and a second pass), one vector
+    below that, and one tile more than still leaves two segments: against the oracle, alone and
+    grouped the same bits."""
+    rng = np.random.default_rng(300 + T)
+    shapes = [(BF16, 1, 24576), (BF16, 64, 32768), (F16, 17, 24584), (F16, 40, 24568), (I8, 33, 49168), (I8, 130, 49152),
+              (BF16, 600, 24576), (BF16, 1217, 24576)]
+    cases = [make(torch, rng, d, M, K, T) for d, M, K in shapes]
+    with wt.Handle([]) as h:
+        h.pass_([desc(c) for c in cases], 0)
+        torch.cuda.synchronize()
+        assert h.device_status() == 0
+        for c in cases:
+            check(c, c["Y"])
+            y2 = torch.full_like(c["Y"], float("nan"))
+            h.pass_([desc(c, y2)], 0)
+            torch.cuda.synchronize()
+            assert torch.equal(y2, c["Y"]), (c["dtype"], c["M"], c["K"])
