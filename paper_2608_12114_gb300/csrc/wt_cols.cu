@@ -30,8 +30,9 @@
 // meet the fp32 sums in ordinary additions: the tensor cores' own accumulation truncates, and
 // these calls had fp32 FMAs before (error against 64 bits, rows of 2731: 9.6e-8 bf16, 9.8e-8 int8,
 // 1.1e-7 f16 at T = 16, against 8.5e-8, 8.7e-8 and 1.7e-7).  Eight bf16 16384 x 2731 matrices at
-// T = 8 take 250 us (2884 GB/s; bound by the instructions of putting vectors together), and took
-// 1940 us with byte loads, one warp per row and the row read again for every column.
+// T = 8 take 197 us (3658 GB/s, two CTAs per SM; 250 with one: bound by the latencies of putting
+// vectors together), and took 1940 us with byte loads, one warp per row and the row read again for
+// every column.
 //
 // Why warp-level MMAs and not tcgen05: the A operand is decoded from int8 in registers and
 // goes to the MMA from there; tcgen05 takes A only from shared or tensor memory, which would
@@ -60,9 +61,9 @@ constexpr uint32_t kColStageBytes = kColRows * kColVecMax * 16;
 static_assert(kColVecMax % 8 == 4, "row pitch 64 bytes past a multiple of 128");
 static_assert(kColStageBytes % 128 == 0, "stages stay 128-byte aligned for the tensor copies");
 
-// Per-launch geometry: NT = 8-column MMA tiles (T <= 8: 1, else 2).  int8 weights run two
-// CTAs per SM with half the ring each (the same bytes in flight per SM, twice the warps; the
-// int8 path is latency-bound on its decode).  The cross-warp partials of one 16-row tile take
+// Per-launch geometry: NT = 8-column MMA tiles (T <= 8: 1, else 2).  int8 weights and
+// ragged operands run two CTAs per SM with half the ring each (the same bytes in flight per SM,
+// twice the warps; those paths are latency-bound on decoding and on shifting).  The cross-warp partials of one 16-row tile take
 // 16 x 8 NT floats per warp, in two alternating halves.
 // Where a partial sum of (column, row) sits among its tile's: a pair of columns takes 32 floats,
 // turned by 8 per pair, so that neither the stores of a fragment (rows g of the columns 2t; in
@@ -73,12 +74,12 @@ __device__ __forceinline__ uint32_t red_at(uint32_t col, uint32_t row) {
 
 template <int DT, int NT, bool RAG = false>
 struct ColGeo {
-  static constexpr int kCtasPerSm = DT == 3 ? 2 : 1;
+  static constexpr int kCtasPerSm = DT == 3 || RAG ? 2 : 1;
   static constexpr int kStages = kCtasPerSm == 2 ? 3 : 6;
   // 16-row tiles per super block (X registers are loaded once per super block and chunk):
   // four, or two for int8 with 16 columns, which then fits two CTAs per SM (registers and
   // partial buffers halve; X is reloaded every 32 rows instead of 64)
-  static constexpr int kBlocks = DT == 3 && NT == 2 ? 2 : 4;
+  static constexpr int kBlocks = kCtasPerSm == 2 && NT == 2 ? 2 : 4;
   // accumulator sets per tile (even / odd k16 steps: shorter MMA chains); int8 with 16
   // columns keeps one, its two column tiles already give two independent chains per A
   static constexpr int kAcc = RAG || (DT == 3 && NT == 2) ? 1 : 2;
@@ -91,7 +92,8 @@ struct ColGeo {
   static constexpr size_t kSmem = kFlagOff + 16;
 };
 static_assert(ColGeo<1, 2>::kSmem <= 232448 && 2 * (ColGeo<3, 1>::kSmem + 1024) <= 233472 &&
-                  2 * (ColGeo<3, 2>::kSmem + 1024) <= 233472,
+                  2 * (ColGeo<3, 2>::kSmem + 1024) <= 233472 && 2 * (ColGeo<1, 1, true>::kSmem + 1024) <= 233472 &&
+                  2 * (ColGeo<1, 2, true>::kSmem + 1024) <= 233472,
               "multi-column shared memory");
 
 // 32-bit words of X per weight vector: 16 fp16 activations for an int8 vector, else 8.
@@ -102,7 +104,7 @@ struct ColX {
 
 template <int DT>
 __device__ __forceinline__ float col_scale(const uint8_t *s, uint64_t row) {
-  if constexpr (DT == 3) return s ? __half2float(reinterpret_cast<const __half *>(s)[row]) : 1.f;
+  if constexpr (DT == 3) return __half2float(reinterpret_cast<const __half *>(s)[row]);
   return 1.f;
 }
 
@@ -265,6 +267,9 @@ template <int DT, int NT, bool RAG>
 __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, const Ring &R, float *red_base,
                                            uint32_t &it, uint32_t &par, int warp, int lane) {
   const uint32_t V = md.V, vc = md.vc, T = md.G;
+  // vectors from one column of X to the next: the whole row of a column segment; int8 has no
+  // segments (96 registers: the second length cost its T = 16 kernel 12 %)
+  const uint32_t xpitch = DT == 3 ? V : md.rs;
   const uint32_t nchunk = (V + vc - 1) / vc;
   const uint32_t g = lane >> 2, t = lane & 3;
   const int ct = threadIdx.x;
@@ -291,7 +296,7 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
         for (int n = 0; n < NT; ++n) {
           const uint32_t col = g + 8 * n;
           if constexpr (RAG) load_xvec_ragged<DT>(md, col, c * vc + v, v < nv && col < T, xr[q][n]);
-          else load_xvec<DT>(md.x, (uint64_t)col * md.rs + (uint64_t)c * vc + v, v < nv && col < T, xr[q][n]);
+          else load_xvec<DT>(md.x, (uint64_t)col * xpitch + (uint64_t)c * vc + v, v < nv && col < T, xr[q][n]);
         }
       }
 #pragma unroll
@@ -437,16 +442,15 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG>::kCtasPerSm)
 
 }  // namespace
 
-int gemm_cols_ctas_per_sm(int dtype, int nt) { return dtype == 3 ? 2 : 1; }
+int gemm_cols_ctas_per_sm(int dtype, bool ragged) { return dtype == 3 || ragged ? 2 : 1; }
 
 template <int DT, int NT>
 static cudaError_t cols_attr() {
-  static_assert(ColGeo<DT, NT>::kSmem == ColGeo<DT, NT, true>::kSmem, "one geometry");
   const cudaError_t e = cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ColGeo<DT, NT>::kSmem);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)ColGeo<DT, NT>::kSmem);
+                              (int)ColGeo<DT, NT, true>::kSmem);
 }
 
 cudaError_t gemm_cols_prepare() {
@@ -460,11 +464,12 @@ cudaError_t gemm_cols_prepare() {
 
 template <int DT, int NT>
 static void cols_launch(const GemvLaunch &L, cudaStream_t s) {
-  constexpr size_t smem = ColGeo<DT, NT>::kSmem;
   if (L.ragged)
-    gemm_cols_kernel<DT, NT, true><<<L.grid, kColThreads, smem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
+    gemm_cols_kernel<DT, NT, true>
+        <<<L.grid, kColThreads, ColGeo<DT, NT, true>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
   else
-    gemm_cols_kernel<DT, NT, false><<<L.grid, kColThreads, smem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
+    gemm_cols_kernel<DT, NT, false>
+        <<<L.grid, kColThreads, ColGeo<DT, NT>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
 }
 
 cudaError_t launch_gemm_cols(const GemvLaunch &L, cudaStream_t s) {

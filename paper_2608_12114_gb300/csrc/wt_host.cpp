@@ -1265,7 +1265,7 @@ wt::MatDesc make_seg_mat(const wt_gemv_desc &d, uint32_t k, bool ragged) {
   return m;
 }
 
-// Multi-column matrices of few long rows (aligned): the warp-MMA kernel gives a 16-row tile to
+// Multi-column matrices of few long rows (aligned, 2-byte weights): the warp-MMA kernel gives a 16-row tile to
 // one CTA, so 64 rows of 32768 elements kept 4 of 152 busy.  They run in column segments as the
 // one-column kernel's long rows do, as many as leave a CTA each a tile and 256 vectors or more.
 // The number depends on the matrix alone, so where a group has many of them the second pass comes
@@ -1274,7 +1274,7 @@ wt::MatDesc make_seg_mat(const wt_gemv_desc &d, uint32_t k, bool ragged) {
 // 20.0, 1024 x 8192 10.3 / 12.0).
 uint32_t cols_segments(const wt_gemv_desc &d) {
   const uint64_t V = d.K * elem_bytes(d.dtype) / 16, tiles = (d.M + wt::kColTileRows - 1) / wt::kColTileRows;
-  if (V < 3072 || cols_forced() == 1 || cols_forced() == 3) return 1;
+  if (V < 3072 || d.dtype == WT_I8 || cols_forced() == 1 || cols_forced() == 3) return 1;
   return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(V / 256, (uint64_t)wt::num_sms() / tiles));
 }
 
@@ -1531,6 +1531,8 @@ double deal_tiles(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<w
   const uint64_t cheapest = cost.row(mats[order.back()]) * cost.block;
   uint64_t last = 0;  // tile cost of the previous matrix: its CTAs are full up to `c` for this one
   int c = 0;
+  std::vector<std::pair<int64_t, int>> by_left(grid);
+  uint64_t heap_tc = 0;  // by_left is a heap of -left for tiles of this cost
   int64_t lack = 0;  // cheapest tiles: what CTAs up to c lack beyond the tiles dealt so far
   for (const uint32_t i : order) {
     const wt::MatDesc &m = mats[i];
@@ -1567,9 +1569,11 @@ double deal_tiles(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<w
       if (r == m.M) break;  // the next matrix of this tile cost goes on here
     }
     if (r < m.M) {  // no CTA has room for a whole tile: one each to those with the most left
-      std::vector<std::pair<int64_t, int>> by_left(grid);
-      for (int k = 0; k < grid; ++k) by_left[k] = {-left[k], k};
-      std::make_heap(by_left.begin(), by_left.end(), std::greater<std::pair<int64_t, int>>());
+      if (heap_tc != tc) {  // matrices of one tile cost in a row share the heap
+        for (int k = 0; k < grid; ++k) by_left[k] = {-left[k], k};
+        std::make_heap(by_left.begin(), by_left.end(), std::greater<std::pair<int64_t, int>>());
+        heap_tc = tc;
+      }
       while (r < m.M) {
         std::pop_heap(by_left.begin(), by_left.end(), std::greater<std::pair<int64_t, int>>());
         give(by_left.back().second, 1);
@@ -1586,6 +1590,16 @@ double deal_tiles(const std::vector<wt::MatDesc> &mats, int &grid, std::vector<w
   for (const auto &d : dealt) pieces[at[d.first]++] = d.second;
   const int64_t most = (int64_t)((C + grid - 1) / grid) - *std::min_element(left.begin(), left.end());
   return (double)most * grid / (double)std::max<uint64_t>(1, B);
+}
+
+// A lower bound of it: the dearest tile alone.
+double largest_tile_share(const std::vector<wt::MatDesc> &mats, int ctas_per_sm, const CostModel &cost) {
+  uint64_t B = 0, most = 0;
+  for (const wt::MatDesc &m : mats) {
+    B += (uint64_t)m.M * m.V * 16;
+    most = std::max(most, cost.row(m) * cost.block);
+  }
+  return (double)most * max_grid(B, ctas_per_sm) / (double)std::max<uint64_t>(1, B);
 }
 
 // 2-byte weights with more than 8 columns run on the warp-level MMA kernel (wt_cols.cu), or on
@@ -1865,7 +1879,10 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
       std::vector<uint32_t> begin;
       CostModel blocks;
       blocks.block = wt::kQ8RowsBlock;
-      if (i8_on_q8rows(deal_tiles(ms, grid, pieces, begin, 2, blocks), w == 1)) {
+      // a block that is itself above the limit settles it without dealing
+      double share = largest_tile_share(ms, 2, blocks);
+      if (cols_forced() == 0 && i8_on_q8rows(share, w == 1)) share = deal_tiles(ms, grid, pieces, begin, 2, blocks);
+      if (i8_on_q8rows(share, w == 1)) {
         (w ? q8r_dt : q8r1_dt)[WT_I8] = std::move(ms);
         continue;
       }
@@ -1967,7 +1984,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         for (const wt::MatDesc &m : ms) L.ragged |= m.rb != 0;
         L.nt = pass == 2 || pass == 6 ? 1 : pass == 5 || pass == 7 ? 2 : 0;
         if (warp_mma) {
-          deal_tiles(ms, L.grid, pieces, begin, wt::gemm_cols_ctas_per_sm(dt, L.nt), warp_mma_cost());
+          deal_tiles(ms, L.grid, pieces, begin, wt::gemm_cols_ctas_per_sm(dt, L.ragged), warp_mma_cost());
         } else {
           partition(ms, L.grid, pieces, begin, 1, pass == 0 ? one_col_slices(dt) : 1,
                     pass == 0 ? wt::gemv_ctas_per_sm(dt) : 1);

@@ -161,7 +161,7 @@ cudaError_t launch_gemv_mapped_cols(const GemvLaunch &L, cudaStream_t s);
 // 8 < T <= 16); int8 with nt = 1 runs two CTAs per SM (gemm_cols_ctas_per_sm).
 cudaError_t gemm_cols_prepare();
 cudaError_t launch_gemm_cols(const GemvLaunch &L, cudaStream_t s);
-int gemm_cols_ctas_per_sm(int dtype, int nt);
+int gemm_cols_ctas_per_sm(int dtype, bool ragged);
 
 // The same for short rows (wt_colshort.cu), at most short_row_bytes each: stages of whole rows,
 // rt of them (32 KB, less kRaggedSlack for ragged ones).  One launch

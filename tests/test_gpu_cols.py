@@ -261,8 +261,8 @@ def test_cols_map_endpoint_bf16_and_f16(torch, tmp_path):
 
 @pytest.mark.parametrize("T", [1, 8, 9, 16])
 def test_cols_few_long_rows(torch, T):
-    """Rows of 3072 vectors and more in few tiles (column segments and a second pass), one vector
-    below that, and one tile more than still leaves two segments: against the oracle, alone and
+    """Rows of 3072 vectors and more in few tiles (2-byte weights: column segments and a second
+    pass; int8: not segmented), one vector below that, and one tile more than still leaves two segments: against the oracle, alone and
     grouped the same bits."""
     rng = np.random.default_rng(300 + T)
     shapes = [(BF16, 1, 24576), (BF16, 64, 32768), (F16, 17, 24584), (F16, 40, 24568), (I8, 33, 49168), (I8, 130, 49152),
