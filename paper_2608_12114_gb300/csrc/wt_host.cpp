@@ -1834,10 +1834,12 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         i8c[0].push_back(q1);
       } else if (q.cols > 0 && q.dtype != WT_F32 && q.K * es < 0x7fffffffull) {
         (q.cols > 8 ? ragcw_dt : ragc_dt)[q.dtype].push_back(make_cols_mat(q, true));
-      } else if (q.cols == 0 && (fast || q.K * es < 0x7fffffffull)) {
-        // device memory, one column: whole 16-byte vectors per row, or ragged rows (any K, W
-        // and x at any byte), which the one-warp-per-row kernel streamed at 500 to 2500 GB/s
-        // and the phase rows stream at 4000 to 6900
+      } else if (q.cols == 0 && (fast || (q.K * es < 0x7fffffffull && reinterpret_cast<uintptr_t>(q.W) % es == 0))) {
+        // device memory, one column: whole 16-byte vectors per row, or ragged rows (any K, W on
+        // an element boundary, x at any byte), which the one-warp-per-row kernel streamed at 500
+        // to 2500 GB/s and the phase rows stream at 4000 to 6900.  W off its element size stays
+        // on that kernel: the phase rows multiply the aligned 16- or 32-bit lanes of W's vectors,
+        // which would hold halves of two elements.
         const uint32_t V = (uint32_t)((q.K * es + 15) / 16);
         if (V <= seg_max(q.dtype, !fast)) {
           wt::MatDesc m = make_mat(q);

@@ -1,5 +1,5 @@
-"""Rows off the 16-byte grid: K of any length, W and x at any byte, in every element type, on
-the tiled kernels; against the oracle."""
+"""Rows off the 16-byte grid: K of any length, in every element type, on the tiled kernels, and
+operands at any byte; against the oracle."""
 import numpy as np
 import pytest
 
@@ -123,3 +123,34 @@ def test_ragged_columns_against_oracle(torch, dtype, T):
             h.pass_([wt.gemv_desc(wp, dtype, M, K, xp, y2.data_ptr(), scale=sp, cols=T)], 0)
             assert torch.equal(y2, y), (dtype, M, K, T)
         assert h.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", [F32, BF16, F16, I8])
+@pytest.mark.parametrize("T", [0, 3, 16])
+def test_operands_off_their_element_size(torch, dtype, T):
+    """W and x at any byte, elements across the boundaries of every load: short rows, whole rows
+    and rows long enough for column segments, one column and several (no f32)."""
+    if T and dtype == F32:
+        pytest.skip("f32 weights have one column")
+    rng = np.random.default_rng(17 * dtype + T)
+    es = ES[dtype]
+    cs = []
+    for wo, xo in ((1, 0), (2, 1), (3, 3), (15, 0), (0, 1), (16, 7)):
+        for M, kb in ((9, 20), (33, 256), (70, 1028), (50, 2732), (21, 8064), (19, 12300)):
+            K = kb // es
+            W, X = weights(rng, dtype, M * K), weights(rng, F16 if dtype == I8 else dtype, max(1, T) * K)
+            s = rng.uniform(0.001, 0.02, M).astype(np.float16).view(np.uint8) if dtype == I8 else None
+            wb, wp = at(torch, W, wo)
+            xb, xp = at(torch, X, xo)
+            sb, sp = at(torch, s, 0) if s is not None else (None, 0)
+            y = torch.full((max(1, T) * M,), float("nan"), dtype=torch.float32, device="cuda")
+            ref = oracle.gemv_cols(W, dtype, M, K, X, T, scale=s) if T else \
+                oracle.gemv_q8(W, s, M, K, X) if dtype == I8 else oracle.gemv(W, dtype, M, K, X)
+            cs.append((wt.gemv_desc(wp, dtype, M, K, xp, y.data_ptr(), scale=sp, cols=T), M, K, wo, xo, y, ref, (wb, xb, sb)))
+    with wt.Handle([]) as h:
+        h.pass_([c[0] for c in cs], 0)
+        torch.cuda.synchronize()
+        assert h.device_status() == 0
+    for _, M, K, wo, xo, y, (yhat, a), _ in cs:
+        err = oracle.gemv_error(y.cpu().numpy(), yhat.reshape(-1), a.reshape(-1))
+        assert err <= (2 if T else 1) * bound(K), (dtype, M, K, T, wo, xo, err)
