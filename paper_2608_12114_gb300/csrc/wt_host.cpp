@@ -1265,6 +1265,23 @@ wt::MatDesc make_seg_mat(const wt_gemv_desc &d, uint32_t k, bool ragged) {
   return m;
 }
 
+// 2-byte weights with more than 8 columns run on the warp-level MMA kernel (wt_cols.cu), or on
+// tcgen05 (wt_umma.cu) where a matrix has at least 16384 rows of at most 3072 bytes.  The choice
+// is by the matrix alone: the kernels round differently, and a row's bits do not depend on what
+// else its launch holds.  tcgen05 keeps the rate of HBM at any T and K where the warp-MMA kernel
+// spends its chunks' latencies on little work (T = 16, bf16, us on tcgen05 / warp-MMA, 1 GiB of
+// 16384-row matrices: K = 576 183 / 223, 768 174 / 259, 1024 167 / 208, 1536 162 / 192; 2048 163 / 170,
+// 4096 161 / 164, 8192 184 / 163), but it deals whole 128-row tiles, and a launch waits for the CTA
+// with one more (alone, K = 1024: 4096 rows 10.6 / 8.4, 8192 11.0 / 10.5, 16384 12.4 / 12.6, 20480
+// 18.5 / 15.4, 32768 18.6 / 20.6, 65536 29 / 33; K = 4096: 4096 rows 27 / 13, 65536 93 / 85).  Up to
+// 8 columns the warp-MMA kernel is the faster throughout.  WT_COLS_KERNEL=mma or =umma forces
+// one kernel (umma still only for 2-byte weights).
+bool cols_on_umma(const wt_gemv_desc &d) {
+  const int f = cols_forced();
+  if (f == 1 || f == 2) return f == 1;
+  return d.cols > 8 && d.M >= 16384 && d.K * elem_bytes(d.dtype) <= 3072;
+}
+
 // Multi-column matrices of few long rows (aligned, 2-byte weights): the warp-MMA kernel gives a 16-row tile to
 // one CTA, so 64 rows of 32768 elements kept 4 of 152 busy.  They run in column segments as the
 // one-column kernel's long rows do, as many as leave a CTA each a tile and 256 vectors or more.
@@ -1602,21 +1619,6 @@ double largest_tile_share(const std::vector<wt::MatDesc> &mats, int ctas_per_sm,
   return (double)most * max_grid(B, ctas_per_sm) / (double)std::max<uint64_t>(1, B);
 }
 
-// 2-byte weights with more than 8 columns run on the warp-level MMA kernel (wt_cols.cu), or on
-// tcgen05 (wt_umma.cu) where a launch has at least 16 of its 128-row tiles per SM.  tcgen05 keeps
-// the rate of HBM at any T but deals whole tiles, and a launch waits for the CTA with one more
-// (T = 16, bf16, us on tcgen05 / warp-MMA: the large decoder, 84 tiles per SM: 2441 / 2533;
-// 65536 x 1024 x 8, 27: 170 / 211; 8192 x 4096 x 16, 6.7: 167 / 165; two large layers, 4.4:
-// 173 / 141; four mid layers 137 / 105; 4096 x 4096: 27 / 12).  Up to 8 columns the warp-MMA
-// kernel is the faster throughout.  WT_COLS_KERNEL=mma or =umma forces one kernel (umma still
-// only for 2-byte weights).
-bool cols_on_umma(const std::vector<wt::MatDesc> &ms) {
-  const int f = cols_forced();
-  uint64_t tiles = 0;
-  for (const wt::MatDesc &m : ms) tiles += (m.M + 127) / 128;
-  return f != 2 && tiles >= 16ull * wt::num_sms();
-}
-
 // int8 weights on the tensor cores (T columns, and one column with rows up to K = 8192) run
 // the row-owner kernel (wt_q8rows.cu) unless its 128-row blocks leave the CTAs uneven: its
 // warps keep no activation registers and meet in no reduction, but a launch waits for the CTA
@@ -1826,7 +1828,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
       } else if (fast && q.cols > 0 && q.dtype == WT_I8) {
         i8c[q.cols > 8 ? 1 : 0].push_back(q);
       } else if (fast && q.cols > 0 && q.dtype != WT_F32) {
-        (cols_forced() == 1 ? umma_dt : q.cols > 8 ? colsw_dt : cols_dt)[q.dtype].push_back(make_cols_mat(q));
+        (cols_on_umma(q) ? umma_dt : q.cols > 8 ? colsw_dt : cols_dt)[q.dtype].push_back(make_cols_mat(q));
       } else if (fast && q.dtype == WT_I8 && i8_onecol_on_mma((uint32_t)(q.K / 16))) {
         // y[M] is Y[1, M] and x[K] is X[1, K]: the one-column GEMV as a T = 1 tensor-core GEMV
         wt_gemv_desc q1 = q;
@@ -1894,8 +1896,6 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
       }
     }
     std::vector<int64_t> cseg_ws[4][2];
-    for (const int dt : {WT_BF16, WT_F16})
-      if (cols_on_umma(colsw_dt[dt])) std::swap(colsw_dt[dt], umma_dt[dt]);
     for (int dt = 0; dt < 4; ++dt)  // segments join their warp-MMA launch last
       for (int w = 0; w < 2; ++w) {
         std::vector<wt::MatDesc> &ms = (w ? colsw_dt : cols_dt)[dt];

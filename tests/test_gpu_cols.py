@@ -278,3 +278,33 @@ def test_cols_few_long_rows(torch, T):
             h.pass_([desc(c, y2)], 0)
             torch.cuda.synchronize()
             assert torch.equal(y2, c["Y"]), (c["dtype"], c["M"], c["K"])
+
+
+@pytest.mark.parametrize("T", [9, 16])
+def test_cols_bits_do_not_depend_on_the_launch(torch, T):
+    """2-byte weights with more than 8 columns: matrices on each side of the line between the
+    warp-MMA and the tcgen05 kernel (16384 rows, 3072 bytes) give the same bits alone and beside
+    a matrix that makes the launch a large one (2432 tiles of 128 rows), and the right ones."""
+    g = torch.Generator("cuda").manual_seed(40 + T)
+    shapes = [(64, 1024), (16383, 1024), (16384, 1024), (16384, 1536), (16384, 1544), (20480, 776)]
+    big = (311296, 520)
+    with wt.Handle([]) as h:
+        for dtype, tdt in ((BF16, torch.bfloat16), (F16, torch.float16)):
+            Ws = [torch.empty(M, K, dtype=tdt, device="cuda").normal_(0, 0.02, generator=g) for M, K in shapes + [big]]
+            Xs = [torch.empty(T, K, dtype=tdt, device="cuda").normal_(0, 1, generator=g) for _, K in shapes + [big]]
+            run = lambda which: [torch.full((T * Ws[i].shape[0],), float("nan"), device="cuda") for i in which]  # noqa: E731
+            ds = lambda which, ys: [wt.gemv_desc(Ws[i].data_ptr(), dtype, *Ws[i].shape, Xs[i].data_ptr(), y.data_ptr(),  # noqa: E731
+                                                 cols=T) for i, y in zip(which, ys)]
+            every = list(range(len(Ws)))
+            together = run(every)
+            h.pass_(ds(every, together), 0)
+            for i in every:
+                alone = run([i])
+                h.pass_(ds([i], alone), 0)
+                torch.cuda.synchronize()
+                assert torch.equal(alone[0], together[i]), (dtype, T, tuple(Ws[i].shape))
+                if i < len(shapes):
+                    ref = Xs[i].double() @ Ws[i].double().t()
+                    mag = Xs[i].double().abs() @ Ws[i].double().abs().t()
+                    assert ((alone[0].view(T, -1).double() - ref).abs() <= TOL * mag).all()
+            assert h.device_status() == 0
