@@ -26,14 +26,14 @@
 // Ragged operands (RAG: rows of W or X that are no whole number of 16-byte vectors, or W or X
 // off a 16-byte boundary): no tensor map can describe such rows, so each lane of the producer
 // warp brings one row's share of a chunk by a 1-D copy, and every weight and X vector is put
-// together from the two 16-byte vectors that hold it.  Each vector's MMAs start from zero and
-// meet the fp32 sums in ordinary additions: the tensor cores' own accumulation truncates, and
-// these calls had fp32 FMAs before (error against 64 bits, then / now: rows of 2731 bf16 8.5e-8 /
-// 9.1e-8, int8 8.7e-8 / 9.6e-8, f16 at T = 16 1.7e-7 / 1.1e-7; rows of 20001 bf16 1.9e-7 / 1.4e-7;
-// adding every MMA by itself 1.1e-7, every stage 1.1e-7).  Eight bf16 16384 x 2731 matrices at
-// T = 8 take 197 us (3658 GB/s, two CTAs per SM; 250 with one: bound by the latencies of putting
-// vectors together), and took 1940 us with byte loads, one warp per row and the row read again for
-// every column.
+// together from the two 16-byte vectors that hold it.  These calls had fp32 FMAs before, one warp
+// per row, and the tensor cores truncate what they accumulate, so every MMA has a second one that
+// brings back what the first dropped (mma16816_kept).  Error against 64 bits at T = 8, with FMAs /
+// with one MMA / now: rows of 1027 bf16 6.9e-8 / 7.9e-8 / 5.6e-8, int8 7.2e-8 / 8.9e-8 / 6.2e-8; rows of
+// 2731 bf16 8.5e-8 / 9.1e-8 / 5.6e-8, int8 8.7e-8 / 9.6e-8 / 6.1e-8, f16 1.7e-7 / 1.1e-7 / 6.0e-8.  Eight 16384 x 2731
+// matrices at T = 8 / 16, with FMAs / with one MMA / now: bf16 1924, 4011 / 198, 341 / 217, 448 us, int8
+// 1532, 3097 / 141, 321 / 192, 433 us (bf16 T = 8: 3310 GB/s, two CTAs per SM, bound by the latencies of
+// putting vectors together; 16 columns on one CTA per SM with twice the registers 594 and 495 us).
 //
 // Why warp-level MMAs and not tcgen05: the A operand is decoded from int8 in registers and
 // goes to the MMA from there; tcgen05 takes A only from shared or tensor memory, which would
@@ -81,10 +81,10 @@ struct ColGeo {
   // four, or two for int8 with 16 columns, which then fits two CTAs per SM (registers and
   // partial buffers halve; X is reloaded every 32 rows instead of 64)
   static constexpr int kBlocks = kCtasPerSm == 2 && NT == 2 ? 2 : 4;
-  // accumulator sets per tile (even / odd k16 steps: shorter MMA chains; ragged
-  // operands: even / odd vectors, shorter chains of fp32 additions); int8 and ragged with 16
-  // columns keep one, its two column tiles already give two independent chains per A
-  static constexpr int kAcc = NT == 2 && (DT == 3 || RAG) ? 1 : 2;
+  // accumulator sets per tile (even / odd k16 steps: shorter MMA chains; ragged operands: the
+  // sums and what they lost); int8 with 16 columns keeps one, its two column tiles already give
+  // two independent chains per A
+  static constexpr int kAcc = NT == 2 && DT == 3 && !RAG ? 1 : 2;
   static constexpr int kSuper = kColRows * kBlocks;
   static constexpr uint32_t kRedStride = 128 * NT;  // floats per (tile, warp)
   static constexpr size_t kRedFloats = (size_t)kBlocks * kColWarps * kRedStride;  // one half
@@ -108,23 +108,6 @@ template <int DT>
 __device__ __forceinline__ float col_scale(const uint8_t *s, uint64_t row) {
   if constexpr (DT == 3) return __half2float(reinterpret_cast<const __half *>(s)[row]);
   return 1.f;
-}
-
-// d += A B on one 16x8x16 tile; bf16 operands for DT 1, f16 otherwise.
-template <int DT>
-__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
-  if constexpr (DT == 1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-  } else {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-  }
 }
 
 // The activations of weight vector `vec` (global vector index col * V + v) of one column.
@@ -225,9 +208,6 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
     }
     const uint32_t ra[4] = {w0.x, w0.y, w0.z, w0.w};
     const uint32_t rb[4] = {w1.x, w1.y, w1.z, w1.w};
-    float part[NT][4];  // RAG: this vector's products
-#pragma unroll
-    for (int n = 0; n < NT; ++n) part[n][0] = part[n][1] = part[n][2] = part[n][3] = 0.f;
     if constexpr (DT == 3) {
       // word j = weights k 4j..4j+3 of the vector; its activations are x words 2j, 2j+1
 #pragma unroll
@@ -236,24 +216,27 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
         const uint32_t a0 = i8x2_to_f16x2(u0, 0x4140u), a2 = i8x2_to_f16x2(u0, 0x4342u);
         const uint32_t a1 = i8x2_to_f16x2(u1, 0x4140u), a3 = i8x2_to_f16x2(u1, 0x4342u);
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
-          mma16816<2>(RAG ? part[n] : acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
+        for (int n = 0; n < NT; ++n) {
+          if constexpr (RAG)
+            mma16816_kept<2>(acc[0][n], acc[1][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
+          else
+            mma16816<2>(acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
+        }
       }
     } else {
       // words 2s, 2s+1 = elements 4s..4s+3 of the vector
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
-          mma16816<DT>(RAG ? part[n] : acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
-                       xr[q][n][2 * s + 1]);
+        for (int n = 0; n < NT; ++n) {
+          if constexpr (RAG)
+            mma16816_kept<DT>(acc[0][n], acc[1][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
+                              xr[q][n][2 * s + 1]);
+          else
+            mma16816<DT>(acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
+                         xr[q][n][2 * s + 1]);
+        }
       }
-    }
-    if constexpr (RAG) {
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[q % H][n][i] += part[n][i];
     }
   }
 }
@@ -328,10 +311,11 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
           const uint32_t c0 = 2 * t + 8 * n;
-          r[red_at(c0, g)] = acc[b][0][n][0] + (H == 2 ? acc[b][H - 1][n][0] : 0.f);
-          r[red_at(c0 + 1, g)] = acc[b][0][n][1] + (H == 2 ? acc[b][H - 1][n][1] : 0.f);
-          r[red_at(c0, g + 8)] = acc[b][0][n][2] + (H == 2 ? acc[b][H - 1][n][2] : 0.f);
-          r[red_at(c0 + 1, g + 8)] = acc[b][0][n][3] + (H == 2 ? acc[b][H - 1][n][3] : 0.f);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float a0 = acc[b][0][n][i], a1 = H == 2 ? acc[b][H - 1][n][i] : 0.f;
+            r[red_at(c0 + (i & 1), g + 8 * (i >> 1))] = RAG ? kept_sum(a0, a1) : a0 + a1;
+          }
         }
       }
     }
@@ -340,10 +324,14 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
       const uint32_t b = o / kStride, e = o % kStride, col = e >> 4, row = b * kColRows + (e & 15);
       if (col < T && row < rows) {
         const float *r = red + b * kColWarps * kStride + red_at(col, e & 15);
-        float sum = 0.f;
+        float p[kColWarps];
 #pragma unroll
-        for (int w = 0; w < kColWarps; ++w) sum += r[w * kStride];
-        md.y[(uint64_t)col * md.M + sb + row] = sum * col_scale<DT>(md.s, sb + row);
+        for (int w = 0; w < kColWarps; ++w) p[w] = r[w * kStride];
+#pragma unroll
+        for (int h = kColWarps / 2; h > 0; h /= 2)  // in pairs: three roundings, not seven
+#pragma unroll
+          for (int w = 0; w < h; ++w) p[w] += p[w + h];
+        md.y[(uint64_t)col * md.M + sb + row] = p[0] * col_scale<DT>(md.s, sb + row);
       }
     }
   }

@@ -14,12 +14,16 @@
 //                   of X, and multiplies them with m16n8k16 MMAs whose four k per thread are
 //                   four consecutive elements of its vectors (wt_cols.cu has the argument)
 //
-// Each 64 bytes of a row start from zero accumulators and meet the row's fp32 sums, one of the even
-// and one of the odd 64 bytes, in ordinary additions (the tensor cores' own accumulation truncates;
-// error against 64 bits at 512 columns, bf16, T = 8: 7.3e-8, as before this kernel).  A row's result depends on its
-// matrix alone.  HBM bounds the kernel where rows have 256 bytes and more; below that, the
-// loads of shared memory and the stores of Y.
-#include <cuda_bf16.h>
+// The tensor cores truncate what they accumulate.  Whole vectors: every MMA starts from zero, the
+// two (int8: four) of 64 bytes meet in ordinary additions, and these the row's fp32 sums, one of the
+// even and one of the odd 64 bytes (error against 64 bits at T = 8, here / on the kernel that had
+// these rows before: 32 columns bf16 3.7e-8 / 3.7e-8, f16 5.5e-8 / 5.5e-8, int8 4.1e-8 / 4.2e-8; 512
+// columns 7.0e-8 / 7.3e-8, 8.3e-8 / 9.3e-8, 6.8e-8 / 7.5e-8).  Ragged rows, which had fp32 FMAs
+// before, keep what the truncation drops (mma16816_kept; 33 columns 2.8e-8 / 3.2e-8, 3.8e-8 / 5.6e-8,
+// 3.5e-8 / 3.8e-8; 333 columns 3.0e-8 / 5.8e-8, 3.8e-8 / 8.0e-8, 3.8e-8 / 6.2e-8), at 3 to 14 % more
+// time for T <= 8 and 14 to 45 % for T = 16.  A row's result depends on its matrix alone.  HBM
+// bounds the kernel where rows have 256 bytes and more; below that, the loads of shared memory and
+// the stores of Y.
 #include <cuda_fp16.h>
 
 #include "wt_device.cuh"
@@ -50,22 +54,6 @@ constexpr size_t kSSmem = kSFlagOff + 16;
 static_assert(kSSmem <= 232448 && kSBarOff % 8 == 0, "short-row shared memory");
 static_assert(16 * (size_t)short_xpitch(3, short_row_bytes(3) / 64) <= kSXBytes, "X of int8 weights");
 
-template <int DT>
-__device__ __forceinline__ void mma_short(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                          uint32_t b0, uint32_t b1) {
-  if constexpr (DT == 1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-  } else {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-  }
-}
-
 // X of the matrix to shared memory: 8 NT columns of nq 64-byte (int8: 128-byte) groups, zeros
 // past column T and past a column's end; all consumers.
 template <int DT, int NT>
@@ -90,6 +78,25 @@ __device__ __forceinline__ void stage_cols(uint32_t xs, const MatDesc &md, uint3
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(xs + col * pitch + o), "r"(v.x), "r"(v.y), "r"(v.z),
                  "r"(v.w)
                  : "memory");
+  }
+}
+
+// Step j of a vector's MMAs: to p, each from zero and added in fp32, or with KEEP to the row's
+// sums s, and what they lost to m.
+template <int DT, bool KEEP>
+__device__ __forceinline__ void mma_step(float (&s)[4], float (&m)[4], float (&p)[4], int j, uint32_t a0, uint32_t a1,
+                                         uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  if constexpr (KEEP) {
+    mma16816_kept<DT>(s, m, a0, a1, a2, a3, b0, b1);
+  } else {
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    if (j == 0) {
+      mma16816<DT>(p, a0, a1, a2, a3, b0, b1);
+    } else {
+      mma16816<DT>(z, a0, a1, a2, a3, b0, b1);
+      add_x2(p[0], p[1], z[0], z[1]);
+      add_x2(p[2], p[3], z[2], z[3]);
+    }
   }
 }
 
@@ -182,13 +189,14 @@ __global__ void __launch_bounds__(kSThreads, 1)
             const uint32_t row = q0 + 8 * k + g;
             a[k] = tile + (row < nr ? row : 0) * rowb + t * 16;
           }
-          float acc[kSTiles][NT][4], odd[kSTiles][NT][4];  // sums of the even and of the odd 64 bytes
+          // sums of the even and of the odd 64 bytes; RAG: the sums and what they lost
+          float acc[kSTiles][NT][4], more[kSTiles][NT][4];
 #pragma unroll
           for (uint32_t k = 0; k < kSTiles; ++k)
 #pragma unroll
             for (int n = 0; n < NT; ++n)
 #pragma unroll
-              for (int i = 0; i < 4; ++i) acc[k][n][i] = odd[k][n][i] = 0.f;
+              for (int i = 0; i < 4; ++i) acc[k][n][i] = more[k][n][i] = 0.f;
 #pragma unroll 2
           for (uint32_t q = 0; q < nq; ++q) {
             uint32_t xr[NT][DT == 3 ? 8 : 4];
@@ -223,24 +231,27 @@ __global__ void __launch_bounds__(kSThreads, 1)
                   const uint32_t a0 = i8x2_to_f16x2(u0, 0x4140u), a2 = i8x2_to_f16x2(u0, 0x4342u);
                   const uint32_t a1 = i8x2_to_f16x2(u1, 0x4140u), a3 = i8x2_to_f16x2(u1, 0x4342u);
 #pragma unroll
-                  for (int n = 0; n < NT; ++n) mma_short<2>(part[n], a0, a1, a2, a3, xr[n][2 * j], xr[n][2 * j + 1]);
+                  for (int n = 0; n < NT; ++n)
+                    mma_step<2, RAG>(acc[k][n], more[k][n], part[n], j, a0, a1, a2, a3, xr[n][2 * j], xr[n][2 * j + 1]);
                 }
               } else {
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
 #pragma unroll
                   for (int n = 0; n < NT; ++n)
-                    mma_short<DT>(part[n], ra[2 * j], rb[2 * j], ra[2 * j + 1], rb[2 * j + 1], xr[n][2 * j],
-                                  xr[n][2 * j + 1]);
+                    mma_step<DT, RAG>(acc[k][n], more[k][n], part[n], j, ra[2 * j], rb[2 * j], ra[2 * j + 1],
+                                      rb[2 * j + 1], xr[n][2 * j], xr[n][2 * j + 1]);
               }
+              if constexpr (!RAG) {
 #pragma unroll
-              for (int n = 0; n < NT; ++n)
+                for (int n = 0; n < NT; ++n)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  const float o = acc[k][n][i] + part[n][i];  // the two sets change places
-                  acc[k][n][i] = odd[k][n][i];
-                  odd[k][n][i] = o;
-                }
+                  for (int i = 0; i < 4; ++i) {
+                    const float o = acc[k][n][i] + part[n][i];  // the two sets change places
+                    acc[k][n][i] = more[k][n][i];
+                    more[k][n][i] = o;
+                  }
+              }
             }
           }
 #pragma unroll
@@ -248,7 +259,8 @@ __global__ void __launch_bounds__(kSThreads, 1)
 #pragma unroll
             for (int n = 0; n < NT; ++n)
 #pragma unroll
-              for (int i = 0; i < 4; ++i) acc[k][n][i] += odd[k][n][i];
+              for (int i = 0; i < 4; ++i)
+                acc[k][n][i] = RAG ? kept_sum(acc[k][n][i], more[k][n][i]) : acc[k][n][i] + more[k][n][i];
           // C fragment: (g, 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1) of each 8-column tile
 #pragma unroll
           for (uint32_t k = 0; k < 2 * kSTiles; ++k) {

@@ -3,6 +3,7 @@
 // Internal to the library (each translation unit gets its own copies).
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 
 #include "wt_kernels.h"
@@ -206,6 +207,62 @@ __device__ __forceinline__ uint32_t i8x2_to_f16x2(uint32_t u, uint32_t sel) {
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(h) : "r"(__byte_perm(u, 0x64646464u, sel)), "r"(0x64806480u));
   return h;
 }
+
+// d += A B on one 16x8x16 tile; bf16 operands for DT 1, f16 otherwise.
+template <int DT>
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  if constexpr (DT == 1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  } else {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  }
+}
+
+// Two fp32 differences or sums in one instruction.
+__device__ __forceinline__ void sub_x2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
+  asm("{\n\t.reg .b64 x, y;\n\t"
+      "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "sub.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(d0), "=f"(d1)
+      : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void add_x2(float &d0, float &d1, float b0, float b1) {
+  asm("{\n\t.reg .b64 x, y;\n\t"
+      "mov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\t"
+      "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(d0), "+f"(d1)
+      : "f"(b0), "f"(b1));
+}
+
+// s + c += A B, s the running sum and c what it lost.  The tensor cores truncate their sum to
+// fp32; a second MMA from the step s took backwards, A B - (s' - s), gives what they dropped,
+// because they align the products with a few bits more than a result keeps (16 random products,
+// 2-norm error of A B against 64 bits: f16 4.7e-8, with the second MMA 2.1e-8, rounded to nearest
+// 2.5e-8; bf16 2.5e-8, 3.9e-9, 1.8e-8; int8 2.1e-8, 2.9e-9, 1.5e-8).
+template <int DT>
+__device__ __forceinline__ void mma16816_kept(float (&s)[4], float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                              uint32_t a3, uint32_t b0, uint32_t b1) {
+  float t[4], r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) t[i] = s[i];
+  mma16816<DT>(t, a0, a1, a2, a3, b0, b1);
+  sub_x2(r[0], r[1], s[0], s[1], t[0], t[1]);
+  sub_x2(r[2], r[3], s[2], s[3], t[2], t[3]);
+  mma16816<DT>(r, a0, a1, a2, a3, b0, b1);
+  add_x2(c[0], c[1], r[0], r[1]);
+  add_x2(c[2], c[3], r[2], r[3]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s[i] = t[i];
+}
+// The sum: beside an infinite s, c means nothing.
+__device__ __forceinline__ float kept_sum(float s, float c) { return fabsf(s) < INFINITY ? s + c : s; }
 
 }  // namespace
 }  // namespace wt
