@@ -1620,17 +1620,21 @@ double largest_tile_share(const std::vector<wt::MatDesc> &mats, int ctas_per_sm,
 }
 
 // int8 weights on the tensor cores (T columns, and one column with rows up to K = 8192) run
-// the row-owner kernel (wt_q8rows.cu) unless its 128-row blocks leave the CTAs uneven: its
-// warps keep no activation registers and meet in no reduction, but a launch waits for the CTA
-// with one block more, where the warp-MMA kernel cuts at 16 rows.  Even, it is the faster by
-// 2, 5 and 30 % at T = 1, 8 and 16 (6663 / 6581 / 6502 GB/s against 6565 / 6250 / 5004); with
-// the largest CTA at 1.2 times an even share (128 MiB of 2048-weight rows) by 18 and 60 % at
-// T = 8 and 16; at 1.8 times (one large decoder layer, 336 blocks for 304 CTAs) it takes 51 /
-// 51 / 56 us and the warp-MMA kernel 39 / 40 / 55.  WT_COLS_KERNEL=mma or =q8rows forces one kernel for every int8 matrix
-// (the parity tests run each routing).
-bool i8_on_q8rows(double share, bool wide) {
+// the row-owner kernel (wt_q8rows.cu) where a group has at least two of its 128-row blocks per
+// CTA slot and they come out even over the CTAs: its warps keep no activation registers and meet
+// in no reduction, but a launch waits for the CTA with one block more, where the warp-MMA kernel
+// cuts at 16 rows.  Even, it is the faster by 2, 5 and 30 % at T = 1, 8 and 16 (6663 / 6581 / 6502
+// GB/s against 6565 / 6250 / 5004); with the largest CTA at 1.2 times an even share (128 MiB of
+// 2048-weight rows) by 18 and 60 % at T = 8 and 16; at 1.8 times (one large decoder layer, 336
+// blocks for 304 CTAs) it takes 51 / 51 / 56 us and the warp-MMA kernel 39 / 40 / 55.  Smaller
+// launches stay off it, also where their blocks come out even (8192 x 512: 64 blocks, 64 CTAs), for
+// precision: it adds up a whole row in the tensor cores, which truncate (2-norm error against 64
+// bits at 512 weights 2.1e-7; warp-MMA kernel 7.5e-8, short-row kernel 6.8e-8).
+// WT_COLS_KERNEL=mma or =q8rows forces one kernel for every int8 matrix (the parity tests run
+// each routing).
+bool i8_on_q8rows(uint64_t blocks, double share, bool wide) {
   const int f = cols_forced();
-  return f == 3 || (f != 2 && share < (wide ? 1.6 : 1.35));
+  return f == 3 || (f != 2 && blocks >= 2ull * wt::num_sms() && share < (wide ? 1.6 : 1.35));
 }
 
 size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
@@ -1747,6 +1751,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         short_dt[4][4],           // [dtype][T > 8, + 2 if ragged]: short rows
         q8r1_dt[4];  // row-owner int8 launches with two 8-column tiles (T > 8) and with one
     std::vector<wt_gemv_desc> i8c[2];  // int8 on the tensor cores, T <= 8 and T > 8: kernel chosen below
+    uint64_t i8_blocks = 0;            // their 128-row blocks
     std::vector<int64_t> seg_ws[4];  // per by_dt entry: workspace float offset of its partials, or -1
     std::vector<std::pair<wt::MatDesc, size_t>> cseg_dt[4][2];  // multi-column segments [dtype][T > 8], likewise
     std::vector<wt::SegReduce> reds;
@@ -1827,6 +1832,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         g.reduce_rows = std::max(g.reduce_rows, (uint32_t)outs);
       } else if (fast && q.cols > 0 && q.dtype == WT_I8) {
         i8c[q.cols > 8 ? 1 : 0].push_back(q);
+        i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
       } else if (fast && q.cols > 0 && q.dtype != WT_F32) {
         (cols_on_umma(q) ? umma_dt : q.cols > 8 ? colsw_dt : cols_dt)[q.dtype].push_back(make_cols_mat(q));
       } else if (fast && q.dtype == WT_I8 && i8_onecol_on_mma((uint32_t)(q.K / 16))) {
@@ -1834,6 +1840,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         wt_gemv_desc q1 = q;
         q1.cols = 1;
         i8c[0].push_back(q1);
+        i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
       } else if (q.cols > 0 && q.dtype != WT_F32 && q.K * es < 0x7fffffffull) {
         (q.cols > 8 ? ragcw_dt : ragc_dt)[q.dtype].push_back(make_cols_mat(q, true));
       } else if (q.cols == 0 && (fast || (q.K * es < 0x7fffffffull && reinterpret_cast<uintptr_t>(q.W) % es == 0))) {
@@ -1885,8 +1892,8 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
       blocks.block = wt::kQ8RowsBlock;
       // a block that is itself above the limit settles it without dealing
       double share = largest_tile_share(ms, 2, blocks);
-      if (cols_forced() == 0 && i8_on_q8rows(share, w == 1)) share = deal_tiles(ms, grid, pieces, begin, 2, blocks);
-      if (i8_on_q8rows(share, w == 1)) {
+      if (cols_forced() == 0 && i8_on_q8rows(i8_blocks, share, w == 1)) share = deal_tiles(ms, grid, pieces, begin, 2, blocks);
+      if (i8_on_q8rows(i8_blocks, share, w == 1)) {
         (w ? q8r_dt : q8r1_dt)[WT_I8] = std::move(ms);
         continue;
       }

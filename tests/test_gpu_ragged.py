@@ -203,6 +203,27 @@ def test_ragged_columns_are_as_exact_as_fp32_fmas(torch, dtype, T):
         assert h.device_status() == 0
 
 
+@pytest.mark.parametrize("T", [0, 8, 12])
+def test_small_int8_launches_stay_exact(torch, T):
+    """Launches of fewer than 304 blocks of 128 rows, evenly dealt ones among them: the tensor
+    cores truncate, so a sum of them may lose twice what fp32 FMAs lose, and no more."""
+    rng = np.random.default_rng(77 + T)
+    with wt.Handle([]) as h:
+        for M, K in ((8192, 128), (8192, 256), (8192, 512), (4096, 576), (2048, 1024)):
+            W, X = weights(rng, I8, M * K), weights(rng, F16, max(1, T) * K)
+            wb, wp = at(torch, W, 0)
+            xb, xp = at(torch, X, 0)
+            sb, sp = at(torch, np.ones(M, np.float16).view(np.uint8), 0)
+            y = torch.full((max(1, T) * M,), float("nan"), dtype=torch.float32, device="cuda")
+            h.pass_([wt.gemv_desc(wp, I8, M, K, xp, y.data_ptr(), scale=sp, cols=T)], 0)
+            Wf, Xf = W.view(np.int8).astype(np.float32).reshape(M, K), floats(F16, X).reshape(-1, K)
+            exact = Xf.astype(np.float64) @ Wf.astype(np.float64).T
+            ours = np.linalg.norm(y.cpu().numpy().reshape(-1, M) - exact)
+            theirs = np.linalg.norm(fma_chains(Wf, Xf) - exact)
+            assert ours <= 2 * theirs, (T, M, K, ours / theirs)
+        assert h.device_status() == 0
+
+
 @pytest.mark.parametrize("K", [45, 1031])
 def test_ragged_columns_with_infinities_and_overflow(torch, K):
     """An infinite weight, sums that leave fp32 on either side, and a NaN, in rows of their own:
