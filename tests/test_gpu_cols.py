@@ -30,10 +30,12 @@ def torch():
 
 @pytest.fixture(params=["default", "mma", "umma", "q8rows"], autouse=True)
 def cols_kernel(request, monkeypatch):
-    """Every test runs under each routing of the multi-column kernels: the default (int8 with
-    T > 8 on the row-owner kernel, 2-byte weights with T > 8 on tcgen05, the rest on the
-    warp-MMA kernel), everything on the warp-MMA kernel (WT_COLS_KERNEL=mma), 2-byte weights
-    on tcgen05 at every T (=umma), and int8 on the row-owner kernel at every T (=q8rows)."""
+    """Every test runs under each routing of the multi-column kernels: the default (short rows on
+    their own kernel, int8 in large even launches on the row-owner kernel, large 2-byte matrices
+    of rows up to 3072 bytes with T > 8 on tcgen05, the rest on the warp-MMA kernel), everything
+    on the warp-MMA kernel (WT_COLS_KERNEL=mma), 2-byte weights on tcgen05 at every T (=umma),
+    and int8 on the row-owner kernel at every T (=q8rows).  Ragged operands take the same kernels
+    under each."""
     if request.param == "default":
         monkeypatch.delenv("WT_COLS_KERNEL", raising=False)
     else:
@@ -308,3 +310,38 @@ def test_cols_bits_do_not_depend_on_the_launch(torch, T):
                     mag = Xs[i].double().abs() @ Ws[i].double().abs().t()
                     assert ((alone[0].view(T, -1).double() - ref).abs() <= TOL * mag).all()
             assert h.device_status() == 0
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_random_sets_are_dealt_whole(torch, seed):
+    """Random sets of matrices in one pass, T on both sides of 8, aligned and ragged, short rows and
+    long ones, even and uneven over the CTAs: every output against 64-bit sums, Y NaN-filled
+    first (a row that no CTA was dealt stays NaN)."""
+    rng = np.random.default_rng(600 + seed)
+    g = torch.Generator("cuda").manual_seed(seed)
+    mats = []
+    for _ in range(int(rng.integers(1, 24))):
+        dtype = int(rng.choice([BF16, F16, I8]))
+        T = int(rng.integers(1, 17))
+        K = int(np.exp(rng.uniform(np.log(16), np.log(9000))))
+        K = max(1, K // int(rng.choice([64, 64, 16, 1])) * 64) if rng.random() < 0.5 else K
+        M = int(np.exp(rng.uniform(np.log(1), np.log(max(2, min(40000, (48 << 20) // K))))))
+        tdt = {BF16: torch.bfloat16, F16: torch.float16, I8: torch.int8}[dtype]
+        W = torch.randint(-128, 128, (M, K), dtype=tdt, device="cuda", generator=g) if dtype == I8 else \
+            torch.empty(M, K, dtype=tdt, device="cuda").normal_(0, 0.02, generator=g)
+        s = torch.rand(M, device="cuda", generator=g).half() if dtype == I8 else None
+        X = torch.empty(T, K, dtype=torch.float16 if dtype == I8 else tdt, device="cuda").normal_(0, 1, generator=g)
+        mats.append((dtype, T, W, s, X, torch.full((T * M,), float("nan"), device="cuda")))
+    with wt.Handle([]) as h:
+        h.pass_([wt.gemv_desc(W.data_ptr(), d, *W.shape, X.data_ptr(), y.data_ptr(), cols=T,
+                              scale=s.data_ptr() if s is not None else 0) for d, T, W, s, X, y in mats], 0)
+        torch.cuda.synchronize()
+        assert h.device_status() == 0
+    for d, T, W, s, X, y in mats:
+        for r in range(0, W.shape[0], 8192):
+            w = W[r:r + 8192].double()
+            ref, mag = X.double() @ w.t(), X.double().abs() @ w.abs().t()
+            if s is not None:
+                ref, mag = ref * s[r:r + 8192].double(), mag * s[r:r + 8192].double()
+            got = y.view(T, -1)[:, r:r + 8192].double()
+            assert ((got - ref).abs() <= TOL * mag).all(), (d, T, tuple(W.shape), r)

@@ -349,6 +349,33 @@ def test_plain_digest_chunks(torch, sizes):
         assert got == [oracle.fnv1a64(data[off:off + n]) for n in sizes]
 
 
+@pytest.mark.parametrize("sizes", [(300, 65536, 7), (65537, 300, 0, 4096), (60000,) * 600])
+def test_plain_digest_in_a_capture(torch, sizes):
+    """The literal digest inside a stream capture holds no allocation: batches of short buffers run
+    in blocks, one buffer above 64 KiB, or more than 32 MiB in all, makes the batch serial.  Both
+    give the digests of the same call outside, and the graph replays."""
+    rng = np.random.default_rng(len(sizes))
+    buf = torch.from_numpy(rng.integers(0, 256, max(sizes) + 64, dtype=np.uint8)).cuda()
+    ptrs = [buf.data_ptr() + 16 * (i % 4) for i in range(len(sizes))]
+    out, ref = (torch.zeros(len(sizes), dtype=torch.int64, device="cuda") for _ in range(2))
+    s = torch.cuda.Stream()
+    with wt.Handle([]) as h:
+        h.checksum(ptrs, sizes, ref.data_ptr(), s.cuda_stream, plain=True)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            h.checksum(ptrs, sizes, out.data_ptr(), s.cuda_stream, plain=True)
+        for _ in range(2):
+            out.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(out, ref)
+    host = buf.cpu().numpy()
+    for i in range(min(4, len(sizes))):
+        o = 16 * (i % 4)
+        assert int(ref[i]) & (2 ** 64 - 1) == oracle.fnv1a64(host[o:o + sizes[i]])
+
+
 @pytest.mark.parametrize("off", [0, 3])
 @pytest.mark.parametrize("leaves", [8192, 8193])
 def test_tree_digest_leaves_by_warps_and_by_threads(torch, off, leaves):
@@ -367,27 +394,31 @@ def test_tree_digest_leaves_by_warps_and_by_threads(torch, off, leaves):
     assert got == [oracle.fnv_tree(data[:n]) for n in sizes]
 
 
-def test_unaligned_operands_take_the_generic_kernel(torch):
-    """W and x 2 bytes past a 16-byte boundary (element-aligned only): the scalar fallback,
-    checked against the oracle; one and several columns."""
+def test_operands_two_bytes_off_a_vector(torch):
+    """W and x 2 bytes past a 16-byte boundary (element-aligned only), one and several columns,
+    against the oracle: in device memory on the ragged-row kernels, and W in pinned host memory on
+    the scalar fallback."""
     rng = np.random.default_rng(13)
     M, K, T = 37, 1000, 3
     Wb = synth.f32_to_bf16_bits((0.02 * rng.standard_normal(M * K)).astype(np.float32)).view(np.uint8)
     X = synth.f32_to_bf16_bits(rng.standard_normal(T * K).astype(np.float32)).view(np.uint8)
     Wd = torch.zeros(Wb.size + 16, dtype=torch.uint8, device="cuda")
     Wd[2:2 + Wb.size] = torch.from_numpy(Wb.copy()).cuda()
+    Wp = torch.zeros(Wb.size + 16, dtype=torch.uint8).pin_memory()
+    Wp[2:2 + Wb.size] = torch.from_numpy(Wb.copy())
     Xd = torch.zeros(X.size + 16, dtype=torch.uint8, device="cuda")
     Xd[2:2 + X.size] = torch.from_numpy(X.copy()).cuda()
-    y1 = torch.full((M,), float("nan"), dtype=torch.float32, device="cuda")
-    yT = torch.full((T * M,), float("nan"), dtype=torch.float32, device="cuda")
-    with wt.Handle([]) as h:
-        h.pass_([wt.gemv_desc(Wd.data_ptr() + 2, wt.WT_BF16, M, K, Xd.data_ptr() + 2, y1.data_ptr()),
-                 wt.gemv_desc(Wd.data_ptr() + 2, wt.WT_BF16, M, K, Xd.data_ptr() + 2, yT.data_ptr(), cols=T)], 0)
-        torch.cuda.synchronize()
-        assert h.device_status() == 0
     Y, A = oracle.gemv_cols(Wb, wt.WT_BF16, M, K, X, T)
-    assert oracle.gemv_error(y1.cpu().numpy(), Y[0], A[0]) <= 2e-3
-    assert oracle.gemv_error(yT.cpu().numpy(), Y.reshape(-1), A.reshape(-1)) <= 2e-3
+    for W in (Wd, Wp):
+        y1 = torch.full((M,), float("nan"), dtype=torch.float32, device="cuda")
+        yT = torch.full((T * M,), float("nan"), dtype=torch.float32, device="cuda")
+        with wt.Handle([]) as h:
+            h.pass_([wt.gemv_desc(W.data_ptr() + 2, wt.WT_BF16, M, K, Xd.data_ptr() + 2, y1.data_ptr()),
+                     wt.gemv_desc(W.data_ptr() + 2, wt.WT_BF16, M, K, Xd.data_ptr() + 2, yT.data_ptr(), cols=T)], 0)
+            torch.cuda.synchronize()
+            assert h.device_status() == 0
+        assert oracle.gemv_error(y1.cpu().numpy(), Y[0], A[0]) <= 2e-3
+        assert oracle.gemv_error(yT.cpu().numpy(), Y.reshape(-1), A.reshape(-1)) <= 2e-3
 
 
 def test_descriptor_bounds_are_refused_before_any_launch(torch):

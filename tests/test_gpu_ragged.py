@@ -86,11 +86,12 @@ def test_ragged_rows_against_oracle(torch, dtype, odd):
 
 # (M, bytes of a row, bytes past a 16-byte boundary of W and of X): a 16-row tile and a 64-row
 # super block and one more row; one 4-vector group; 84 vectors (one chunk) and one more; several
-# uneven chunks; aligned rows, also at unaligned addresses; the longest short rows (2048 bytes;
-# int8: 1024) and one byte or element either way; 32-row groups and several stages of them
+# uneven chunks; aligned rows, also at unaligned addresses; on both sides of the longest short
+# rows (1024 bytes; int8: 512); several stages of 32-row groups
 COL_SHAPES = [(1, 4, 0, 0), (17, 20, 4, 4), (64, 64, 4, 0), (65, 132, 0, 0), (33, 1340, 0, 4), (16, 1344, 4, 0),
               (80, 1348, 0, 0), (130, 2732, 8, 8), (40, 5460, 0, 0), (23, 20004, 4, 4), (1100, 32, 0, 0), (600, 48, 0, 0),
-              (70, 1024, 0, 0), (33, 1028, 4, 0), (200, 2048, 0, 0), (35, 2052, 0, 0)]
+              (70, 1024, 0, 0), (33, 1028, 4, 0), (200, 2048, 0, 0), (35, 2052, 0, 0), (100, 300, 0, 2), (70, 508, 2, 0),
+              (100, 512, 4, 0), (70, 514, 0, 0), (70, 516, 2, 2), (70, 1022, 0, 0), (100, 1024, 2, 0), (70, 1026, 0, 0)]
 
 
 @pytest.mark.parametrize("dtype", [BF16, F16, I8])
@@ -200,6 +201,32 @@ def test_ragged_columns_are_as_exact_as_fp32_fmas(torch, dtype, T):
             ours = np.linalg.norm(y.cpu().numpy().reshape(T, M) - exact)
             theirs = np.linalg.norm(fma_chains(Wf, Xf) - exact)
             assert ours <= 1.02 * theirs, (dtype, T, K, ours / theirs)
+        assert h.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", [BF16, F16, I8])
+@pytest.mark.parametrize("T", [5, 16])
+def test_short_rows_over_many_stages(torch, dtype, T):
+    """Short rows, aligned and ragged, with some 200 KB for each CTA: the ring of five 32 KB stages
+    wraps within one matrix.  Against 64-bit sums, Y NaN-filled first."""
+    g = torch.Generator("cuda").manual_seed(50 + T)
+    tdt = {BF16: torch.bfloat16, F16: torch.float16, I8: torch.int8}[dtype]
+    shapes = ((60001, 509), (30001 * 20, 48)) if dtype == I8 else ((30001, 512), (30001, 511), (40 * 30001, 13))
+    with wt.Handle([]) as h:
+        for M, K in shapes:
+            if dtype == I8:
+                W = torch.randint(-128, 128, (M, K), dtype=tdt, device="cuda", generator=g)
+                s = torch.rand(M, device="cuda", generator=g).half()
+            else:
+                W, s = torch.empty(M, K, dtype=tdt, device="cuda").normal_(0, 0.02, generator=g), None
+            X = torch.empty(T, K, dtype=torch.float16 if dtype == I8 else tdt, device="cuda").normal_(0, 1, generator=g)
+            y = torch.full((T * M,), float("nan"), device="cuda")
+            h.pass_([wt.gemv_desc(W.data_ptr(), dtype, M, K, X.data_ptr(), y.data_ptr(), cols=T,
+                                  scale=s.data_ptr() if s is not None else 0)], 0)
+            ref, mag = X.double() @ W.double().t(), X.double().abs() @ W.double().abs().t()
+            if s is not None:
+                ref, mag = ref * s.double(), mag * s.double()
+            assert ((y.view(T, M).double() - ref).abs() <= 2 * bound(K) * mag).all(), (dtype, T, M, K)
         assert h.device_status() == 0
 
 
