@@ -295,9 +295,12 @@ int wt_checksum(wt_handle *h, const void *const *ptr, const uint64_t *nbytes, si
                 uint64_t *out_dev, void *stream);
 
 /* Literal FNV-1a-64 of each device buffer (meant for verification).  Buffers above 256 MiB
- * are rejected with WT_EINVAL.  The serial chain of a buffer runs in parallel chunks with
- * temporary stream-ordered storage (about 2 bytes for each 256 of input at most); where none
- * is to be had, and inside a stream capture, one thread runs each buffer above 64 KiB. */
+ * are rejected with WT_EINVAL.  The serial chain of a buffer runs in parallel chunks.  The
+ * buffers of a call are taken in batches of up to 1344.  A batch of buffers of up to 64 KiB that
+ * has no more than 32 MiB in all needs no storage.  Others take temporary stream-ordered
+ * storage, 16 bytes for each chunk: of 256 bytes up to 32 MiB of input (a sixteenth of it), of up
+ * to 4096 bytes for more, so that 2 MiB serve 512 MiB.  Where none is to be had, and inside
+ * a stream capture, one thread runs each buffer of such a batch, at about 1 ms for 64 KiB. */
 int wt_checksum_plain(wt_handle *h, const void *const *ptr, const uint64_t *nbytes, size_t n,
                       uint64_t *out_dev, void *stream);
 

@@ -62,10 +62,6 @@ constexpr uint32_t kColStageBytes = kColRows * kColVecMax * 16;
 static_assert(kColVecMax % 8 == 4, "row pitch 64 bytes past a multiple of 128");
 static_assert(kColStageBytes % 128 == 0, "stages stay 128-byte aligned for the tensor copies");
 
-// Per-launch geometry: NT = 8-column MMA tiles (T <= 8: 1, else 2).  int8 weights and
-// ragged operands run two CTAs per SM with half the ring each (the same bytes in flight per SM,
-// twice the warps; those paths are latency-bound on decoding and on shifting).  The cross-warp partials of one 16-row tile take
-// 16 x 8 NT floats per warp, in two alternating halves.
 // Where a partial sum of (column, row) sits among its tile's: a pair of columns takes 32 floats,
 // turned by 8 per pair, so that neither the stores of a fragment (rows g of the columns 2t; in
 // plain order the four shared a bank) nor the sums over a pair meet in a bank.
@@ -73,6 +69,10 @@ __device__ __forceinline__ uint32_t red_at(uint32_t col, uint32_t row) {
   return (col >> 1) * 32 + ((((col & 1) << 4) + row + 8 * (col >> 1)) & 31);
 }
 
+// Per-launch geometry: NT = 8-column MMA tiles (T <= 8: 1, else 2).  int8 weights and
+// ragged operands run two CTAs per SM with half the ring each (the same bytes in flight per SM,
+// twice the warps; those paths are latency-bound on decoding and on shifting).  The cross-warp
+// partials of one 16-row tile take 16 x 8 NT floats per warp, in two alternating halves.
 template <int DT, int NT, bool RAG = false>
 struct ColGeo {
   static constexpr int kCtasPerSm = DT == 3 || RAG ? 2 : 1;

@@ -43,7 +43,8 @@ constexpr size_t kChunkScratchBytes = 4 + 4 + 8;
 
 // Fills b with the leading buffers of the list (*taken of them, at least one) and returns the
 // device scratch bytes that launch_fnv_tree, or with `plain` launch_fnv_plain, needs for them
-// (0 for literal digests of buffers of up to 64 KiB).  Digest i goes to out[i].
+// (0 for literal digests where no buffer has more than 64 KiB and the batch no more than 32 MiB).
+// Digest i goes to out[i].
 size_t fnv_fill_batch(FnvBatch &b, const void *const *ptr, const uint64_t *nbytes, uint64_t *out, size_t n, bool plain,
                       size_t *taken);
 
@@ -53,7 +54,7 @@ int fnv_tree_launches(const FnvBatch &b);
 cudaError_t launch_fnv_tree(const FnvBatch &b, void *scratch, cudaStream_t s);
 
 // The literal digests.  With the scratch that fnv_fill_batch asked for the chains run in chunks;
-// where there is none to be had, in one thread per buffer.
+// where there is none to be had, every buffer of the batch in one thread.
 int fnv_plain_launches(const FnvBatch &b, bool scratch);
 cudaError_t launch_fnv_plain(const FnvBatch &b, void *scratch, cudaStream_t s);
 

@@ -54,7 +54,7 @@ struct alignas(16) MatDesc {
   float *y;
   const uint8_t *s;  // f16 row scales (int8 weights), else null
   uint32_t M;     // rows
-  uint32_t V;     // 16-byte vectors per row (K * sizeof(elem) / 16)
+  uint32_t V;     // 16-byte vectors per row (K * sizeof(elem) / 16, rounded up)
   uint32_t rt;    // rows per tile (modes 0/1) or per row block (mode 2)
   uint32_t vc;    // vectors per column chunk (mode 2); V otherwise
   uint16_t mode;  // GemvMode
@@ -74,14 +74,15 @@ static_assert(sizeof(MatDesc) == 64, "MatDesc is one 64-byte record");
 // segments of each row in segment order and applies the row scale.  Segment boundaries
 // depend only on the matrix, so a row's result never depends on how rows and segments were
 // spread over CTAs.
-// What a stage of whole ragged rows needs besides them: the phases of its two ends.
-constexpr uint32_t kRaggedSlack = 32;
-
-// Ragged rows: at most this many vectors, counted from the grid point at or before the row's
-// start (the x registers of a lane: 64, or 48 for int8, which runs two CTAs per SM).
-constexpr uint32_t kPhaseVec(int dtype) { return dtype == 3 ? 192 : 512; }
 constexpr uint32_t kSegVec = 2048;  // bf16 / f16 / f32: 32 KB per segment row
 constexpr uint32_t seg_vectors(int dtype) { return dtype == 3 ? kSegVec / 4 : kSegVec; }  // int8: 8 KB
+
+// Ragged rows: what a stage of whole rows needs besides them, the phases of its two ends.
+constexpr uint32_t kRaggedSlack = 32;
+// Ragged rows of the one-column kernel: at most this many vectors, counted from the grid point
+// at or before the row's start (the x registers of a lane: 64, or 48 for int8, which runs two CTAs
+// per SM).  Longer ones go in column segments.
+constexpr uint32_t kPhaseVec(int dtype) { return dtype == 3 ? 192 : 512; }
 
 struct alignas(16) SegReduce {
   const float *ws;   // nseg x M partial sums (segment-major)
@@ -188,9 +189,9 @@ struct UmmaLaunch {
 cudaError_t gemm_cols_umma_prepare();
 cudaError_t launch_gemm_cols_umma(const UmmaLaunch &L, cudaStream_t s);
 
-// Fallback for operands the tiled kernels cannot take (W read in place from host memory with
-// unaligned W/x or rows whose byte length is not a multiple of 16, and such rows of 2^31 bytes
-// and more): one warp per row, scalar loads.  cols = 0 or 1: y = W x; cols = T > 1: Y [T, M] from X [T, K].
+// Fallback for operands the tiled kernels cannot take: W read in place from host memory with
+// unaligned W/x or rows whose byte length is not a multiple of 16, such rows of 2^31 bytes and
+// more, and one-column W off its element size.  One warp per row, scalar loads.  cols = 0 or 1: y = W x; cols = T > 1: Y [T, M] from X [T, K].
 cudaError_t launch_gemv_generic(int dtype, const uint8_t *W, const uint8_t *x, float *y,
                                 uint64_t M, uint64_t K, const uint8_t *scale, uint32_t cols,
                                 cudaStream_t s);
