@@ -271,7 +271,7 @@ int wt_adopt(wt_handle *h, const size_t *idx, void *const *dst, size_t n, unsign
  * calls with identical descriptors reuse a cached launch plan.  Results are deterministic (no
  * floating-point atomics), and a row's result does not depend on how rows were grouped or split,
  * with one exception: int8 matrices in device memory whose operands lie on 16-byte boundaries
- * run on one of three tensor-core kernels, chosen by the int8 matrices of the whole group, and
+ * run on one of several kernels, chosen by the int8 matrices of the whole group, and
  * these round differently (in fp32 sums, so by the last bits).
  *
  * Stream capture: a wt_pass issued on a stream that is being captured into a CUDA graph

@@ -1396,11 +1396,25 @@ int encode_q8rows_maps(const wt::MatDesc &m, uint8_t *out) {
 // tests run both ways).
 // Rows of up to 64 weights stay on the CUDA cores too: an MMA's k is mostly padding there
 // (128 MiB of 32-weight rows: 53 us against 108 us on the short-row kernel and 167 us on the
-// row-owner kernel; 64 weights: 45, 52, 53 us; 128: 48, 38, 32 us).
-bool i8_onecol_on_mma(uint32_t V) {
+// row-owner kernel; 64 weights: 45, 52, 53 us; 128: 48, 38, 32 us); unless there are less than
+// 20 MiB of them beside longer ones, where the launch of their own costs more than it saves (the
+// first n matrices of the many-small set, us with / without: n = 40 30.0 / 23.7, 70 34.9 / 30.3, 100
+// 39.4 / 30.1, 140 43.7 / 30.1 (17 MiB), 200 38.6 / 48.5 (24 MiB)).
+bool tiny_i8_on_mma(const wt_gemv_desc *d, const std::vector<size_t> &group) {
+  uint64_t tiny = 0;
+  bool longer = false;
+  for (const size_t k : group) {
+    if (d[k].dtype != WT_I8 || d[k].cols != 0) continue;
+    if (d[k].K <= 64) tiny += d[k].M * d[k].K;
+    else longer |= d[k].M > 0 && d[k].K % 16 == 0 && d[k].K / 16 <= wt::seg_vectors(WT_I8);
+  }
+  return longer && tiny < 20ull << 20;
+}
+
+bool i8_onecol_on_mma(uint32_t V, bool tiny) {
   const char *e = getenv("WT_I8_ONECOL");
   if (e && strcmp(e, "cuda") == 0) return false;
-  return (V > 4 || cols_forced()) && V <= wt::seg_vectors(WT_I8);
+  return (V > 4 || tiny || cols_forced()) && V <= wt::seg_vectors(WT_I8);
 }
 
 // The two tensor maps of a tcgen05 multi-column matrix (2-byte weights; see wt::UmmaLaunch).
@@ -1757,6 +1771,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
     std::vector<wt::SegReduce> reds;
     std::vector<size_t> red_ws;      // per reds entry: workspace float offset
     RangeCache rcw, rcx, rcy, rcs;
+    const bool i8_tiny = tiny_i8_on_mma(d, mem);
     for (const size_t k : mem) {
       const wt_gemv_desc &q = d[k];
       if (q.M == 0) continue;
@@ -1835,7 +1850,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
       } else if (fast && q.cols > 0 && q.dtype != WT_F32) {
         (cols_on_umma(q) ? umma_dt : q.cols > 8 ? colsw_dt : cols_dt)[q.dtype].push_back(make_cols_mat(q));
-      } else if (fast && q.dtype == WT_I8 && i8_onecol_on_mma((uint32_t)(q.K / 16))) {
+      } else if (fast && q.dtype == WT_I8 && i8_onecol_on_mma((uint32_t)(q.K / 16), i8_tiny)) {
         // y[M] is Y[1, M] and x[K] is X[1, K]: the one-column GEMV as a T = 1 tensor-core GEMV
         wt_gemv_desc q1 = q;
         q1.cols = 1;
