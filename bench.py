@@ -1114,9 +1114,9 @@ def run_tsweep(args):
             two_byte = all(dev.mats[k].dtype in (wt.WT_BF16, wt.WT_F16) for k in ks)
             force = os.environ.get("WT_COLS_KERNEL")
             shapes = [dev.mats[k].shape for k in ks]
-            # as the library decides, matrix by matrix: large ones of rows up to 3072 bytes
+            # as the library decides, matrix by matrix: very large ones of rows up to 3072 bytes
             on_umma = two_byte and (force == "umma" or (force != "mma" and T > 8 and
-                                                        all(M >= 16384 and 1024 < 2 * K <= 3072 for M, K in shapes)))
+                                                        all(-(-M // 128) >= 16 * 152 and 1024 < 2 * K <= 3072 for M, K in shapes)))
             int8 = all(dev.mats[k].dtype == wt.WT_I8 for k in ks)
             kname = (onecol_kernel_name(DT_NAME[dev.mats[ks[0]].dtype], shapes) if T == 0 else
                      "gemm_cols_umma (tcgen05, M128 N16 K16)" if on_umma else

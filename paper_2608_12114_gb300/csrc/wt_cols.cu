@@ -73,9 +73,14 @@ __device__ __forceinline__ uint32_t red_at(uint32_t col, uint32_t row) {
 // ragged operands run two CTAs per SM with half the ring each (the same bytes in flight per SM,
 // twice the warps; those paths are latency-bound on decoding and on shifting).  The cross-warp
 // partials of one 16-row tile take 16 x 8 NT floats per warp, in two alternating halves.
-template <int DT, int NT, bool RAG = false>
+// So do, with TWO, 2-byte weights with 16 columns in launches that are mostly of few short chunks
+// (the host's cols_two_ctas): there the waits for X and for the other warps' partials are a large
+// part of a super block, and the second CTA fills them (T = 16, bf16, 1 GiB of 16384-row matrices, us
+// with one / two: K = 768 259 / 207, 1024 210 / 188, 1536 196 / 177; but 2048 173 / 177, 8192 165 /
+// 168).  The sums are the same in either.
+template <int DT, int NT, bool RAG = false, bool TWO = false>
 struct ColGeo {
-  static constexpr int kCtasPerSm = DT == 3 || RAG ? 2 : 1;
+  static constexpr int kCtasPerSm = DT == 3 || RAG || TWO ? 2 : 1;
   static constexpr int kStages = kCtasPerSm == 2 ? 3 : 6;
   // 16-row tiles per super block (X registers are loaded once per super block and chunk):
   // four, or two for int8 with 16 columns, which then fits two CTAs per SM (registers and
@@ -95,7 +100,7 @@ struct ColGeo {
 };
 static_assert(ColGeo<1, 2>::kSmem <= 232448 && 2 * (ColGeo<3, 1>::kSmem + 1024) <= 233472 &&
                   2 * (ColGeo<3, 2>::kSmem + 1024) <= 233472 && 2 * (ColGeo<1, 1, true>::kSmem + 1024) <= 233472 &&
-                  2 * (ColGeo<1, 2, true>::kSmem + 1024) <= 233472,
+                  2 * (ColGeo<1, 2, true>::kSmem + 1024) <= 233472 && 2 * (ColGeo<1, 2, false, true>::kSmem + 1024) <= 233472,
               "multi-column shared memory");
 
 // 32-bit words of X per weight vector: 16 fp16 activations for an int8 vector, else 8.
@@ -248,7 +253,7 @@ struct Ring {
 };
 
 // Consumer side of one piece (rows [r0, r1) of one matrix), NT = 8-column MMA tiles.
-template <int DT, int NT, bool RAG>
+template <int DT, int NT, bool RAG, bool TWO>
 __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, const Ring &R, float *red_base,
                                            uint32_t &it, uint32_t &par, int warp, int lane) {
   const uint32_t V = md.V, vc = md.vc, T = md.G;
@@ -258,12 +263,12 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
   const uint32_t nchunk = (V + vc - 1) / vc;
   const uint32_t g = lane >> 2, t = lane & 3;
   const int ct = threadIdx.x;
-  constexpr int kColBlocks = ColGeo<DT, NT, RAG>::kBlocks;
-  constexpr int kColSuper = ColGeo<DT, NT, RAG>::kSuper;
+  constexpr int kColBlocks = ColGeo<DT, NT, RAG, TWO>::kBlocks;
+  constexpr int kColSuper = ColGeo<DT, NT, RAG, TWO>::kSuper;
   for (uint32_t sb = pc.r0; sb < pc.r1; sb += kColSuper) {
     const uint32_t rows = min((uint32_t)kColSuper, pc.r1 - sb);
     const uint32_t nrb = (rows + kColRows - 1) / kColRows;
-    constexpr int H = ColGeo<DT, NT, RAG>::kAcc;
+    constexpr int H = ColGeo<DT, NT, RAG, TWO>::kAcc;
     float acc[kColBlocks][H][NT][4];
 #pragma unroll
     for (int b = 0; b < kColBlocks; ++b)
@@ -287,8 +292,8 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
 #pragma unroll
       for (int b = 0; b < kColBlocks; ++b) {
         if ((uint32_t)b < nrb) {
-          const uint32_t s = it % ColGeo<DT, NT, RAG>::kStages;
-          bounded_wait(R.full0 + 8 * s, (it / ColGeo<DT, NT, RAG>::kStages) & 1, R.abort_flag, R.status);
+          const uint32_t s = it % ColGeo<DT, NT, RAG, TWO>::kStages;
+          bounded_wait(R.full0 + 8 * s, (it / ColGeo<DT, NT, RAG, TWO>::kStages) & 1, R.abort_flag, R.status);
           const uint64_t row = reinterpret_cast<uint64_t>(md.W) + (uint64_t)(sb + b * kColRows + g) * md.rb;
           cols_stage<DT, NT, H, RAG>(R.stage0 + s * kColStageBytes, vc, nv, warp, g, t, xr, acc[b], (uint32_t)row & 15u,
                                      (uint32_t)(row + 8ull * md.rb) & 15u, md.rb - c * vc * 16);
@@ -301,8 +306,8 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
     // warp partials -> red[b][warp][col][row]; C fragment: (g, 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1).
     // Two halves alternate, so one barrier per super block suffices: a half is rewritten
     // only after every thread has passed the next super block's barrier.
-    constexpr uint32_t kStride = ColGeo<DT, NT, RAG>::kRedStride;
-    float *red = red_base + par * ColGeo<DT, NT, RAG>::kRedFloats;
+    constexpr uint32_t kStride = ColGeo<DT, NT, RAG, TWO>::kRedStride;
+    float *red = red_base + par * ColGeo<DT, NT, RAG, TWO>::kRedFloats;
     par ^= 1;
 #pragma unroll
     for (int b = 0; b < kColBlocks; ++b) {
@@ -337,11 +342,11 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
   }
 }
 
-template <int DT, int NT, bool RAG>
-__global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG>::kCtasPerSm))
+template <int DT, int NT, bool RAG, bool TWO>
+__global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG, TWO>::kCtasPerSm))
     gemm_cols_kernel(const MatDesc *__restrict__ mats, const Piece *__restrict__ pieces,
                      const uint32_t *__restrict__ begin, int *status, const uint8_t *__restrict__ maps) {
-  using Geo = ColGeo<DT, NT, RAG>;
+  using Geo = ColGeo<DT, NT, RAG, TWO>;
   constexpr int kColStages = Geo::kStages;
   extern __shared__ __align__(128) uint8_t smem[];
   Ring R;
@@ -424,7 +429,7 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG>::kCtasPerSm)
     for (uint32_t pi = p0; pi < p1; ++pi) {
       const Piece pc = pieces[pi];
       const MatDesc md = mats[pc.mat];
-      cols_piece<DT, NT, RAG>(md, pc, R, red, it, par, warp, lane);
+      cols_piece<DT, NT, RAG, TWO>(md, pc, R, red, it, par, warp, lane);
     }
   }
   __syncthreads();
@@ -432,34 +437,41 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG>::kCtasPerSm)
 
 }  // namespace
 
-int gemm_cols_ctas_per_sm(int dtype, bool ragged) { return dtype == 3 || ragged ? 2 : 1; }
+int gemm_cols_ctas_per_sm(int dtype, bool ragged, bool two) { return dtype == 3 || ragged || two ? 2 : 1; }
 
-template <int DT, int NT>
+template <int DT, int NT, bool RAG, bool TWO>
 static cudaError_t cols_attr() {
-  const cudaError_t e = cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ColGeo<DT, NT>::kSmem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)ColGeo<DT, NT, true>::kSmem);
+  return cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, RAG, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)ColGeo<DT, NT, RAG, TWO>::kSmem);
+}
+
+// Every variant of one dtype: one and two column tiles, ragged or not, TWO where it applies.
+template <int DT>
+static cudaError_t cols_attrs() {
+  cudaError_t e;
+  if ((e = cols_attr<DT, 1, false, false>()) != cudaSuccess || (e = cols_attr<DT, 2, false, false>()) != cudaSuccess ||
+      (e = cols_attr<DT, 1, true, false>()) != cudaSuccess || (e = cols_attr<DT, 2, true, false>()) != cudaSuccess)
+    return e;
+  return cols_attr<DT, 2, false, DT != 3>();
 }
 
 cudaError_t gemm_cols_prepare() {
   cudaError_t e;
-  if ((e = cols_attr<1, 1>()) != cudaSuccess || (e = cols_attr<1, 2>()) != cudaSuccess ||
-      (e = cols_attr<2, 1>()) != cudaSuccess || (e = cols_attr<2, 2>()) != cudaSuccess ||
-      (e = cols_attr<3, 1>()) != cudaSuccess)
-    return e;
-  return cols_attr<3, 2>();
+  if ((e = cols_attrs<1>()) != cudaSuccess || (e = cols_attrs<2>()) != cudaSuccess) return e;
+  return cols_attrs<3>();
+}
+
+template <int DT, int NT, bool RAG, bool TWO>
+static void cols_go(const GemvLaunch &L, cudaStream_t s) {
+  gemm_cols_kernel<DT, NT, RAG, TWO>
+      <<<L.grid, kColThreads, ColGeo<DT, NT, RAG, TWO>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
 }
 
 template <int DT, int NT>
 static void cols_launch(const GemvLaunch &L, cudaStream_t s) {
-  if (L.ragged)
-    gemm_cols_kernel<DT, NT, true>
-        <<<L.grid, kColThreads, ColGeo<DT, NT, true>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
-  else
-    gemm_cols_kernel<DT, NT, false>
-        <<<L.grid, kColThreads, ColGeo<DT, NT>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
+  if (L.ragged) cols_go<DT, NT, true, false>(L, s);
+  else if (L.two) cols_go<DT, NT, false, DT != 3 && NT == 2>(L, s);
+  else cols_go<DT, NT, false, false>(L, s);
 }
 
 cudaError_t launch_gemm_cols(const GemvLaunch &L, cudaStream_t s) {

@@ -367,6 +367,7 @@ struct Plan {
     bool short_rows = false;     // multi-column launch on the short-row kernel (wt_colshort.cu)
     bool mapped_cols = false;    // map endpoint with T columns
     bool ragged = false;         // some matrix has ragged rows (multi-column launches: every one)
+    bool two = false;            // warp-MMA launch on two CTAs per SM (2-byte weights, T > 8)
     int nt = 0;                  // warp-MMA multi-column launches: 8-column tiles (1 or 2)
     uint32_t nmat = 0, ntiles = 0;
   };
@@ -1265,21 +1266,38 @@ wt::MatDesc make_seg_mat(const wt_gemv_desc &d, uint32_t k, bool ragged) {
   return m;
 }
 
-// 2-byte weights with more than 8 columns run on the warp-level MMA kernel (wt_cols.cu), or on
-// tcgen05 (wt_umma.cu) where a matrix has at least 16384 rows of at most 3072 bytes.  The choice
-// is by the matrix alone: the kernels round differently, and a row's bits do not depend on what
-// else its launch holds.  tcgen05 keeps the rate of HBM at any T and K where the warp-MMA kernel
-// spends its chunks' latencies on little work (T = 16, bf16, us on tcgen05 / warp-MMA, 1 GiB of
-// 16384-row matrices: K = 576 183 / 223, 768 174 / 259, 1024 167 / 208, 1536 162 / 192; 2048 163 / 170,
-// 4096 161 / 164, 8192 184 / 163), but it deals whole 128-row tiles, and a launch waits for the CTA
-// with one more (alone, K = 1024: 4096 rows 10.6 / 8.4, 8192 11.0 / 10.5, 16384 12.4 / 12.6, 20480
-// 18.5 / 15.4, 32768 18.6 / 20.6, 65536 29 / 33; K = 4096: 4096 rows 27 / 13, 65536 93 / 85).  Up to
-// 8 columns the warp-MMA kernel is the faster throughout.  WT_COLS_KERNEL=mma or =umma forces
-// one kernel (umma still only for 2-byte weights).
+// 2-byte weights with more than 8 columns run on the warp-level MMA kernel (wt_cols.cu), and on
+// tcgen05 (wt_umma.cu) where a matrix has at least 16 of its 128-row tiles per SM and rows of at
+// most 3072 bytes.  The choice is by the matrix alone: the kernels round differently, and a row's
+// bits do not depend on what else its launch holds.  tcgen05 keeps the rate of HBM at any T, but
+// deals whole tiles, and a launch waits for the CTA with one more (T = 16, bf16, us on tcgen05 /
+// warp-MMA: 4096 x 4096 27 / 13, 65536 x 4096 93 / 85; 1 GiB of 16384-row matrices: K = 1024 167 / 188,
+// 4096 164 / 166, 8192 187 / 165), and it adds up a whole row in the tensor cores, which truncate
+// (2-norm error against 64 bits at 1024 columns 9.9e-7, on the warp-MMA kernel 9e-8), so nothing
+// went over to it when the choice became the matrix's.  Up to 8 columns the warp-MMA kernel is
+// the faster throughout.  WT_COLS_KERNEL=mma or =umma forces one kernel (umma still only for
+// 2-byte weights).
 bool cols_on_umma(const wt_gemv_desc &d) {
   const int f = cols_forced();
   if (f == 1 || f == 2) return f == 1;
-  return d.cols > 8 && d.M >= 16384 && d.K * elem_bytes(d.dtype) <= 3072;
+  return d.cols > 8 && (d.M + 127) / 128 >= 16ull * wt::num_sms() && d.K * elem_bytes(d.dtype) <= 3072;
+}
+
+// Multi-column launches of 2-byte weights with more than 8 columns run two CTAs per SM where most
+// of their weights lie in rows of at most three chunks of at most 76 vectors, whose stages are too
+// short for one CTA to hide its waits in (T = 16, bf16, 10432 rows each, 256 MiB, us on one / two: 520
+// columns, one chunk of 68 vectors, 65.3 / 62.8; 712, one of 92, 57.8 / 62.3; 768, two of 52, 68.7 /
+// 56.2; 1024, 68, 56.2 / 52.1; 1216, 76, 50.4 / 49.7; 1280, 84, 52.3 / 53.1; 1472, 92, 46.1 / 48.0;
+// 1536, three of 68, 54.0 / 50.0; 2048, 92, 48.2 / 49.7), and where they have 64 KB for each such CTA
+// (4096 x 1536 alone 8.6 / 10.4).
+bool cols_two_ctas(const std::vector<wt::MatDesc> &ms) {
+  uint64_t all = 0, low = 0;
+  for (const wt::MatDesc &m : ms) {
+    const uint64_t b = (uint64_t)m.M * m.V * 16;
+    all += b;
+    if (m.vc <= 76 && m.V <= 3 * 76) low += b;
+  }
+  return 2 * low > all && all >= 2ull * wt::num_sms() * (64 << 10);
 }
 
 // Multi-column matrices of few long rows (aligned, 2-byte weights): the warp-MMA kernel gives a 16-row tile to
@@ -2008,7 +2026,8 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         for (const wt::MatDesc &m : ms) L.ragged |= m.rb != 0;
         L.nt = pass == 2 || pass == 6 ? 1 : pass == 5 || pass == 7 ? 2 : 0;
         if (warp_mma) {
-          deal_tiles(ms, L.grid, pieces, begin, wt::gemm_cols_ctas_per_sm(dt, L.ragged), warp_mma_cost());
+          L.two = pass == 5 && dt != WT_I8 && cols_two_ctas(ms);
+          deal_tiles(ms, L.grid, pieces, begin, wt::gemm_cols_ctas_per_sm(dt, L.ragged, L.two), warp_mma_cost());
         } else {
           partition(ms, L.grid, pieces, begin, 1, pass == 0 ? one_col_slices(dt) : 1,
                     pass == 0 ? wt::gemv_ctas_per_sm(dt) : 1);
@@ -2179,6 +2198,7 @@ int run_plan(wt_handle *h, Plan *P, const wt_gemv_desc *d, cudaStream_t s, bool 
       gl.status = h->status;
       gl.maps = L.maps == SIZE_MAX ? nullptr : P->dev + L.maps;
       gl.ragged = L.ragged;
+      gl.two = L.two;
       gl.nt = L.nt;
       if (L.short_rows) {
         CU(wt::launch_gemm_short(gl, s));

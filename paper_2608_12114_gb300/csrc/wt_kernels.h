@@ -119,6 +119,7 @@ struct GemvLaunch {
   int nt = 0;     // multi-column kernel: 8-column MMA tiles of every matrix (T <= 8 nt)
   int ragged = 0;  // one-column kernel: some matrix has ragged rows (MatDesc.rb > 0);
                    // multi-column kernel: every matrix has (maps stays null)
+  int two = 0;    // multi-column kernel, 2-byte weights, nt 2, not ragged: two CTAs per SM
   int pdl = 0;    // one-column kernel: launch with programmatic stream serialization (the
                   // launch and prologue may overlap the previous kernel of the stream)
   uint64_t *stamps = nullptr;  // one-column kernel: non-null runs the stamping instantiation,
@@ -162,7 +163,7 @@ cudaError_t launch_gemv_mapped_cols(const GemvLaunch &L, cudaStream_t s);
 // 8 < T <= 16); int8 with nt = 1 runs two CTAs per SM (gemm_cols_ctas_per_sm).
 cudaError_t gemm_cols_prepare();
 cudaError_t launch_gemm_cols(const GemvLaunch &L, cudaStream_t s);
-int gemm_cols_ctas_per_sm(int dtype, bool ragged);
+int gemm_cols_ctas_per_sm(int dtype, bool ragged, bool two);
 
 // The same for short rows (wt_colshort.cu), at most short_row_bytes each: stages of whole rows,
 // rt of them (32 KB, less kRaggedSlack for ragged ones).  One launch

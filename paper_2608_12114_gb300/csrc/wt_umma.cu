@@ -14,9 +14,9 @@
 //   epilogue warps  tcgen05.ld (32 lanes x 16 columns per warp) and the stores of Y
 //
 // The tensor-core time does not grow with T (N = 16 always), so this kernel serves T > 8 where
-// the warp-level MMA kernel slows down: matrices of many rows of up to 3072 bytes.  int8 weights stay on that kernel: their
-// decode runs in registers there, while here it would have to pass through shared memory
-// before every MMA (measured: 3.1 TB/s against 5.8-6.0 TB/s).
+// the warp-level MMA kernel slows down: matrices of very many rows of up to 3072 bytes.  int8
+// weights stay on that kernel: their decode runs in registers there, while here it would have to
+// pass through shared memory before every MMA (measured: 3.1 TB/s against 5.8-6.0 TB/s).
 //
 // Every mbarrier wait is bounded; a timeout records WT_ETIMEDOUT and every role stops.  The
 // allocating warp frees the tensor memory after the whole CTA has synchronised.

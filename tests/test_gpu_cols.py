@@ -31,8 +31,8 @@ def torch():
 @pytest.fixture(params=["default", "mma", "umma", "q8rows"], autouse=True)
 def cols_kernel(request, monkeypatch):
     """Every test runs under each routing of the multi-column kernels: the default (short rows on
-    their own kernel, int8 in large even launches on the row-owner kernel, large 2-byte matrices
-    of rows up to 3072 bytes with T > 8 on tcgen05, the rest on the warp-MMA kernel), everything
+    their own kernel, int8 in large even launches on the row-owner kernel, 2-byte matrices of
+    311169 rows and more of up to 3072 bytes with T > 8 on tcgen05, the rest on the warp-MMA kernel), everything
     on the warp-MMA kernel (WT_COLS_KERNEL=mma), 2-byte weights on tcgen05 at every T (=umma),
     and int8 on the row-owner kernel at every T (=q8rows).  Ragged operands take the same kernels
     under each."""
@@ -285,11 +285,11 @@ def test_cols_few_long_rows(torch, T):
 @pytest.mark.parametrize("T", [9, 16])
 def test_cols_bits_do_not_depend_on_the_launch(torch, T):
     """2-byte weights with more than 8 columns: matrices on each side of the line between the
-    warp-MMA and the tcgen05 kernel (16384 rows, 3072 bytes) give the same bits alone and beside
-    a matrix that makes the launch a large one (2432 tiles of 128 rows), and the right ones."""
+    warp-MMA and the tcgen05 kernel (2432 tiles of 128 rows) give the same bits alone, on one CTA
+    per SM or two, and all together in a large launch, and the right ones."""
     g = torch.Generator("cuda").manual_seed(40 + T)
-    shapes = [(64, 1024), (16383, 1024), (16384, 1024), (16384, 1536), (16384, 1544), (20480, 776)]
-    big = (311296, 520)
+    shapes = [(64, 1024), (16383, 1024), (16384, 1536), (16384, 1544), (20480, 776), (311168, 520)]
+    big = (311169, 520)
     with wt.Handle([]) as h:
         for dtype, tdt in ((BF16, torch.bfloat16), (F16, torch.float16)):
             Ws = [torch.empty(M, K, dtype=tdt, device="cuda").normal_(0, 0.02, generator=g) for M, K in shapes + [big]]
