@@ -18,10 +18,10 @@
 // same four k of X: A and B fragments come straight from whole vector loads, and an int8
 // word decodes into exactly the two f16x2 registers a fragment needs.
 //
-// Four 16-row tiles (two for int8 with T > 8) form a super block whose X registers are loaded
-// once per K chunk.  At
-// the end of a super block the warps' partial tiles meet in shared memory and are summed in
-// warp order (deterministic; rows never depend on the partition across CTAs).
+// Four 16-row tiles (two where T > 8 runs two CTAs per SM) form a super block whose X registers
+// are loaded once per K chunk.  At the end of a super block the warps' partial tiles meet in
+// shared memory and are summed in pairs, in a fixed order (deterministic; rows never depend on
+// the partition across CTAs).
 //
 // Ragged operands (RAG: rows of W or X that are no whole number of 16-byte vectors, or W or X
 // off a 16-byte boundary): no tensor map can describe such rows, so each lane of the producer
