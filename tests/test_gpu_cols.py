@@ -314,15 +314,15 @@ def test_cols_bits_do_not_depend_on_the_launch(torch, T):
 
 @pytest.mark.parametrize("seed", range(6))
 def test_random_sets_are_dealt_whole(torch, seed):
-    """Random sets of matrices in one pass, T on both sides of 8, aligned and ragged, short rows and
-    long ones, even and uneven over the CTAs: every output against 64-bit sums, Y NaN-filled
-    first (a row that no CTA was dealt stays NaN)."""
+    """Random sets of matrices in one pass, one column and T on both sides of 8, aligned and ragged,
+    short rows and long ones, even and uneven over the CTAs: every output against 64-bit sums, Y
+    NaN-filled first (a row that no CTA was dealt stays NaN)."""
     rng = np.random.default_rng(600 + seed)
     g = torch.Generator("cuda").manual_seed(seed)
     mats = []
     for _ in range(int(rng.integers(1, 24))):
         dtype = int(rng.choice([BF16, F16, I8]))
-        T = int(rng.integers(1, 17))
+        T = int(rng.choice([0, 0, *range(1, 17)]))
         K = int(np.exp(rng.uniform(np.log(16), np.log(9000))))
         K = max(1, K // int(rng.choice([64, 64, 16, 1])) * 64) if rng.random() < 0.5 else K
         M = int(np.exp(rng.uniform(np.log(1), np.log(max(2, min(40000, (48 << 20) // K))))))
@@ -330,8 +330,8 @@ def test_random_sets_are_dealt_whole(torch, seed):
         W = torch.randint(-128, 128, (M, K), dtype=tdt, device="cuda", generator=g) if dtype == I8 else \
             torch.empty(M, K, dtype=tdt, device="cuda").normal_(0, 0.02, generator=g)
         s = torch.rand(M, device="cuda", generator=g).half() if dtype == I8 else None
-        X = torch.empty(T, K, dtype=torch.float16 if dtype == I8 else tdt, device="cuda").normal_(0, 1, generator=g)
-        mats.append((dtype, T, W, s, X, torch.full((T * M,), float("nan"), device="cuda")))
+        X = torch.empty(max(1, T), K, dtype=torch.float16 if dtype == I8 else tdt, device="cuda").normal_(0, 1, generator=g)
+        mats.append((dtype, T, W, s, X, torch.full((max(1, T) * M,), float("nan"), device="cuda")))
     with wt.Handle([]) as h:
         h.pass_([wt.gemv_desc(W.data_ptr(), d, *W.shape, X.data_ptr(), y.data_ptr(), cols=T,
                               scale=s.data_ptr() if s is not None else 0) for d, T, W, s, X, y in mats], 0)
@@ -343,5 +343,5 @@ def test_random_sets_are_dealt_whole(torch, seed):
             ref, mag = X.double() @ w.t(), X.double().abs() @ w.abs().t()
             if s is not None:
                 ref, mag = ref * s[r:r + 8192].double(), mag * s[r:r + 8192].double()
-            got = y.view(T, -1)[:, r:r + 8192].double()
+            got = y.view(max(1, T), -1)[:, r:r + 8192].double()
             assert ((got - ref).abs() <= TOL * mag).all(), (d, T, tuple(W.shape), r)
