@@ -27,13 +27,14 @@
 // off a 16-byte boundary): no tensor map can describe such rows, so each lane of the producer
 // warp brings one row's share of a chunk by a 1-D copy, and every weight and X vector is put
 // together from the two 16-byte vectors that hold it.  These calls had fp32 FMAs before, one warp
-// per row, and the tensor cores truncate what they accumulate, so every MMA has a second one that
-// brings back what the first dropped (mma16816_kept).  Error against 64 bits at T = 8, with FMAs /
-// with one MMA / now: rows of 1027 bf16 6.9e-8 / 7.9e-8 / 5.6e-8, int8 7.2e-8 / 8.9e-8 / 6.2e-8; rows of
-// 2731 bf16 8.5e-8 / 9.1e-8 / 5.6e-8, int8 8.7e-8 / 9.6e-8 / 6.1e-8, f16 1.7e-7 / 1.1e-7 / 6.0e-8.  Eight 16384 x 2731
-// matrices at T = 8 / 16, with FMAs / with one MMA / now: bf16 1924, 4011 / 198, 341 / 217, 448 us, int8
-// 1532, 3097 / 141, 321 / 192, 433 us (bf16 T = 8: 3310 GB/s, two CTAs per SM, bound by the latencies of
-// putting vectors together; 16 columns on one CTA per SM with twice the registers 594 and 495 us).
+// per row, and the tensor cores truncate what they accumulate.  So each vector's MMAs start from
+// zero and meet the fp32 sums in ordinary additions (adding every MMA by itself is no better); and in
+// kRaggedKept every MMA has a second one that brings back what the first dropped
+// (mma16816_kept).  The host's cols_kept takes it where the error against 64 bits would be larger
+// than with FMAs.  Eight 16384 x 2731 matrices at T = 8 / 16, with FMAs / here / kept: bf16 1924, 4011 /
+// 198, 374 / 217, 448 us, int8 1532, 3097 / 143, 319 / 192, 433 us (bf16 T = 8: 3610 GB/s, two CTAs per
+// SM, bound by the latencies of putting vectors together; 16 columns kept on one CTA per SM with
+// twice the registers 594 and 495 us).
 //
 // Why warp-level MMAs and not tcgen05: the A operand is decoded from int8 in registers and
 // goes to the MMA from there; tcgen05 takes A only from shared or tensor memory, which would
@@ -73,23 +74,26 @@ __device__ __forceinline__ uint32_t red_at(uint32_t col, uint32_t row) {
 // ragged operands run two CTAs per SM with half the ring each (the same bytes in flight per SM,
 // twice the warps; those paths are latency-bound on decoding and on shifting).  The cross-warp
 // partials of one 16-row tile take 16 x 8 NT floats per warp, in two alternating halves.
-// So do, with TWO, 2-byte weights with 16 columns in launches that are mostly of few short chunks
+// So do, in kAlignedTwo, 2-byte weights with 16 columns in launches that are mostly of few short chunks
 // (the host's cols_two_ctas): there the waits for X and for the other warps' partials are a large
 // part of a super block, and the second CTA fills them (T = 16, bf16, 1 GiB of 16384-row matrices, us
 // with one / two: K = 768 259 / 207, 1024 210 / 188, 1536 196 / 177; but 2048 173 / 177, 8192 165 /
 // 168).  The sums are the same in either.
-template <int DT, int NT, bool RAG = false, bool TWO = false>
+enum ColMode : int { kAligned = 0, kAlignedTwo = 1, kRagged = 2, kRaggedKept = 3 };
+template <int DT, int NT, int MODE = kAligned>
 struct ColGeo {
-  static constexpr int kCtasPerSm = DT == 3 || RAG || TWO ? 2 : 1;
+  static constexpr bool RAG = MODE >= kRagged, KEEP = MODE == kRaggedKept;
+  static constexpr int kCtasPerSm = DT == 3 || MODE != kAligned ? 2 : 1;
   static constexpr int kStages = kCtasPerSm == 2 ? 3 : 6;
   // 16-row tiles per super block (X registers are loaded once per super block and chunk):
   // four, or two for int8 with 16 columns, which then fits two CTAs per SM (registers and
   // partial buffers halve; X is reloaded every 32 rows instead of 64)
   static constexpr int kBlocks = kCtasPerSm == 2 && NT == 2 ? 2 : 4;
-  // accumulator sets per tile (even / odd k16 steps: shorter MMA chains; ragged operands: the
-  // sums and what they lost); int8 with 16 columns keeps one, its two column tiles already give
-  // two independent chains per A
-  static constexpr int kAcc = NT == 2 && DT == 3 && !RAG ? 1 : 2;
+  // accumulator sets per tile (even / odd k16 steps: shorter MMA chains; ragged operands: even /
+  // odd vectors, or the sums and what they lost); int8 and ragged f16 with 16 columns have one,
+  // their two column tiles already give two independent chains per A (ragged bf16 needs the second
+  // for precision, at 10 % more time)
+  static constexpr int kAcc = NT == 2 && !KEEP && (DT == 3 || (RAG && DT == 2)) ? 1 : 2;
   static constexpr int kSuper = kColRows * kBlocks;
   static constexpr uint32_t kRedStride = 128 * NT;  // floats per (tile, warp)
   static constexpr size_t kRedFloats = (size_t)kBlocks * kColWarps * kRedStride;  // one half
@@ -99,8 +103,8 @@ struct ColGeo {
   static constexpr size_t kSmem = kFlagOff + 16;
 };
 static_assert(ColGeo<1, 2>::kSmem <= 232448 && 2 * (ColGeo<3, 1>::kSmem + 1024) <= 233472 &&
-                  2 * (ColGeo<3, 2>::kSmem + 1024) <= 233472 && 2 * (ColGeo<1, 1, true>::kSmem + 1024) <= 233472 &&
-                  2 * (ColGeo<1, 2, true>::kSmem + 1024) <= 233472 && 2 * (ColGeo<1, 2, false, true>::kSmem + 1024) <= 233472,
+                  2 * (ColGeo<3, 2>::kSmem + 1024) <= 233472 && 2 * (ColGeo<1, 1, kRagged>::kSmem + 1024) <= 233472 &&
+                  2 * (ColGeo<1, 2, kRagged>::kSmem + 1024) <= 233472 && 2 * (ColGeo<1, 2, kAlignedTwo>::kSmem + 1024) <= 233472,
               "multi-column shared memory");
 
 // 32-bit words of X per weight vector: 16 fp16 activations for an int8 vector, else 8.
@@ -188,10 +192,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int3
 // RAG: row g starts ph0 bytes past its pitch's start, row g + 8 ph1 bytes; of vector v only the
 // row's own bytes count (left: those from the chunk's start on; an int8 neighbour meets a zero
 // of X and is a finite number, so only the 2-byte types mask it).
-template <int DT, int NT, int H, bool RAG>
+template <int DT, int NT, int H, int MODE>
 __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t nv, int warp, uint32_t g, uint32_t t,
                                            const uint32_t (&xr)[kColGroups][NT][ColX<DT>::W], float (&acc)[H][NT][4],
                                            uint32_t ph0, uint32_t ph1, uint32_t left) {
+  constexpr bool RAG = MODE >= kRagged, KEEP = MODE == kRaggedKept;
   const uint32_t pitch = RAG ? (vc + kColRagPad) * 16 : vc * 16;
 #pragma unroll
   for (int q = 0; q < kColGroups; ++q) {
@@ -213,6 +218,9 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
     }
     const uint32_t ra[4] = {w0.x, w0.y, w0.z, w0.w};
     const uint32_t rb[4] = {w1.x, w1.y, w1.z, w1.w};
+    float part[NT][4];  // kRagged: this vector's products
+#pragma unroll
+    for (int n = 0; n < NT; ++n) part[n][0] = part[n][1] = part[n][2] = part[n][3] = 0.f;
     if constexpr (DT == 3) {
       // word j = weights k 4j..4j+3 of the vector; its activations are x words 2j, 2j+1
 #pragma unroll
@@ -222,10 +230,10 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
         const uint32_t a1 = i8x2_to_f16x2(u1, 0x4140u), a3 = i8x2_to_f16x2(u1, 0x4342u);
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
-          if constexpr (RAG)
+          if constexpr (KEEP)
             mma16816_kept<2>(acc[0][n], acc[1][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
           else
-            mma16816<2>(acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
+            mma16816<2>(RAG ? part[n] : acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
         }
       }
     } else {
@@ -234,14 +242,20 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
       for (int s = 0; s < 2; ++s) {
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
-          if constexpr (RAG)
+          if constexpr (KEEP)
             mma16816_kept<DT>(acc[0][n], acc[1][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
                               xr[q][n][2 * s + 1]);
           else
-            mma16816<DT>(acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
-                         xr[q][n][2 * s + 1]);
+            mma16816<DT>(RAG ? part[n] : acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1],
+                         xr[q][n][2 * s], xr[q][n][2 * s + 1]);
         }
       }
+    }
+    if constexpr (RAG && !KEEP) {
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[q % H][n][i] += part[n][i];
     }
   }
 }
@@ -253,7 +267,7 @@ struct Ring {
 };
 
 // Consumer side of one piece (rows [r0, r1) of one matrix), NT = 8-column MMA tiles.
-template <int DT, int NT, bool RAG, bool TWO>
+template <int DT, int NT, int MODE>
 __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, const Ring &R, float *red_base,
                                            uint32_t &it, uint32_t &par, int warp, int lane) {
   const uint32_t V = md.V, vc = md.vc, T = md.G;
@@ -263,12 +277,13 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
   const uint32_t nchunk = (V + vc - 1) / vc;
   const uint32_t g = lane >> 2, t = lane & 3;
   const int ct = threadIdx.x;
-  constexpr int kColBlocks = ColGeo<DT, NT, RAG, TWO>::kBlocks;
-  constexpr int kColSuper = ColGeo<DT, NT, RAG, TWO>::kSuper;
+  constexpr bool RAG = ColGeo<DT, NT, MODE>::RAG, KEEP = ColGeo<DT, NT, MODE>::KEEP;
+  constexpr int kColBlocks = ColGeo<DT, NT, MODE>::kBlocks;
+  constexpr int kColSuper = ColGeo<DT, NT, MODE>::kSuper;
   for (uint32_t sb = pc.r0; sb < pc.r1; sb += kColSuper) {
     const uint32_t rows = min((uint32_t)kColSuper, pc.r1 - sb);
     const uint32_t nrb = (rows + kColRows - 1) / kColRows;
-    constexpr int H = ColGeo<DT, NT, RAG, TWO>::kAcc;
+    constexpr int H = ColGeo<DT, NT, MODE>::kAcc;
     float acc[kColBlocks][H][NT][4];
 #pragma unroll
     for (int b = 0; b < kColBlocks; ++b)
@@ -292,10 +307,10 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
 #pragma unroll
       for (int b = 0; b < kColBlocks; ++b) {
         if ((uint32_t)b < nrb) {
-          const uint32_t s = it % ColGeo<DT, NT, RAG, TWO>::kStages;
-          bounded_wait(R.full0 + 8 * s, (it / ColGeo<DT, NT, RAG, TWO>::kStages) & 1, R.abort_flag, R.status);
+          const uint32_t s = it % ColGeo<DT, NT, MODE>::kStages;
+          bounded_wait(R.full0 + 8 * s, (it / ColGeo<DT, NT, MODE>::kStages) & 1, R.abort_flag, R.status);
           const uint64_t row = reinterpret_cast<uint64_t>(md.W) + (uint64_t)(sb + b * kColRows + g) * md.rb;
-          cols_stage<DT, NT, H, RAG>(R.stage0 + s * kColStageBytes, vc, nv, warp, g, t, xr, acc[b], (uint32_t)row & 15u,
+          cols_stage<DT, NT, H, MODE>(R.stage0 + s * kColStageBytes, vc, nv, warp, g, t, xr, acc[b], (uint32_t)row & 15u,
                                      (uint32_t)(row + 8ull * md.rb) & 15u, md.rb - c * vc * 16);
           __syncwarp();
           if (lane == 0) mbar_arrive(R.empty0 + 8 * s);
@@ -306,8 +321,8 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
     // warp partials -> red[b][warp][col][row]; C fragment: (g, 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1).
     // Two halves alternate, so one barrier per super block suffices: a half is rewritten
     // only after every thread has passed the next super block's barrier.
-    constexpr uint32_t kStride = ColGeo<DT, NT, RAG, TWO>::kRedStride;
-    float *red = red_base + par * ColGeo<DT, NT, RAG, TWO>::kRedFloats;
+    constexpr uint32_t kStride = ColGeo<DT, NT, MODE>::kRedStride;
+    float *red = red_base + par * ColGeo<DT, NT, MODE>::kRedFloats;
     par ^= 1;
 #pragma unroll
     for (int b = 0; b < kColBlocks; ++b) {
@@ -319,7 +334,7 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const float a0 = acc[b][0][n][i], a1 = H == 2 ? acc[b][H - 1][n][i] : 0.f;
-            r[red_at(c0 + (i & 1), g + 8 * (i >> 1))] = RAG ? kept_sum(a0, a1) : a0 + a1;
+            r[red_at(c0 + (i & 1), g + 8 * (i >> 1))] = KEEP ? kept_sum(a0, a1) : a0 + a1;
           }
         }
       }
@@ -342,11 +357,12 @@ __device__ __forceinline__ void cols_piece(const MatDesc &md, const Piece &pc, c
   }
 }
 
-template <int DT, int NT, bool RAG, bool TWO>
-__global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG, TWO>::kCtasPerSm))
+template <int DT, int NT, int MODE>
+__global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, MODE>::kCtasPerSm))
     gemm_cols_kernel(const MatDesc *__restrict__ mats, const Piece *__restrict__ pieces,
                      const uint32_t *__restrict__ begin, int *status, const uint8_t *__restrict__ maps) {
-  using Geo = ColGeo<DT, NT, RAG, TWO>;
+  using Geo = ColGeo<DT, NT, MODE>;
+  constexpr bool RAG = Geo::RAG;
   constexpr int kColStages = Geo::kStages;
   extern __shared__ __align__(128) uint8_t smem[];
   Ring R;
@@ -429,7 +445,7 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG, TWO>::kCtasP
     for (uint32_t pi = p0; pi < p1; ++pi) {
       const Piece pc = pieces[pi];
       const MatDesc md = mats[pc.mat];
-      cols_piece<DT, NT, RAG, TWO>(md, pc, R, red, it, par, warp, lane);
+      cols_piece<DT, NT, MODE>(md, pc, R, red, it, par, warp, lane);
     }
   }
   __syncthreads();
@@ -439,20 +455,27 @@ __global__ void __launch_bounds__(kColThreads, (ColGeo<DT, NT, RAG, TWO>::kCtasP
 
 int gemm_cols_ctas_per_sm(int dtype, bool ragged, bool two) { return dtype == 3 || ragged || two ? 2 : 1; }
 
-template <int DT, int NT, bool RAG, bool TWO>
+template <int DT, int NT, int MODE>
 static cudaError_t cols_attr() {
-  return cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, RAG, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)ColGeo<DT, NT, RAG, TWO>::kSmem);
+  return cudaFuncSetAttribute(gemm_cols_kernel<DT, NT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)ColGeo<DT, NT, MODE>::kSmem);
 }
 
-// Every variant of one dtype: one and two column tiles, ragged or not, TWO where it applies.
+// The modes that some types do without: f16 never keeps (the host's cols_kept).
+template <int DT>
+constexpr int kKept = DT == 2 ? kRagged : kRaggedKept;
+template <int DT, int NT>
+constexpr int kTwo = DT != 3 && NT == 2 ? kAlignedTwo : kAligned;
+
+// Every variant of one dtype.
 template <int DT>
 static cudaError_t cols_attrs() {
   cudaError_t e;
-  if ((e = cols_attr<DT, 1, false, false>()) != cudaSuccess || (e = cols_attr<DT, 2, false, false>()) != cudaSuccess ||
-      (e = cols_attr<DT, 1, true, false>()) != cudaSuccess || (e = cols_attr<DT, 2, true, false>()) != cudaSuccess)
+  if ((e = cols_attr<DT, 1, kAligned>()) != cudaSuccess || (e = cols_attr<DT, 2, kAligned>()) != cudaSuccess ||
+      (e = cols_attr<DT, 1, kRagged>()) != cudaSuccess || (e = cols_attr<DT, 2, kRagged>()) != cudaSuccess ||
+      (e = cols_attr<DT, 1, kKept<DT>>()) != cudaSuccess || (e = cols_attr<DT, 2, kKept<DT>>()) != cudaSuccess)
     return e;
-  return cols_attr<DT, 2, false, DT != 3>();
+  return cols_attr<DT, 2, kTwo<DT, 2>>();
 }
 
 cudaError_t gemm_cols_prepare() {
@@ -461,17 +484,18 @@ cudaError_t gemm_cols_prepare() {
   return cols_attrs<3>();
 }
 
-template <int DT, int NT, bool RAG, bool TWO>
+template <int DT, int NT, int MODE>
 static void cols_go(const GemvLaunch &L, cudaStream_t s) {
-  gemm_cols_kernel<DT, NT, RAG, TWO>
-      <<<L.grid, kColThreads, ColGeo<DT, NT, RAG, TWO>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
+  gemm_cols_kernel<DT, NT, MODE>
+      <<<L.grid, kColThreads, ColGeo<DT, NT, MODE>::kSmem, s>>>(L.mats, L.pieces, L.begin, L.status, L.maps);
 }
 
 template <int DT, int NT>
 static void cols_launch(const GemvLaunch &L, cudaStream_t s) {
-  if (L.ragged) cols_go<DT, NT, true, false>(L, s);
-  else if (L.two) cols_go<DT, NT, false, DT != 3 && NT == 2>(L, s);
-  else cols_go<DT, NT, false, false>(L, s);
+  if (L.ragged && L.keep) cols_go<DT, NT, kKept<DT>>(L, s);
+  else if (L.ragged) cols_go<DT, NT, kRagged>(L, s);
+  else if (L.two) cols_go<DT, NT, kTwo<DT, NT>>(L, s);
+  else cols_go<DT, NT, kAligned>(L, s);
 }
 
 cudaError_t launch_gemm_cols(const GemvLaunch &L, cudaStream_t s) {

@@ -368,6 +368,7 @@ struct Plan {
     bool mapped_cols = false;    // map endpoint with T columns
     bool ragged = false;         // some matrix has ragged rows (multi-column launches: every one)
     bool two = false;            // warp-MMA launch on two CTAs per SM (2-byte weights, T > 8)
+    bool keep = false;           // ragged warp-MMA launch that keeps what truncation drops
     int nt = 0;                  // warp-MMA multi-column launches: 8-column tiles (1 or 2)
     uint32_t nmat = 0, ntiles = 0;
   };
@@ -1283,6 +1284,13 @@ bool cols_on_umma(const wt_gemv_desc &d) {
   return d.cols > 8 && (d.M + 127) / 128 >= 16ull * wt::num_sms() && d.K * elem_bytes(d.dtype) <= 3072;
 }
 
+// Ragged multi-column matrices whose MMAs keep what truncation drops: those that would be further
+// from 64-bit sums than the fp32 FMAs which they had before, whose error grows with K (ratio of the
+// errors without / with, T = 8: bf16 K = 513 1.08 / 0.90, 1365 1.02 / 0.77, 2047 0.99 / 0.71; int8 1113
+// 1.15 / 0.85, 3331 1.03 / 0.68, 3901 0.99 / 0.65, at T = 16 3901 1.02, 4601 1.00; f16 513 0.99 / 0.69,
+// 2731 0.60 / 0.36).  Keeping costs bf16 6 to 10 % of the time at T = 8 and 20 % at T = 16, int8 16 to 35 %.
+bool cols_kept(const wt_gemv_desc &d) { return d.K < (d.dtype == WT_BF16 ? 2048u : d.dtype == WT_I8 ? 4608u : 0u); }
+
 // Multi-column launches of 2-byte weights with more than 8 columns run two CTAs per SM where most
 // of their weights lie in rows of at most three chunks of at most 76 vectors, whose stages are too
 // short for one CTA to hide its waits in (T = 16, bf16, 10432 rows each, 256 MiB, us on one / two: 520
@@ -1779,7 +1787,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
     g.first = mem.front();
     // cols_dt: warp-MMA multi-column with T <= 8, colsw_dt: with 8 < T <= 16
     std::vector<wt::MatDesc> by_dt[4], mapped_dt[4], cols_dt[4], umma_dt[4], mcols_dt[4], colsw_dt[4], q8r_dt[4],
-        ragc_dt[4], ragcw_dt[4],  // warp-MMA with ragged operands, T <= 8 and T > 8
+        rag_dt[4][4],             // warp-MMA with ragged operands: [dtype][T > 8, + 2 if kept]
         short_dt[4][4],           // [dtype][T > 8, + 2 if ragged]: short rows
         q8r1_dt[4];  // row-owner int8 launches with two 8-column tiles (T > 8) and with one
     std::vector<wt_gemv_desc> i8c[2];  // int8 on the tensor cores, T <= 8 and T > 8: kernel chosen below
@@ -1875,7 +1883,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
         i8c[0].push_back(q1);
         i8_blocks += (q.M + wt::kQ8RowsBlock - 1) / wt::kQ8RowsBlock;
       } else if (q.cols > 0 && q.dtype != WT_F32 && q.K * es < 0x7fffffffull) {
-        (q.cols > 8 ? ragcw_dt : ragc_dt)[q.dtype].push_back(make_cols_mat(q, true));
+        rag_dt[q.dtype][(q.cols > 8) + 2 * cols_kept(q)].push_back(make_cols_mat(q, true));
       } else if (q.cols == 0 && (fast || (q.K * es < 0x7fffffffull && reinterpret_cast<uintptr_t>(q.W) % es == 0))) {
         // device memory, one column: whole 16-byte vectors per row, or ragged rows (any K, W on
         // an element boundary, x at any byte), which the one-warp-per-row kernel streamed at 500
@@ -1945,7 +1953,7 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           cseg_ws[dt][w].push_back((int64_t)sg.second);
         }
       }
-    for (int pass = 0; pass < 14; ++pass) {
+    for (int pass = 0; pass < 16; ++pass) {
       for (int dt = 0; dt < 4; ++dt) {
         std::vector<wt::MatDesc> &ms = pass == 0   ? by_dt[dt]
                                        : pass == 1 ? mapped_dt[dt]
@@ -1953,12 +1961,11 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
                                        : pass == 3 ? umma_dt[dt]
                                        : pass == 4 ? mcols_dt[dt]
                                        : pass == 5 ? colsw_dt[dt]
-                                       : pass == 6 ? ragc_dt[dt]
-                                       : pass == 7 ? ragcw_dt[dt]
-                                       : pass == 8 ? q8r_dt[dt]
-                                       : pass == 9 ? q8r1_dt[dt]
-                                                   : short_dt[dt][pass - 10];
-        const bool warp_mma = pass == 2 || (pass >= 5 && pass < 8);
+                                       : pass < 10 ? rag_dt[dt][pass - 6]
+                                       : pass == 10 ? q8r_dt[dt]
+                                       : pass == 11 ? q8r1_dt[dt]
+                                                    : short_dt[dt][pass - 12];
+        const bool warp_mma = pass == 2 || (pass >= 5 && pass < 10);
         if (ms.empty()) continue;
         Plan::Launch L;
         L.dtype = dt;
@@ -1988,11 +1995,11 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           g.cols.push_back(L);
           continue;
         }
-        if (pass >= 10) {
+        if (pass >= 12) {
           // short rows: pieces cut at 32-row groups
           L.short_rows = true;
-          L.nt = (pass - 10) % 2 + 1;
-          L.ragged = pass >= 12;
+          L.nt = (pass - 12) % 2 + 1;
+          L.ragged = pass >= 14;
           CostModel cm;
           cm.row_extra = 4 * 8 * L.nt + (dt == WT_I8 ? 160 : 16);
           partition(ms, L.grid, pieces, begin, 32, 1, 1, cm);
@@ -2002,10 +2009,10 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
           g.cols.push_back(L);
           continue;
         }
-        if (pass >= 8) {
+        if (pass >= 10) {
           // row-owner int8 launch: pieces cut at 128-row blocks, two tensor maps per matrix
           L.q8rows = true;
-          L.nt = pass == 8 ? 2 : 1;
+          L.nt = pass == 10 ? 2 : 1;
           deal_tiles(ms, L.grid, pieces, begin, 2, q8rows_cost());
           L.mats = append(P->table, ms);
           L.pieces = append(P->table, pieces);
@@ -2024,7 +2031,8 @@ int build_plan(wt_handle *h, const wt_gemv_desc *d, size_t n, Plan *P) {
             if (m.mode != wt::kModeWarpRows && m.mode != wt::kModeBlockRows && m.mode != wt::kModePhaseRows)
               return set_err(WT_ENOTSUP, "wt_pass: internal: a %u-vector row reached the TMA kernel unsegmented", m.V);
         for (const wt::MatDesc &m : ms) L.ragged |= m.rb != 0;
-        L.nt = pass == 2 || pass == 6 ? 1 : pass == 5 || pass == 7 ? 2 : 0;
+        L.nt = pass == 2 || pass == 6 || pass == 8 ? 1 : pass == 5 || pass == 7 || pass == 9 ? 2 : 0;
+        L.keep = pass == 8 || pass == 9;
         if (warp_mma) {
           L.two = pass == 5 && dt != WT_I8 && cols_two_ctas(ms);
           deal_tiles(ms, L.grid, pieces, begin, wt::gemm_cols_ctas_per_sm(dt, L.ragged, L.two), warp_mma_cost());
@@ -2199,6 +2207,7 @@ int run_plan(wt_handle *h, Plan *P, const wt_gemv_desc *d, cudaStream_t s, bool 
       gl.maps = L.maps == SIZE_MAX ? nullptr : P->dev + L.maps;
       gl.ragged = L.ragged;
       gl.two = L.two;
+      gl.keep = L.keep;
       gl.nt = L.nt;
       if (L.short_rows) {
         CU(wt::launch_gemm_short(gl, s));

@@ -120,6 +120,7 @@ struct GemvLaunch {
   int ragged = 0;  // one-column kernel: some matrix has ragged rows (MatDesc.rb > 0);
                    // multi-column kernel: every matrix has (maps stays null)
   int two = 0;    // multi-column kernel, 2-byte weights, nt 2, not ragged: two CTAs per SM
+  int keep = 0;   // multi-column kernel, ragged: keep what the tensor cores' truncation drops
   int pdl = 0;    // one-column kernel: launch with programmatic stream serialization (the
                   // launch and prologue may overlap the previous kernel of the stream)
   uint64_t *stamps = nullptr;  // one-column kernel: non-null runs the stamping instantiation,
