@@ -27,12 +27,13 @@
 // off a 16-byte boundary): no tensor map can describe such rows, so each lane of the producer
 // warp brings one row's share of a chunk by a 1-D copy, and every weight and X vector is put
 // together from the two 16-byte vectors that hold it.  These calls had fp32 FMAs before, one warp
-// per row, and the tensor cores truncate what they accumulate.  So each vector's MMAs start from
-// zero and meet the fp32 sums in ordinary additions (adding every MMA by itself is no better); and in
-// kRaggedKept every MMA has a second one that brings back what the first dropped
+// per row, and the tensor cores truncate what they accumulate.  So the MMAs of each half of a vector
+// start from zero and meet in ordinary additions, and these the fp32 sums (bf16, 801 and 2731
+// columns, T = 8: FMAs 6.7e-8 and 8.5e-8, whole vectors 7.0e-8 and 8.3e-8, halves 6.8e-8 and 8.1e-8);
+// and in kRaggedKept every MMA has a second one that brings back what the first dropped
 // (mma16816_kept).  The host's cols_kept takes it where the error against 64 bits would be larger
-// than with FMAs.  Eight 16384 x 2731 matrices at T = 8 / 16, with FMAs / here / kept: bf16 1924, 4011 /
-// 198, 374 / 217, 448 us, int8 1532, 3097 / 143, 319 / 192, 433 us (bf16 T = 8: 3610 GB/s, two CTAs per
+// than with FMAs.  Eight 16384 x 2731 matrices at T = 8 / 16, with FMAs / in halves / kept: bf16 1924, 4011 /
+// 199, 375 / 217, 448 us, int8 1532, 3097 / 145, 321 / 192, 433 us (bf16 T = 8: 3600 GB/s, two CTAs per
 // SM, bound by the latencies of putting vectors together; 16 columns kept on one CTA per SM with
 // twice the registers 594 and 495 us).
 //
@@ -218,9 +219,11 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
     }
     const uint32_t ra[4] = {w0.x, w0.y, w0.z, w0.w};
     const uint32_t rb[4] = {w1.x, w1.y, w1.z, w1.w};
-    float part[NT][4];  // kRagged: this vector's products
+    float part[2][NT][4];  // kRagged: the products of the vector's two halves
 #pragma unroll
-    for (int n = 0; n < NT; ++n) part[n][0] = part[n][1] = part[n][2] = part[n][3] = 0.f;
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int n = 0; n < NT; ++n) part[h][n][0] = part[h][n][1] = part[h][n][2] = part[h][n][3] = 0.f;
     if constexpr (DT == 3) {
       // word j = weights k 4j..4j+3 of the vector; its activations are x words 2j, 2j+1
 #pragma unroll
@@ -233,7 +236,7 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
           if constexpr (KEEP)
             mma16816_kept<2>(acc[0][n], acc[1][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
           else
-            mma16816<2>(RAG ? part[n] : acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
+            mma16816<2>(RAG ? part[j / 2][n] : acc[(j & 1) % H][n], a0, a1, a2, a3, xr[q][n][2 * j], xr[q][n][2 * j + 1]);
         }
       }
     } else {
@@ -246,7 +249,7 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
             mma16816_kept<DT>(acc[0][n], acc[1][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1], xr[q][n][2 * s],
                               xr[q][n][2 * s + 1]);
           else
-            mma16816<DT>(RAG ? part[n] : acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1],
+            mma16816<DT>(RAG ? part[s][n] : acc[s % H][n], ra[2 * s], rb[2 * s], ra[2 * s + 1], rb[2 * s + 1],
                          xr[q][n][2 * s], xr[q][n][2 * s + 1]);
         }
       }
@@ -255,7 +258,7 @@ __device__ __forceinline__ void cols_stage(uint32_t tile, uint32_t vc, uint32_t 
 #pragma unroll
       for (int n = 0; n < NT; ++n)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[q % H][n][i] += part[n][i];
+        for (int i = 0; i < 4; ++i) acc[q % H][n][i] += part[0][n][i] + part[1][n][i];
     }
   }
 }

@@ -1286,10 +1286,10 @@ bool cols_on_umma(const wt_gemv_desc &d) {
 
 // Ragged multi-column matrices whose MMAs keep what truncation drops: those that would be further
 // from 64-bit sums than the fp32 FMAs which they had before, whose error grows with K (ratio of the
-// errors without / with, T = 8: bf16 K = 513 1.08 / 0.90, 1365 1.02 / 0.77, 2047 0.99 / 0.71; int8 1113
-// 1.15 / 0.85, 3331 1.03 / 0.68, 3901 0.99 / 0.65, at T = 16 3901 1.02, 4601 1.00; f16 513 0.99 / 0.69,
-// 2731 0.60 / 0.36).  Keeping costs bf16 6 to 10 % of the time at T = 8 and 20 % at T = 16, int8 16 to 35 %.
-bool cols_kept(const wt_gemv_desc &d) { return d.K < (d.dtype == WT_BF16 ? 2048u : d.dtype == WT_I8 ? 4608u : 0u); }
+// errors without / with, T = 8: bf16 K = 513 1.03 / 0.90, 901 1.01 / 0.83, 1201 0.99 / 0.78; int8 1113
+// 1.03 / 0.85, 1801 0.99 / 0.77, at T = 16 1801 1.00, 1965 0.99; f16 513 0.86 / 0.69).  Keeping costs bf16
+// 6 % of the time at T = 8 and 16 % at T = 16, int8 15 and 35 % (eight 16384 x 777 matrices).
+bool cols_kept(const wt_gemv_desc &d) { return d.K < (d.dtype == WT_BF16 ? 1152u : d.dtype == WT_I8 ? 2048u : 0u); }
 
 // Multi-column launches of 2-byte weights with more than 8 columns run two CTAs per SM where most
 // of their weights lie in rows of at most three chunks of at most 76 vectors, whose stages are too
