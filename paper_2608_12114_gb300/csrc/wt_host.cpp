@@ -1217,8 +1217,8 @@ int cols_forced() {
 // Multi-column matrices whose rows the short-row kernel takes: up to 1024 bytes (128 MiB in
 // bf16, T = 8 / 16, by row bytes: 64: 38 / 52 us against 334 / 107 us on the warp-MMA kernel
 // and tcgen05; 1024: 25.5 / 29.3 against 28.5 / 29.2; 2048: 32 / 39 against 26 / 31).  int8
-// rows of 64 to 512 weights go there only where the row-owner kernel's blocks leave the CTAs
-// uneven (T = 8: 64 weights 72 us against 68, 128: 48 against 41, 512: 28 against 25; but 153 and 45 us
+// rows of 64 to 512 weights go there only where the row-owner kernel's blocks are few or leave the
+// CTAs uneven (T = 8: 64 weights 72 us against 68, 128: 48 against 41, 512: 28 against 25; but 153 and 45 us
 // on the warp-MMA kernel, which such small launches took), shorter ones always (32: 132 us
 // against 246).  WT_COLS_KERNEL, which names one of the other kernels, keeps the aligned ones
 // away from it.
